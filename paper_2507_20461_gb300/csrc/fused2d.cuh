@@ -228,8 +228,8 @@ __device__ __forceinline__ void fused2d_strip(const KP &P, const FusedGeo &geo, 
                 else CubicEval<float, 2, 0, 0>::run(g, c, out);
                 cw[side][v] = wv[v];
                 st[side][v][0] = wv[v] + out[0];
-                st[side][v][1] = (xd ? out[1] : out[2]) * ih;
-                st[side][v][2] = (xd ? out[2] : out[1]) * ih;
+                st[side][v][1] = xd ? out[1] : out[2];
+                st[side][v][2] = xd ? out[2] : out[1];
             }
             float s[NV];
 #pragma unroll
@@ -258,7 +258,7 @@ __device__ __forceinline__ void fused2d_strip(const KP &P, const FusedGeo &geo, 
             dWr[1][v] = yd ? st[1][u][1] : st[1][v][2];
         }
         float F[NV], Ft[NV], Wh[NV];
-        if (!gks_point<float, 2, NS>(P.fp, dtf, Wl, Wr, dWl, dWr, F, Ft, Wh)) {
+        if (!gks_point_scaled<float, 2, NS>(P.fp, dtf, 1.f / dtf, ih, Wl, Wr, dWl, dWr, F, Ft, Wh)) {
             atomicOr(status, ST_FLUX);
 #pragma unroll
             for (int v = 0; v < NV; ++v) F[v] = Ft[v] = Wh[v] = 0.f;

@@ -765,7 +765,9 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncthreads();
     }
-    /* interface states, global axes: st[side][v][c], c = 0 value, 1 + e d/dx_e */
+    /* interface states, global axes: st[side][v][c], c = 0 value, 1 + e
+     * h d/dx_e (cell units, which the flux takes as they are) */
+    const R ih = pick<R>(P.ih, P.fih);
     R st[2][NV][M + 1], cw[2][NV];
     /* a face inside the grid has two real cells: no ghost mapping, no signs */
     const bool inner = idx[D] > 0 && idx[D] < P.n[D];
@@ -793,7 +795,7 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
             cw[side][v] = w0;
             st[side][v][0] = w0 + out[0];
 #pragma unroll
-            for (int a = 0; a < M; ++a) st[side][v][1 + a] = out[1 + a] * pick<R>(P.ih, P.fih);
+            for (int a = 0; a < M; ++a) st[side][v][1 + a] = out[1 + a];
         }
         R s[NV];
 #pragma unroll
@@ -816,7 +818,7 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
             for (int v = 0; v < NV; ++v)
 #pragma unroll
                 for (int c = 0; c < M + 1; ++c)
-                    fs[(((long)(side * NV + v) * (M + 1) + c) * NG + g) * nft + face] = (double)st[side][v][c];
+                    fs[(((long)(side * NV + v) * (M + 1) + c) * NG + g) * nft + face] = (double)(c ? st[side][v][c] * ih : st[side][v][c]);
         return;
     }
     /* face frame: axis order (D, then the others ascending) */
@@ -843,7 +845,7 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
     }
     R F[NV], Ft[NV], Wh[NV];
     const R dt = R(dtv);
-    if (!gks_point<R, M, NS>(P.fp, dt, Wl, Wr, dWl, dWr, F, Ft, Wh)) {
+    if (!gks_point_scaled<R, M, NS>(P.fp, dt, R(1) / dt, ih, Wl, Wr, dWl, dWr, F, Ft, Wh)) {
         atomicOr(status, ST_FLUX);
 #pragma unroll
         for (int v = 0; v < NV; ++v) F[v] = Ft[v] = Wh[v] = R(0);
