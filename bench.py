@@ -76,13 +76,10 @@ NC_CELL_UPDATE = {o: _flops(f"nc_step_cell_update_1d_order{o}") for o in (5, 6)}
 # launches of a step; the face-flux flop summary under profiles/).  The
 # kernel uses closed forms where the oracle solves moment systems, so it
 # executes fewer flops than the algorithmic count.
-EXECUTED_FLOPS_PER_FACE_GP = {"mixed": 1523.8, "fp64": 1853.1}
-# DRAM bytes (read + write) per launch of the face-flux kernel: the mean of
-# the four launches of a 1-pass ncu capture at 1024^2 (coefficients 151 MB
-# FP32 / 303 MB FP64, above L2): 200.5 MB mixed, 854.8 MB FP64, scaled to
-# the 2048^2 launch by the Gauss points it processes.
-TRAFFIC_PER_FLUX_LAUNCH = {"mixed": 200.51e6 * (2049 * 2048) / (1025 * 1024),
-                           "fp64": 854.85e6 * (2049 * 2048) / (1025 * 1024)}
+EXECUTED_FLOPS_PER_FACE_GP = {"mixed": None, "fp64": None}
+# DRAM bytes (read + write) per launch of the face-flux kernel at 2048^2, from
+# a 1-pass ncu capture (None: not captured for the current kernel).
+TRAFFIC_PER_FLUX_LAUNCH = {"mixed": None, "fp64": None}
 # Algorithmic HBM bytes per cell-update of the whole step (FP64 state,
 # stage buffers, accumulator), 2D: 60 doubles.
 BYTES_PER_CELL_UPDATE = 480.0
@@ -267,11 +264,10 @@ def run_reference(args):
     return 0
 
 
-def time_path(B, torch, W, G, h, precision, steps, warmup, dev, limiter=0, stage_kernels=0):
+def time_path(B, torch, W, G, h, precision, steps, warmup, dev, limiter=0):
     """Device-timed steps of one precision; returns (ms/step, profile, final density)."""
     stream = torch.cuda.current_stream()
-    s = B.Solver((N, N), bc=B.BC_PERIODIC, precision=precision, stream=stream, limiter=limiter,
-                 stage_kernels=stage_kernels)
+    s = B.Solver((N, N), bc=B.BC_PERIODIC, precision=precision, stream=stream, limiter=limiter)
     Wd = torch.from_numpy(W).to(dev)
     Gd = torch.from_numpy(G).to(dev)
     s.set_state(Wd, Gd)
@@ -285,7 +281,7 @@ def time_path(B, torch, W, G, h, precision, steps, warmup, dev, limiter=0, stage
     e1.record(stream)
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / steps
-    prof = {k: s.profile_read(k) for k in (B.KC_RECON, B.KC_FACE, B.KC_UPDATE, B.KC_DT, B.KC_STAGE)}
+    prof = {k: s.profile_read(k) for k in (B.KC_RECON, B.KC_FACE, B.KC_UPDATE, B.KC_DT)}
     s.profile(False, False)
     st = s.status()
     s.get_state(Wd, Gd)
@@ -534,10 +530,9 @@ def run_case_batch(count, steps):
     return 0 if st == 0 else 1
 
 
-def run_case(n, precision, steps, stage_kernels=0):
+def run_case(n, precision, steps):
     """A small run of the headline workload for ncu captures: the n^2
-    periodic Fourier-mode + shock state, `steps` CFL steps through the C ABI
-    (stage_kernels 1: the fused stage kernel)."""
+    periodic Fourier-mode + shock state, `steps` CFL steps through the C ABI."""
     import numpy as np
     import torch
 
@@ -545,7 +540,7 @@ def run_case(n, precision, steps, stage_kernels=0):
     from paper_2507_20461_gb300 import inputs as I
 
     W, G, h = I.fourier_shocks_2d(n, SEED)
-    s = B.Solver((n, n), bc=B.BC_PERIODIC, precision=precision, stage_kernels=stage_kernels)
+    s = B.Solver((n, n), bc=B.BC_PERIODIC, precision=precision)
     Wd = torch.from_numpy(np.ascontiguousarray(W)).cuda()
     Gd = torch.from_numpy(np.ascontiguousarray(G)).cuda()
     s.set_state(Wd, Gd)
@@ -553,7 +548,7 @@ def run_case(n, precision, steps, stage_kernels=0):
     torch.cuda.synchronize()
     st = s.status()
     s.close()
-    print(f"case n={n} precision={precision} steps={steps} stage_kernels={stage_kernels} status={st}")
+    print(f"case n={n} precision={precision} steps={steps} status={st}")
     return 0 if st == 0 else 1
 
 
@@ -603,7 +598,6 @@ def main():
                     help="profiling case: N^2 cells of the headline IC, --case-steps CFL steps, then exit (no JSON)")
     ap.add_argument("--case-precision", type=int, default=1, choices=[0, 1])
     ap.add_argument("--case-steps", type=int, default=2)
-    ap.add_argument("--case-stage-kernels", type=int, default=0, choices=[0, 1])
     ap.add_argument("--case-batch", type=int, default=0, metavar="G",
                     help="ncu helper: a small batch of G grids of the batched recipe, then exit")
     ap.add_argument("--cpu-sample", type=int, default=0, metavar="N",
@@ -613,7 +607,7 @@ def main():
     if args.impl == "reference":
         return run_reference(args)
     if args.case:
-        return run_case(args.case, args.case_precision, args.case_steps, args.case_stage_kernels)
+        return run_case(args.case, args.case_precision, args.case_steps)
     if args.case_batch:
         return run_case_batch(args.case_batch, args.case_steps)
     if args.cpu_sample:
@@ -648,10 +642,9 @@ def main():
     torch.cuda.synchronize()
     pipes = measured_pipes(B)
     ms_mixed, prof_mixed, rho_mixed, st_mixed = time_path(B, torch, W, G, h, 1, args.steps, args.warmup, dev)
-    ms_fused, prof_fused, _, st_fused = time_path(B, torch, W, G, h, 1, args.steps, args.warmup, dev, stage_kernels=1)
     ms_fp64, prof_fp64, rho_fp64, st_fp64 = time_path(B, torch, W, G, h, 0, steps64, args.warmup, dev)
     torch.cuda.synchronize()
-    ms_mixed, ms_fused, ms_fp64 = aggregate(ws, [ms_mixed, ms_fused, ms_fp64], dist if ws > 1 else None, dev)
+    ms_mixed, ms_fp64 = aggregate(ws, [ms_mixed, ms_fp64], dist if ws > 1 else None, dev)
     clk = clocks.stop()
 
     # mixed vs FP64 on the same CFL steps (the FP64 path's time steps drive
@@ -708,19 +701,19 @@ def main():
     fp32_nominal = nsm * 128 * 2 * sm_clock * 1e6 / 1e12
     fp64_nominal = nsm * 2 * 2 * sm_clock * 1e6 / 1e12
 
-    # the dominant kernel: the face flux, one launch per direction; units per
-    # launch = faces of one direction x 2 Gauss points
-    units_per_launch = (N + 1) * N * 2
+    # the dominant kernel: the face flux, one launch for both directions;
+    # units per launch = faces x 2 Gauss points
+    units_per_launch = 2 * (N + 1) * N * 2
     n_face, t_face = prof_mixed[B.KC_FACE]
     avg_face_ms = t_face / max(n_face, 1)
     n64, t64 = prof_fp64[B.KC_FACE]
     avg64 = t64 / max(n64, 1)
-    roof = alu_roofline(FACE_GP_2D, units_per_launch / (avg_face_ms * 1e-3), ffma, "face_flux_kernel<float,2,D,true>",
+    roof = alu_roofline(FACE_GP_2D, units_per_launch / (avg_face_ms * 1e-3), ffma, "step_flux_kernel<float,2,false>",
                         "face Gauss point", "measured: FP32 FMA probe (scalar or packed, the larger)", TRAFFIC_PER_FLUX_LAUNCH["mixed"], fp32_nominal)
     roof["transcendentals_per_unit"] = FACE_GP_2D_TRANS
     roof["launch_ms"] = avg_face_ms
     roof["units_per_launch"] = units_per_launch
-    roof64 = alu_roofline(FACE_GP_2D, units_per_launch / (avg64 * 1e-3), dfma, "face_flux_kernel<double,2,D,true>",
+    roof64 = alu_roofline(FACE_GP_2D, units_per_launch / (avg64 * 1e-3), dfma, "step_flux_kernel<double,2,false>",
                           "face Gauss point", "measured: DFMA probe", TRAFFIC_PER_FLUX_LAUNCH["fp64"], fp64_nominal)
     roof64["launch_ms"] = avg64
     for r, key in ((roof, "mixed"), (roof64, "fp64")):
@@ -728,15 +721,7 @@ def main():
         if ex:
             r["executed_flops_per_unit"] = ex
             r["frac_executed"] = r["frac"] * ex / FACE_GP_2D
-    # the fused stage kernel: units per launch = cells (one stage of each)
-    n_st, t_st = prof_fused[B.KC_STAGE]
-    avg_stage_ms = t_st / max(n_st, 1)
-    fused = {"value": ws * N * N / (ms_fused * 1e-3), "unit": "cell-updates/s", "ms_per_step": ms_fused,
-             "stage_launch_ms": avg_stage_ms, "status": st_fused, "vs_three_kernel_ms": ms_fused / ms_mixed,
-             "roofline": alu_roofline(CELL_UPDATE_2D / 2, N * N / (avg_stage_ms * 1e-3), ffma,
-                                      "fused2d_stage_kernel", "cell-stage", "measured: FP32 FMA probe (scalar or packed, the larger)")}
-
-    launches_per_step = 1 + 1 + 2 * (1 + 2 + 1)  # wavespeed, dt, 2 x (poly, 2 face dirs, update)
+    launches_per_step = 1 + 1 + 2 * (1 + 1 + 1)  # wavespeed, dt, 2 x (poly, face flux, update)
     value = ws * N * N / (ms_mixed * 1e-3)
     value64 = ws * N * N / (ms_fp64 * 1e-3)
     hbm_frac = BYTES_PER_CELL_UPDATE * value / ws / (peaks.get("hbm_gbs", 6800.0) * 1e9)
@@ -779,7 +764,6 @@ def main():
         "measured_pipes": pipes,
         "kernel_ms": {name: prof_mixed[k][1] / max(prof_mixed[k][0], 1) for k, name in
                       ((B.KC_RECON, "cell_poly"), (B.KC_FACE, "face_flux"), (B.KC_UPDATE, "update"), (B.KC_DT, "dt"))},
-        "fused_stage_kernel": fused,
         "status": {"mixed": st_mixed, "fp64": st_fp64, "error_run": st_l1},
         "e2e": {"value": ws * e2e_val, "unit": "cell-updates/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
         "gpu_launches": launches_per_step * args.steps,

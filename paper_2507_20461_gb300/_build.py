@@ -13,7 +13,7 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libgenogks.so")
-SOURCES = ["k1d.cu", "k2d.cu", "k3d.cu", "k2d_batch.cu", "k2d_fused.cu", "api.cu", "batch.cu", "static_flux.cu", "analysis.cu", "probe.cu", "k1d_nc.cu"]
+SOURCES = ["k1d.cu", "k2d.cu", "k3d.cu", "k2d_batch.cu", "api.cu", "batch.cu", "static_flux.cu", "analysis.cu", "probe.cu", "k1d_nc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # FP32 division and square root compile to the approximate forms (at most 2
 # and about 1 ulp off; FP64 code is unaffected): the mixed-precision flux and
@@ -40,11 +40,10 @@ def _newest_input() -> float:
     return t
 
 
-# extra flags per translation unit: the fused stage kernels flush FP32
-# denormals (their double-float update never comes near them; measured 1.5%
-# shorter fused stage, 2.4% faster batch), the three-kernel update does not
+# extra flags per translation unit: the batched stage kernel flushes FP32
+# denormals (its double-float update never comes near them; 2.4% faster), the three-kernel update does not
 # (it ran 17% slower)
-UNIT_FLAGS: dict[str, list[str]] = {"k2d_fused.cu": ["-ftz=true"], "k2d_batch.cu": ["-ftz=true"]}
+UNIT_FLAGS: dict[str, list[str]] = {"k2d_batch.cu": ["-ftz=true"]}
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

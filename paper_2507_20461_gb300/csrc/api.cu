@@ -1,12 +1,14 @@
 /* C ABI of libgenogks: handle lifetime, state transfer, and the step driver.
  * The numerics are in kernels.cuh / gks_device.cuh; see include/genogks.h
  * for the contract of every entry point. */
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstring>
 #include <new>
 
 #include "internal.h"
+#include "step_flux.cuh"
 
 namespace {
 
@@ -77,6 +79,10 @@ Layout layout(const gks_grid_t *g, int precision)
     const size_t rs = precision ? sizeof(float) : sizeof(double);
     L.B_elems = (m >= 2) ? (size_t)nv * gks::ncubic(m) * next : 0;
     L.ff_elems = (size_t)3 * nv * ng * face_count(g);
+    /* the step path's grouped layouts share the buffers (step_flux.cuh) */
+    const size_t faces = face_count(g);
+    const size_t Bs = (m >= 2) ? std::max(L.B_elems, gks::group_elems(next, nv * (gks::ncubic(m) + 1))) : 0;
+    const size_t fs = (m >= 2) ? std::max(L.ff_elems, gks::group_elems(faces, 3 * nv)) : L.ff_elems;
     size_t off = 0;
     L.W = off; off = align_up(off + sizeof(double) * nv * ncell);
     L.G = off; off = align_up(off + sizeof(double) * m * nv * ncell);
@@ -84,8 +90,8 @@ Layout layout(const gks_grid_t *g, int precision)
     L.Gs = off; off = align_up(off + sizeof(double) * m * nv * ncell);
     L.Acc = off; off = align_up(off + sizeof(double) * nv * ncell);
     L.small = off; off = align_up(off + 256);
-    L.B = off; off = align_up(off + rs * L.B_elems);
-    L.ff = off; off = align_up(off + rs * L.ff_elems);
+    L.B = off; off = align_up(off + rs * Bs);
+    L.ff = off; off = align_up(off + rs * fs);
     /* FP32 shadows (mixed precision, 2D/3D): hi, lo (nv x cells), g (m x nv x cells) */
     L.shadows = (precision == 1 && m >= 2);
     const size_t shb = L.shadows ? sizeof(float) * (size_t)(2 + m) * nv * ncell : 0;
@@ -166,11 +172,6 @@ int two_stages(gks_ctx *c)
     if (c->shadows) c->g_stale = 1;
     if (c->dim == 1 && c->order != 8) {
         if ((e = gks::nc_launch_step(c)) != cudaSuccess) return cuda_fail(c, e, "RK4 step");
-        return GKS_OK;
-    }
-    if (c->fused) {
-        if ((e = gks::launch_fused2d(c, 1)) != cudaSuccess) return cuda_fail(c, e, "stage 1");
-        if ((e = gks::launch_fused2d(c, 2)) != cudaSuccess) return cuda_fail(c, e, "stage 2");
         return GKS_OK;
     }
     if ((e = run_flux(c, 0, true)) != cudaSuccess) return cuda_fail(c, e, "stage 1 flux");
@@ -311,7 +312,6 @@ int geno_gks_create_sides(const gks_grid_t *grid, double gamma, int order, const
     }
     c->B_elems = L.B_elems;
     c->ff_elems = L.ff_elems;
-    c->fused = (L.shadows && grid->dim == 2 && o.stage_kernels == 1) ? 1 : 0;
 
     gks::KP &P = c->kp;
     std::memset(&P, 0, sizeof(P));

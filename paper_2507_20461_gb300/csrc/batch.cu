@@ -245,7 +245,8 @@ const char *class_name(int k)
 
 /* Size class of a batch: powers of two of the grid count, of the total cell
  * count and of the largest side, with the dimension, precision, limiter
- * and the device's SM count. */
+ * the device's SM count and the fused stage kernel's block size (a cache file
+ * written for another one is not used). */
 std::string size_class(const gks_batch_ctx *b)
 {
     long cells = 0;
@@ -256,8 +257,8 @@ std::string size_class(const gks_batch_ctx *b)
     }
     auto lg = [](double x) { return (int)std::lround(std::log2(x > 1.0 ? x : 1.0)); };
     char k[160];
-    snprintf(k, sizeof k, "2d/p%d/l%d/nb%d/cells%d/side%d/sm%d", b->precision, b->opts.limiter, lg(b->nb), lg((double)cells),
-             lg(side), b->nsm);
+    snprintf(k, sizeof k, "2d/p%d/l%d/nb%d/cells%d/side%d/sm%d/t%d", b->precision, b->opts.limiter, lg(b->nb),
+             lg((double)cells), lg(side), b->nsm, gks::kStageThreads);
     return k;
 }
 
@@ -365,9 +366,9 @@ int tune(gks_batch_ctx *b, double cfl)
         const bool stg = k == gks::BK_STAGE;
         if (stg) nblk = 1;
         float best = 1e30f;
-        LaunchShape bs{stg ? 256 : 128, 2048, b->nsm};
+        LaunchShape bs{128, 2048, b->nsm};
         for (int bi = 0; bi < nblk; ++bi) {
-            const int block = stg ? 256 : blocks_c[bi];
+            const int block = stg ? gks::kStageThreads : blocks_c[bi];
             const int occ = gks::batch_occupancy(k, b->precision, block);
             for (int ci = 0; ci < 4; ++ci) {
                 const long t = stg ? rows_c[ci] : tiles[ci];
@@ -518,7 +519,7 @@ int gks_batch_create(int nbatch, const int *nx, const int *ny, const double *hs,
         return r;
     }
     for (int k : classes_of(b)) {
-        const int block = (k == gks::BK_STAGE) ? 256 : 128;
+        const int block = (k == gks::BK_STAGE) ? gks::kStageThreads : 128;
         const int occ = gks::batch_occupancy(k, b->precision, block);
         b->shape[k] = LaunchShape{block, k == gks::BK_STAGE ? 32 : 4096, b->nsm * (occ > 0 ? occ : 1)};
         int r = build_tiles(b, k, b->shape[k].tile);

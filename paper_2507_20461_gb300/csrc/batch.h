@@ -26,8 +26,9 @@ struct Tile {
 
 enum BatchKernel { BK_SPEED = 0, BK_POLY = 1, BK_FLUX = 2, BK_UPDATE = 3, BK_STAGE = 4, BK_COUNT = 5 };
 
-/* strip width of the fused stage kernel (columns per tile) */
-constexpr int kStageStrip = 62;
+/* strip width of the fused stage kernel (columns per tile) and its threads:
+ * the 63 x faces and 62 y faces of a row are one round of 128 threads */
+constexpr int kStageStrip = 62, kStageThreads = 128;
 
 struct LaunchShape {
     int block;   /* threads per block */

@@ -20,10 +20,8 @@
  *   A  the cubics of row j + 1 and the stage update of row j - 1
  *      (mixed_update_var), each one item per (cell, variable);
  *   B  the faces of row j: its TX + 1 x faces and the TX y faces between
- *      rows j and j + 1, at both Gauss points; a warp takes 32 faces at one
- *      Gauss point (the evaluation of the cubics does not diverge); with
- *      TX = 62 and 256 threads (or TX = 30 and 128) both phases are one
- *      full round.
+ *      rows j and j + 1, a face with both its Gauss points per thread
+ *      (face_pair, face_point); TX = 62 and 128 threads make it one round.
  * Only the first cubic rows and y faces of a chunk, and the two columns on
  * each side of a strip, are evaluated twice (by both blocks that touch them,
  * from the same inputs by the same instructions, so both get the same bits
@@ -32,7 +30,7 @@
  * cubic coefficients nor the face fluxes go through device memory.
  */
 #pragma once
-#include "kernels.cuh"
+#include "step_flux.cuh"
 
 namespace gks {
 
@@ -48,14 +46,13 @@ template <int TX_> struct SweepStrip {
     static constexpr int CX = TX + 2;
     static constexpr int REC = NV * NC;
     static constexpr int BROW = CX * REC, WROW = CX * NV;
-    /* face values: per (face, Gauss point) F, dF/dt, W(dt/2) of the four
-     * variables, global variable order */
+    /* face values: per face F, dF/dt, W(dt/2) of the four variables summed
+     * over its Gauss points, global variable order */
     static constexpr int FV = 3 * NV;
     static constexpr int NXF = TX + 1, NYF = TX;
-    static constexpr int XROW = NXF * 2 * FV, YROW = NYF * 2 * FV;
-    /* flux work: 32-face blocks of x faces, then of y faces, each at two
-     * Gauss points */
-    static constexpr int NXB = (NXF + 31) / 32, NYB = (NYF + 31) / 32, NWI = 2 * (NXB + NYB);
+    static constexpr int XROW = NXF * FV, YROW = NYF * FV;
+    /* flux work: 32-face blocks of x faces, then of y faces */
+    static constexpr int NXB = (NXF + 31) / 32, NYB = (NYF + 31) / 32;
     static constexpr int O_STATE = 0, O_B = O_STATE + NSLOT * SROW, O_W0 = O_B + 2 * BROW, O_XF = O_W0 + 2 * WROW,
                          O_YF = O_XF + XROW, FLOATS = O_YF + 2 * YROW;
     static constexpr size_t SMEM = sizeof(float) * (size_t)FLOATS;
@@ -79,11 +76,6 @@ struct FusedGeo {
     float fh, fih;
 };
 
-__host__ __device__ __forceinline__ FusedGeo fused_geo(const KP &P)
-{
-    return FusedGeo{P.n[0], P.n[1], P.ncell, P.ih, P.fh, P.fih};
-}
-
 /* The stage on the strip of columns x0 .. x0 + TX - 1, rows y0 .. y0 + rows
  * - 1 (clipped to the grid), by the NT threads of the calling block; P holds
  * the scheme constants and boundary types, geo the grid's geometry; smem
@@ -97,7 +89,7 @@ __device__ __forceinline__ void fused2d_strip(const KP &P, const FusedGeo &geo, 
 {
     using T = SweepStrip<TX>;
     constexpr int NV = T::NV, NC = T::NC, WX = T::WX, CX = T::CX;
-    static_assert(NT >= 4 * TX && NT % 32 == 0, "the update of a row takes one thread per (cell, variable)");
+    static_assert(NT % 32 == 0, "the four variables of a cell are updated by neighbouring lanes");
     float *const S = smem + T::O_STATE; /* [slot][field][WX] */
     float *const Bc = smem + T::O_B;    /* [slot][cx][v * NC + k] */
     float *const W0 = smem + T::O_W0;   /* [slot][cx][v] signed cell averages (FP32 hi) */
@@ -172,14 +164,13 @@ __device__ __forceinline__ void fused2d_strip(const KP &P, const FusedGeo &geo, 
         W0[(r & 1) * T::WROW + cx * NV + v] = h0;
     };
 
-    /* flux work item wi (warp-uniform).  y_only: the y faces between rows
-     * j - 1 and j; else the x faces of row j (the first NXB face blocks) and
-     * the y faces between rows j and j + 1 */
-    const float dtf = (float)dt;
-    auto flux_item = [&](int j, int wi, bool y_only) {
-        const int lane = tid & 31, g = wi & 1, fb = wi >> 1;
-        const bool xd = !y_only && fb < T::NXB;
-        const int ix = (xd ? fb : fb - (y_only ? 0 : T::NXB)) * 32 + lane;
+    /* face it of row j (its direction is warp-uniform), both Gauss points.
+     * y_only: the y faces between rows j - 1 and j; else the x faces of row j
+     * (it < 32 NXB), then the y faces between rows j and j + 1 */
+    const float dtf = (float)dt, idt = 1.f / dtf;
+    auto flux_item = [&](int j, int it, bool y_only) {
+        const bool xd = !y_only && it < 32 * T::NXB;
+        const int ix = (xd || y_only) ? it : it - 32 * T::NXB;
         if (xd ? ix >= T::NXF : ix >= T::NYF) return;
         const int yr = y_only ? j : j + 1; /* row of the y faces' upper cells */
         const int fi = x0 + ix;
@@ -198,110 +189,97 @@ __device__ __forceinline__ void fused2d_strip(const KP &P, const FusedGeo &geo, 
         }
         const bool wall = xd ? ((fi == 0 && P.bcs[0][0] >= 2) || (fi == nx && P.bcs[0][1] >= 2))
                              : ((yr == 0 && P.bcs[1][0] >= 2) || (yr == ny && P.bcs[1][1] >= 2));
-        const float gm1 = P.fgm1, ih = geo.fih, adm = P.fadm;
-        float st[2][NV][3], cw[2][NV];
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-            const float4 *cr = reinterpret_cast<const float4 *>(side ? cR : cL);
-            const float4 w4 = *reinterpret_cast<const float4 *>(side ? wR : wL);
-            const float wv[4] = {w4.x, w4.y, w4.z, w4.w};
-            float rc[T::REC];
+        /* one copy of the code for both directions: a y face of the cubic
+         * P(x, y) is the x face of P(y, x), whose coefficients are P's with x
+         * and y swapped (monomials y, x, y^2, xy, x^2, y^3, xy^2, x^2y, x^3),
+         * its momenta swapped (selects on the warp-uniform direction) */
+        constexpr int swp[NC] = {1, 0, 4, 3, 2, 8, 7, 6, 5};
+        LR Wp[2][1][NV], dWp[2][1][2][NV], rc[1], dqc[1];
+        {
+            float rl[T::REC], rr[T::REC];
 #pragma unroll
             for (int k = 0; k < T::REC / 4; ++k) {
-                const float4 q = cr[k];
-                rc[4 * k] = q.x;
-                rc[4 * k + 1] = q.y;
-                rc[4 * k + 2] = q.z;
-                rc[4 * k + 3] = q.w;
+                const float4 l = reinterpret_cast<const float4 *>(cL)[k], q = reinterpret_cast<const float4 *>(cR)[k];
+                rl[4 * k] = l.x, rl[4 * k + 1] = l.y, rl[4 * k + 2] = l.z, rl[4 * k + 3] = l.w;
+                rr[4 * k] = q.x, rr[4 * k + 1] = q.y, rr[4 * k + 2] = q.z, rr[4 * k + 3] = q.w;
             }
-            /* one evaluation code for both directions: a y face of the cubic
-             * P(x, y) is the x face of P(y, x), whose coefficients are P's with
-             * x and y swapped (monomials y, x, y^2, xy, x^2, y^3, xy^2, x^2y,
-             * x^3); its two derivatives swap back */
-            constexpr int swp[NC] = {1, 0, 4, 3, 2, 8, 7, 6, 5};
+            const float4 al = *reinterpret_cast<const float4 *>(wL), ar = *reinterpret_cast<const float4 *>(wR);
+            const LR w[NV] = {LR(al.x, ar.x), xd ? LR(al.y, ar.y) : LR(al.z, ar.z), xd ? LR(al.z, ar.z) : LR(al.y, ar.y),
+                              LR(al.w, ar.w)};
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                float c[NC], out[3];
+                const int u = (v == 1 || v == 2) ? 3 - v : v; /* the swapped variable */
+                LR c[NC], o0[3], o1[3];
 #pragma unroll
-                for (int k = 0; k < NC; ++k) c[k] = xd ? rc[v * NC + k] : rc[v * NC + swp[k]];
-                if (side == 0) CubicEval<float, 2, 0, 1>::run(g, c, out);
-                else CubicEval<float, 2, 0, 0>::run(g, c, out);
-                cw[side][v] = wv[v];
-                st[side][v][0] = wv[v] + out[0];
-                st[side][v][1] = xd ? out[1] : out[2];
-                st[side][v][2] = xd ? out[2] : out[1];
+                for (int k = 0; k < NC; ++k)
+                    c[k] = LR(xd ? rl[v * NC + k] : rl[u * NC + swp[k]], xd ? rr[v * NC + k] : rr[u * NC + swp[k]]);
+                face_pair<LR, 2, 0>(c, w[v], LR(1.f, -1.f), LR(0.f), o0, o1);
+                Wp[0][0][v] = o0[0];
+                Wp[1][0][v] = o1[0];
+                dWp[0][0][0][v] = o0[1];
+                dWp[1][0][0][v] = o1[1];
+                dWp[0][0][1][v] = o0[2];
+                dWp[1][0][1][v] = o1[2];
             }
-            float s[NV];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) s[v] = st[side][v][0];
-            if (!admissible<float, 2>(s, cw[side], gm1, adm)) {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    st[side][v][0] = cw[side][v];
-                    st[side][v][1] = st[side][v][2] = 0.f;
-                }
-            }
+            const LR kc = w[1] * w[1] + w[2] * w[2];
+            rc[0] = w[0];
+            dqc[0] = LR(P.fadm) * (w[0] * w[3] - LR(0.5f) * kc);
         }
-        /* face frame: normal first; for y faces the momenta and the
-         * derivative axes swap (selects on the warp-uniform direction, so
-         * every array index stays a constant) */
-        const bool yd = !xd;
-        float Wl[NV], Wr[NV], dWl[2][NV], dWr[2][NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int u = (v == 1 || v == 2) ? 3 - v : v; /* the swapped variable */
-            Wl[v] = yd ? st[0][u][0] : st[0][v][0];
-            Wr[v] = yd ? st[1][u][0] : st[1][v][0];
-            dWl[0][v] = yd ? st[0][u][2] : st[0][v][1];
-            dWr[0][v] = yd ? st[1][u][2] : st[1][v][1];
-            dWl[1][v] = yd ? st[0][u][1] : st[0][v][2];
-            dWr[1][v] = yd ? st[1][u][1] : st[1][v][2];
-        }
-        float F[NV], Ft[NV], Wh[NV];
-        if (!gks_point_scaled<float, 2, NS>(P.fp, dtf, 1.f / dtf, ih, Wl, Wr, dWl, dWr, F, Ft, Wh)) {
-            atomicOr(status, ST_FLUX);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) F[v] = Ft[v] = Wh[v] = 0.f;
-        }
-        if (wall) F[0] = F[NV - 1] = Ft[0] = Ft[NV - 1] = 0.f;
         float q[3][NV];
+        bool bad = false;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int u = (v == 1 || v == 2) ? 3 - v : v;
-            q[0][v] = yd ? F[u] : F[v];
-            q[1][v] = yd ? Ft[u] : Ft[v];
-            q[2][v] = yd ? Wh[u] : Wh[v];
+        for (int p = 0; p < 2; ++p) {
+            auto average = [&](int, int v) -> LR {
+                const int u = (v == 1 || v == 2) && !xd ? 3 - v : v;
+                return LR(wL[u], wR[u]);
+            };
+            float F[NV], Ft[NV], Wh[NV];
+            if (!face_point<float, 2, NS>(P.fp, P.fadm, dtf, idt, geo.fih, Wp[p], dWp[p], rc, dqc, average, F, Ft, Wh)) {
+                bad = true;
+#pragma unroll
+                for (int v = 0; v < NV; ++v) F[v] = Ft[v] = Wh[v] = 0.f;
+            }
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                q[0][v] = p ? q[0][v] + F[v] : F[v];
+                q[1][v] = p ? q[1][v] + Ft[v] : Ft[v];
+                q[2][v] = p ? q[2][v] + Wh[v] : Wh[v];
+            }
         }
+        if (bad) atomicOr(status, ST_FLUX);
+        if (wall) q[0][0] = q[0][NV - 1] = q[1][0] = q[1][NV - 1] = 0.f;
         float *base = xd ? XF : YF + (yr & 1) * T::YROW;
-        float4 *o = reinterpret_cast<float4 *>(base + (ix * 2 + g) * T::FV);
+        float4 *o = reinterpret_cast<float4 *>(base + ix * T::FV);
 #pragma unroll
-        for (int r = 0; r < 3; ++r) o[r] = make_float4(q[r][0], q[r][1], q[r][2], q[r][3]);
+        for (int r = 0; r < 3; ++r)
+            o[r] = make_float4(q[r][0], xd ? q[r][1] : q[r][2], xd ? q[r][2] : q[r][1], q[r][3]);
     };
 
-    /* stage update of row j, one item per (cell, variable): thread t takes
+    /* stage update of row j, one item per (cell, variable): item t is
      * variable t % 4 of cell t / 4 (the four variables of a cell in four
      * neighbouring lanes, which then gather the new state for its
      * admissibility flags).  Faces: x faces of row j, y faces below (slot of
-     * row j) and above (slot of row j + 1), each face's Gauss points summed
-     * in the order (F0 + F1).  Every thread of the block calls it. */
+     * row j) and above (slot of row j + 1).  Every thread of the block calls it. */
     auto update_row = [&](int j) {
-        const int tx = tid >> 2, v = tid & 3;
-        const int gx = x0 + tx;
-        const bool valid = tid < NV * TX && gx < nx && j < ny;
-        float wn = 1.f;
-        if (valid) {
-            const float *ylo = YF + (j & 1) * T::YROW, *yhi = YF + ((j + 1) & 1) * T::YROW;
-            auto fsum = [&](int q, int vv, int d, int plus) -> float {
-                const float *p = d == 0 ? XF + (tx + plus) * 2 * T::FV : (plus ? yhi : ylo) + tx * 2 * T::FV;
-                return p[q * NV + vv] + p[T::FV + q * NV + vv];
-            };
-            wn = mixed_update_var<2, STAGE>(nc, geo.fih, fsum, uc, W, acc, s0, s1, (long)j * nx + gx, v);
-        }
-        const int base = (tid & 31) & ~3;
-        float w4[NV];
+        for (int it = tid; it < (NV * TX + NT - 1) / NT * NT; it += NT) {
+            const int tx = it >> 2, v = it & 3;
+            const int gx = x0 + tx;
+            const bool valid = it < NV * TX && gx < nx && j < ny;
+            float wn = 1.f;
+            if (valid) {
+                const float *ylo = YF + (j & 1) * T::YROW, *yhi = YF + ((j + 1) & 1) * T::YROW;
+                auto fsum = [&](int q, int vv, int d, int plus) -> float {
+                    const float *p = d == 0 ? XF + (tx + plus) * T::FV : (plus ? yhi : ylo) + tx * T::FV;
+                    return p[q * NV + vv];
+                };
+                wn = mixed_update_var<2, STAGE>(nc, geo.fih, fsum, uc, W, acc, s0, s1, (long)j * nx + gx, v);
+            }
+            const int base = (tid & 31) & ~3;
+            float w4[NV];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) w4[k] = __shfl_sync(0xffffffffu, wn, base + k);
-        if (valid && v == 0) mixed_state_flags<2>(P, w4, status);
+            for (int k = 0; k < NV; ++k) w4[k] = __shfl_sync(0xffffffffu, wn, base + k);
+            if (valid && v == 0) mixed_state_flags<2>(P, w4, status);
+        }
     };
 
     /* The sweep, one loop for the whole chunk.  Iteration j: phase A, the
@@ -338,25 +316,12 @@ __device__ __forceinline__ void fused2d_strip(const KP &P, const FusedGeo &geo, 
         if (j + 1 < y1) load_row(j + 3);
         if (phase != 2) {
             const bool yo = phase == 1;
-            const int nwi = yo ? 2 * T::NYB : T::NWI;
-            for (int wi = tid >> 5; wi < nwi; wi += NT / 32) flux_item(yo ? y0 : j, wi, yo);
+            const int nfi = 32 * (yo ? T::NYB : T::NXB + T::NYB);
+            for (int it = tid; it < nfi; it += NT) flux_item(yo ? y0 : j, it, yo);
         }
         cp_wait();
         __syncthreads();
     }
-}
-
-/* one grid: block (bx, by) sweeps strip bx over the rows' chunk by */
-template <int STAGE, bool NS, int TX, int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) fused2d_stage_kernel(KP P, Shadow s0, Shadow s1, double *__restrict__ W,
-                                                                 float *__restrict__ acc,
-                                                                 const double *__restrict__ dtp,
-                                                                 int *__restrict__ status, int rows)
-{
-    extern __shared__ __align__(16) float smem[];
-    __shared__ UpdC uc;
-    fused2d_strip<STAGE, NS, TX, NT>(P, fused_geo(P), s0, s1, W, acc, dtp[0], status, blockIdx.x * TX,
-                                     blockIdx.y * rows, rows, smem, uc);
 }
 
 } // namespace gks

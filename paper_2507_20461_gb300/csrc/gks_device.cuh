@@ -306,77 +306,91 @@ inline void fill_flux(FluxParams &fp, double gamma, double c1, double c2)
     fp.fmu = (float)fp.mu;
 }
 
-/* The flux of one interface point from derivatives in units of 1 / ih (ih = 1
- * for physical derivatives, 1 / h for cell units: the scale enters the time
- * coefficients instead of every derivative); idt = 1 / dt.  Returns false (and
- * leaves outputs untouched) when a state is not admissible.
+/* The two half streams of a point together: the equilibrium state W0 and its
+ * flux Fk from their collision, the sums of their slope (and time slope)
+ * moments, and the sums S[e] of the two sides' derivatives. */
+template <typename R, int M> struct Streams {
+    R W0[M + 2], Fk[M + 2], WT[M + 2], FT[M + 2], WA[M + 2], FA[M + 2], S[M][M + 2], pl, pr;
+};
+
+/* FP32: both sides at once on left/right lane pairs (packed two-lane instructions) */
+template <int M, bool NS>
+__device__ __forceinline__ bool streams_of(const FluxParams &fp, const LR *W, const LR (*dW)[M + 2], Streams<float, M> &o)
+{
+    HalfStream<LR, M> q;
+    if (!half_stream<LR, M, NS>(W, dW, LR(fp.fgm1), LR(fp.fNtot), LR(1.f, -1.f), q)) return false;
+    o.pl = q.p.l();
+    o.pr = q.p.r();
+#pragma unroll
+    for (int b = 0; b < M + 2; ++b) {
+        o.W0[b] = q.W0[b].sum();
+        o.Fk[b] = q.Fk[b].sum();
+        o.WT[b] = q.WT[b].sum();
+        o.FT[b] = q.FT[b].sum();
+        if constexpr (NS) {
+            o.WA[b] = q.WA[b].sum();
+            o.FA[b] = q.FA[b].sum();
+        }
+#pragma unroll
+        for (int e = 0; e < M; ++e) o.S[e][b] = dW[e][b].sum();
+    }
+    return true;
+}
+
+/* FP64: one side after the other */
+template <int M, bool NS>
+__device__ __forceinline__ bool streams_of(const FluxParams &fp, const double *Wl, const double *Wr,
+                                           const double (*dWl)[M + 2], const double (*dWr)[M + 2], Streams<double, M> &o)
+{
+    HalfStream<double, M> q;
+    if (!half_stream<double, M, NS>(Wl, dWl, fp.gm1, fp.Ntot, 1.0, q)) return false;
+    o.pl = q.p;
+#pragma unroll
+    for (int b = 0; b < M + 2; ++b) {
+        o.W0[b] = q.W0[b];
+        o.Fk[b] = q.Fk[b];
+        o.WT[b] = q.WT[b];
+        o.FT[b] = q.FT[b];
+        if constexpr (NS) {
+            o.WA[b] = q.WA[b];
+            o.FA[b] = q.FA[b];
+        }
+    }
+    if (!half_stream<double, M, NS>(Wr, dWr, fp.gm1, fp.Ntot, -1.0, q)) return false;
+    o.pr = q.p;
+#pragma unroll
+    for (int b = 0; b < M + 2; ++b) {
+        o.W0[b] += q.W0[b];
+        o.Fk[b] += q.Fk[b];
+        o.WT[b] += q.WT[b];
+        o.FT[b] += q.FT[b];
+        if constexpr (NS) {
+            o.WA[b] += q.WA[b];
+            o.FA[b] += q.FA[b];
+        }
+#pragma unroll
+        for (int e = 0; e < M; ++e) o.S[e][b] = dWl[e][b] + dWr[e][b];
+    }
+    return true;
+}
+
+/* The flux of one interface point from its half streams; derivatives in units
+ * of 1 / ih (ih = 1 for physical derivatives, 1 / h for cell units: the scale
+ * enters the time coefficients instead of every derivative); idt = 1 / dt.
+ * Returns false (and leaves outputs untouched) when the equilibrium is not
+ * admissible.
  * NS = false: the Euler flux (physical collision time 0 in the Chapman-Enskog
  * terms).  NS = true: the Navier-Stokes flux with Prandtl number 1, physical
  * collision time tau = mu / p0 of the interface equilibrium, added to the
  * numerical one in the relaxation factor. */
-template <typename R, int M, bool NS = false>
-__device__ __forceinline__ bool gks_point_scaled(const FluxParams &fp, R dt, R idt, R ih, const R *Wl, const R *Wr,
-                                                 const R (*dWl)[M + 2], const R (*dWr)[M + 2], R *F, R *Ft, R *Wh)
+template <typename R, int M, bool NS>
+__device__ __forceinline__ bool flux_of_streams(const FluxParams &fp, R dt, R idt, R ih, const Streams<R, M> &q, R *F,
+                                                R *Ft, R *Wh)
 {
     constexpr int NV = M + 2;
     const R gm1 = pick<R>(fp.gm1, fp.fgm1);
     const R Ntot = pick<R>(fp.Ntot, fp.fNtot);
-    /* Both half streams: the equilibrium state W0 and its flux Fk from their
-     * collision, and the sums of their slope moments.  FP32 takes both sides
-     * at once on left/right lane pairs (packed two-lane instructions). */
-    R W0[NV], Fk[NV], WTs[NV], FTs[NV], WA[NV], FA[NV], pl, pr;
-    if constexpr (std::is_same_v<R, float>) {
-        LR Wq[NV], dq[M][NV];
-#pragma unroll
-        for (int b = 0; b < NV; ++b) {
-            Wq[b] = LR(Wl[b], Wr[b]);
-#pragma unroll
-            for (int e = 0; e < M; ++e) dq[e][b] = LR(dWl[e][b], dWr[e][b]);
-        }
-        HalfStream<LR, M> q;
-        if (!half_stream<LR, M, NS>(Wq, dq, LR(gm1), LR(Ntot), LR(1.f, -1.f), q)) return false;
-        pl = q.p.l();
-        pr = q.p.r();
-#pragma unroll
-        for (int b = 0; b < NV; ++b) {
-            W0[b] = q.W0[b].sum();
-            Fk[b] = q.Fk[b].sum();
-            WTs[b] = q.WT[b].sum();
-            FTs[b] = q.FT[b].sum();
-            if constexpr (NS) {
-                WA[b] = q.WA[b].sum();
-                FA[b] = q.FA[b].sum();
-            }
-        }
-    } else {
-        HalfStream<R, M> q;
-        if (!half_stream<R, M, NS>(Wl, dWl, gm1, Ntot, R(1), q)) return false;
-        pl = q.p;
-#pragma unroll
-        for (int b = 0; b < NV; ++b) {
-            W0[b] = q.W0[b];
-            Fk[b] = q.Fk[b];
-            WTs[b] = q.WT[b];
-            FTs[b] = q.FT[b];
-            if constexpr (NS) {
-                WA[b] = q.WA[b];
-                FA[b] = q.FA[b];
-            }
-        }
-        if (!half_stream<R, M, NS>(Wr, dWr, gm1, Ntot, R(-1), q)) return false;
-        pr = q.p;
-#pragma unroll
-        for (int b = 0; b < NV; ++b) {
-            W0[b] += q.W0[b];
-            Fk[b] += q.Fk[b];
-            WTs[b] += q.WT[b];
-            FTs[b] += q.FT[b];
-            if constexpr (NS) {
-                WA[b] += q.WA[b];
-                FA[b] += q.FA[b];
-            }
-        }
-    }
+    const R *W0 = q.W0, *Fk = q.Fk, *WTs = q.WT, *FTs = q.FT, *WA = q.WA, *FA = q.FA, pl = q.pl, pr = q.pr;
 
     /* Equilibrium.  Its slope and time-slope moments have closed forms in the
      * primitive derivatives:
@@ -403,11 +417,11 @@ __device__ __forceinline__ bool gks_point_scaled(const FluxParams &fp, R dt, R i
         R dr[M], dp[M], dU[M][M], div = R(0);
 #pragma unroll
         for (int e = 0; e < M; ++e) {
-            dr[e] = dWl[e][0] + dWr[e][0];
-            R dE = (dWl[e][M + 1] + dWr[e][M + 1]) - hUU * dr[e];
+            dr[e] = q.S[e][0];
+            R dE = q.S[e][M + 1] - hUU * dr[e];
 #pragma unroll
             for (int i = 0; i < M; ++i) {
-                const R sv = (dWl[e][1 + i] + dWr[e][1 + i]) - U[i] * dr[e];
+                const R sv = q.S[e][1 + i] - U[i] * dr[e];
                 dE -= U[i] * sv;
                 dU[e][i] = sv * inv;
             }
@@ -491,6 +505,27 @@ __device__ __forceinline__ bool gks_point_scaled(const FluxParams &fp, R dt, R i
         }
     }
     return true;
+}
+
+/* one interface point: states and derivatives (units of 1 / ih) of the two sides */
+template <typename R, int M, bool NS = false>
+__device__ __forceinline__ bool gks_point_scaled(const FluxParams &fp, R dt, R idt, R ih, const R *Wl, const R *Wr,
+                                                 const R (*dWl)[M + 2], const R (*dWr)[M + 2], R *F, R *Ft, R *Wh)
+{
+    Streams<R, M> q;
+    if constexpr (std::is_same_v<R, float>) {
+        LR W[M + 2], dW[M][M + 2];
+#pragma unroll
+        for (int b = 0; b < M + 2; ++b) {
+            W[b] = LR(Wl[b], Wr[b]);
+#pragma unroll
+            for (int e = 0; e < M; ++e) dW[e][b] = LR(dWl[e][b], dWr[e][b]);
+        }
+        if (!streams_of<M, NS>(fp, W, dW, q)) return false;
+    } else {
+        if (!streams_of<M, NS>(fp, Wl, Wr, dWl, dWr, q)) return false;
+    }
+    return flux_of_streams<R, M, NS>(fp, dt, idt, ih, q, F, Ft, Wh);
 }
 
 /* the same from physical derivatives */

@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) bk_update(const GridDesc *__restrict__ gd
  * share every scheme constant and boundary type, so the kernel takes one
  * parameter block (its geometry fields unused) as a launch parameter, and
  * per strip only the grid's geometry, state pointers and time step. */
-constexpr int kStageThreads = 256, kStageMinBlocks = 2;
+constexpr int kStageMinBlocks = 4;
 
 template <int STAGE>
 __global__ void __launch_bounds__(kStageThreads, kStageMinBlocks)

@@ -588,7 +588,10 @@ __device__ __forceinline__ void blend_cubic(const KP &P, const R *d, R *b)
     }
 }
 
-template <typename R, int M>
+/* GROUPED = false: B[v][k][ext cell]; true: the step path's layout, the fields
+ * of 32 consecutive cells in rows of 32, v (NC + 1) + k with k = NC the
+ * (mirrored) average itself (step_flux.cuh). */
+template <typename R, int M, bool GROUPED = false>
 __device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R *__restrict__ B, long t)
 {
     constexpr int NV = M + 2, NC = Cubic<R, M>::NC, ND = Cubic<R, M>::ND;
@@ -663,17 +666,25 @@ __device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R
         }
         R b[NC];
         blend_cubic<R, M>(P, d, b);
-        const long base = (long)v * NC;
+        if constexpr (GROUPED) {
+            R *o = B + (size_t)(t >> 5) * (NV * (NC + 1) * 32) + (t & 31) + v * (NC + 1) * 32;
 #pragma unroll
-        for (int kk = 0; kk < NC; ++kk) B[(base + kk) * P.next + t] = b[kk];
+            for (int kk = 0; kk < NC; ++kk) o[kk * 32] = b[kk];
+            const R w = src.w0(v * P.ncell + cl[0]);
+            o[NC * 32] = ((sm[0] >> v) & 1u) ? -w : w;
+        } else {
+            const long base = (long)v * NC;
+#pragma unroll
+            for (int kk = 0; kk < NC; ++kk) B[(base + kk) * P.next + t] = b[kk];
+        }
     }
 }
 
-template <typename R, int M>
+template <typename R, int M, bool GROUPED = false>
 __global__ void __launch_bounds__(128) cell_poly_kernel(KP P, Src<R> src, R *__restrict__ B)
 {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < P.next) cell_poly_item<R, M>(P, src, B, t);
+    if (t < P.next) cell_poly_item<R, M, GROUPED>(P, src, B, t);
 }
 
 template <int M>
@@ -1159,9 +1170,52 @@ __device__ __forceinline__ void mixed_update_cell(const KP &P, const FaceSum &fs
     mixed_state_flags<M>(P, wn, status);
 }
 
-/* STAGE 1: Ws = W - dt/2 L(F) - dt^2/8 L(Ft), Gs = Gauss(W(dt/2)), Acc = -dt L(F) - dt^2/6 L(Ft)
+/* The FP64 stage update of one cell from the face sums over the Gauss points
+ * (weight wg each), fsum(q, v, d, plus) as in mixed_update_var.
+ * STAGE 1: Ws = W - dt/2 L(F) - dt^2/8 L(Ft), Gs = Gauss(W(dt/2)), Acc = -dt L(F) - dt^2/6 L(Ft)
  * STAGE 2: W += Acc - dt^2/3 L(Ft*),        G  = Gauss(W*(dt/2))
  * with L(q)_j = (1/h) sum_d sum_g w_g (q(+d face) - q(-d face)). */
+template <int M, int STAGE, typename FaceSum>
+__device__ __forceinline__ void fp64_update_cell(const KP &P, const FaceSum &fsum, double wg, double dt,
+                                                 double *__restrict__ W, double *__restrict__ G, double *__restrict__ Ws,
+                                                 double *__restrict__ Gs, double *__restrict__ Acc,
+                                                 int *__restrict__ status, long cell)
+{
+    constexpr int NV = M + 2;
+    const double cw = wg * P.ih;
+    double Wn[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        double DF = 0.0, DFt = 0.0;
+#pragma unroll
+        for (int d = 0; d < M; ++d) {
+            if (STAGE == 1) DF += fsum(0, v, d, 1) - fsum(0, v, d, 0);
+            DFt += fsum(1, v, d, 1) - fsum(1, v, d, 0);
+            double *Gout = (STAGE == 1) ? Gs : G;
+            Gout[(d * NV + v) * P.ncell + cell] = (fsum(2, v, d, 1) - fsum(2, v, d, 0)) * cw;
+        }
+        DF *= cw;
+        DFt *= cw;
+        if (STAGE == 1) {
+            Wn[v] = W[v * P.ncell + cell] - 0.5 * dt * DF - dt * dt * 0.125 * DFt;
+            Ws[v * P.ncell + cell] = Wn[v];
+            Acc[v * P.ncell + cell] = -dt * DF - dt * dt / 6.0 * DFt;
+        } else {
+            Wn[v] = W[v * P.ncell + cell] + Acc[v * P.ncell + cell] - dt * dt / 3.0 * DFt;
+            W[v * P.ncell + cell] = Wn[v];
+        }
+    }
+    double ke = 0.0;
+#pragma unroll
+    for (int a = 0; a < M; ++a) ke += Wn[1 + a] * Wn[1 + a];
+    const double p = (P.gamma - 1.0) * (Wn[M + 1] - 0.5 * ke / Wn[0]);
+    int st = 0;
+    if (!(Wn[0] > 0.0)) st |= ST_RHO;
+    if (!(p > 0.0)) st |= ST_P;
+    if (!isfinite(p) || !isfinite(Wn[0])) st |= ST_NAN;
+    if (st) atomicOr(status, st);
+}
+
 template <typename R, int M, int STAGE>
 __device__ __forceinline__ void update_item(const KP &P, const R *__restrict__ ff, double dt, double *__restrict__ W,
                                             double *__restrict__ G, double *__restrict__ Ws, double *__restrict__ Gs,
@@ -1194,7 +1248,6 @@ __device__ __forceinline__ void update_item(const KP &P, const R *__restrict__ f
     const int i = (int)fdivmod(P.dn[0], (unsigned)cell, q0);
     const int j = (M >= 2) ? (int)fdivmod(P.dn[1], q0, q1) : 0;
     const int k = (M >= 3) ? (int)q1 : 0;
-    const double ih = P.ih, wg = 1.0 / NG;
     const long nft = P.nftot;
     long fp[M], fm[M];
 #pragma unroll
@@ -1202,45 +1255,14 @@ __device__ __forceinline__ void update_item(const KP &P, const R *__restrict__ f
         fp[d] = face_of<M>(P, d, i, j, k, 1);
         fm[d] = face_of<M>(P, d, i, j, k, 0);
     }
-    double Wn[NV];
+    /* sums over the Gauss points ff[q][v][g][face] */
+    auto fsum = [&](int q, int v, int d, int plus) -> double {
+        double a = 0.0;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        double DF = 0.0, DFt = 0.0;
-#pragma unroll
-        for (int d = 0; d < M; ++d) {
-            double Dh = 0.0;
-#pragma unroll
-            for (int g = 0; g < NG; ++g) {
-                const long o0 = ((long)(0 * NV + v) * NG + g) * nft, o1 = ((long)(1 * NV + v) * NG + g) * nft,
-                           o2 = ((long)(2 * NV + v) * NG + g) * nft;
-                DF += (double)ff[o0 + fp[d]] - (double)ff[o0 + fm[d]];
-                DFt += (double)ff[o1 + fp[d]] - (double)ff[o1 + fm[d]];
-                Dh += (double)ff[o2 + fp[d]] - (double)ff[o2 + fm[d]];
-            }
-            double *Gout = (STAGE == 1) ? Gs : G;
-            Gout[(d * NV + v) * P.ncell + cell] = Dh * wg * ih;
-        }
-        DF *= wg * ih;
-        DFt *= wg * ih;
-        if (STAGE == 1) {
-            Ws[v * P.ncell + cell] = W[v * P.ncell + cell] - 0.5 * dt * DF - dt * dt * 0.125 * DFt;
-            Acc[v * P.ncell + cell] = -dt * DF - dt * dt / 6.0 * DFt;
-            Wn[v] = Ws[v * P.ncell + cell];
-        } else {
-            const double w = W[v * P.ncell + cell] + Acc[v * P.ncell + cell] - dt * dt / 3.0 * DFt;
-            W[v * P.ncell + cell] = w;
-            Wn[v] = w;
-        }
-    }
-    double ke = 0.0;
-#pragma unroll
-    for (int a = 0; a < M; ++a) ke += Wn[1 + a] * Wn[1 + a];
-    const double p = (P.gamma - 1.0) * (Wn[M + 1] - 0.5 * ke / Wn[0]);
-    int st = 0;
-    if (!(Wn[0] > 0.0)) st |= ST_RHO;
-    if (!(p > 0.0)) st |= ST_P;
-    if (!isfinite(p) || !isfinite(Wn[0])) st |= ST_NAN;
-    if (st) atomicOr(status, st);
+        for (int g = 0; g < NG; ++g) a += (double)ff[((long)(q * NV + v) * NG + g) * nft + (plus ? fp[d] : fm[d])];
+        return a;
+    };
+    fp64_update_cell<M, STAGE>(P, fsum, 1.0 / NG, dt, W, G, Ws, Gs, Acc, status, cell);
 }
 
 template <typename R, int M, int STAGE>
@@ -1345,6 +1367,7 @@ static __global__ void dt_from_speed_kernel(const unsigned long long *__restrict
         dt = fmin(dt, cfl_h / nu);
     }
     dtp[0] = dt;
+    dtp[1] = 1.0 / dt;
     if (updc) store_updc(updc, make_updc(dt, cw));
 }
 
@@ -1352,6 +1375,7 @@ static __global__ void dt_from_speed_kernel(const unsigned long long *__restrict
 static __global__ void set_dt_kernel(double *__restrict__ dtp, double dt, float *__restrict__ updc, double cw)
 {
     dtp[0] = dt;
+    dtp[1] = 1.0 / dt;
     if (updc) store_updc(updc, make_updc(dt, cw));
 }
 

@@ -2,6 +2,7 @@
  * per-dimension translation units k1d.cu, k2d.cu, k3d.cu. */
 #pragma once
 #include "internal.h"
+#include "step_flux.cuh"
 
 namespace gks {
 
@@ -17,10 +18,8 @@ template <> inline Src<float> stage_src<float>(gks_ctx *c, int input)
 }
 
 /* flux = false: interface states into fs_dev; flux = true: fluxes per Gauss
- * point into c->ff, or (sums, FP32 multi-D step path) per-face sums over the
- * Gauss points */
-template <typename R, int M>
-static cudaError_t flux_impl(gks_ctx *c, int input, double *fs_dev, bool flux, bool sums = false)
+ * point into c->ff */
+template <typename R, int M> static cudaError_t flux_impl(gks_ctx *c, int input, double *fs_dev, bool flux)
 {
     const KP &P = c->kp;
     R *ff = (R *)c->ff;
@@ -46,17 +45,9 @@ static cudaError_t flux_impl(gks_ctx *c, int input, double *fs_dev, bool flux, b
             ProfScope ps(c, GKS_KC_FACE);
 #define GKS_FACE(D)                                                                                           \
     if (d == D) {                                                                                             \
-        if constexpr (sizeof(R) == sizeof(float)) {                                                           \
-            if (flux && sums && P.fp.mu > 0.0)                                                                \
-                { face_flux_prepare<R, M, D, true, true, true>(); face_flux_kernel<R, M, D, true, true, true><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, nullptr, ff, c->status); } \
-            else if (flux && sums)                                                                            \
-                { face_flux_prepare<R, M, D, true, false, true>(); face_flux_kernel<R, M, D, true, false, true><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, nullptr, ff, c->status); } \
-        }                                                                                                     \
-        if (flux && !(sizeof(R) == sizeof(float) && sums)) {                                                 \
-            if (P.fp.mu > 0.0) { face_flux_prepare<R, M, D, true, true>(); face_flux_kernel<R, M, D, true, true><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, nullptr, ff, c->status); } \
-            else { face_flux_prepare<R, M, D, true>(); face_flux_kernel<R, M, D, true><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, nullptr, ff, c->status); } \
-        }                                                                                                     \
         if (!flux) { face_flux_prepare<R, M, D, false>(); face_flux_kernel<R, M, D, false><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, fs_dev, nullptr, c->status); } \
+        else if (P.fp.mu > 0.0) { face_flux_prepare<R, M, D, true, true>(); face_flux_kernel<R, M, D, true, true><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, nullptr, ff, c->status); } \
+        else { face_flux_prepare<R, M, D, true>(); face_flux_kernel<R, M, D, true><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, nullptr, ff, c->status); } \
     }
             GKS_FACE(0)
             GKS_FACE(1)
@@ -67,6 +58,25 @@ static cudaError_t flux_impl(gks_ctx *c, int input, double *fs_dev, bool flux, b
     return cudaGetLastError();
 }
 
+/* the multi-D step path: reconstruction and face sums (step_flux.cuh) */
+template <typename R, int M, bool NS> static cudaError_t step_flux_impl(gks_ctx *c, int input)
+{
+    const KP &P = c->kp;
+    R *B = (R *)c->B;
+    constexpr int BT = kStepFluxBlock;
+    static const bool prep = (smem_carveout_for(step_flux_kernel<R, M, NS>, kStepFluxMinBlocks<R, M, NS>), true);
+    (void)prep;
+    {
+        ProfScope ps(c, GKS_KC_RECON);
+        cell_poly_kernel<R, M, true><<<blocks_for(P.next), kBlock, 0, c->stream>>>(P, stage_src<R>(c, input), B);
+    }
+    const unsigned nb0 = blocks_for(P.nface[0], BT), nb1 = nb0 + blocks_for(P.nface[1], BT);
+    const unsigned nb = M == 3 ? nb1 + blocks_for(P.nface[2], BT) : nb1;
+    ProfScope ps(c, GKS_KC_FACE);
+    step_flux_kernel<R, M, NS><<<nb, BT, 0, c->stream>>>(P, B, c->dt, (R *)c->ff, c->status, nb0, nb1);
+    return cudaGetLastError();
+}
+
 template <int M> cudaError_t launch_states(gks_ctx *c, int input, double *fs_dev)
 {
     return c->precision ? flux_impl<float, M>(c, input, fs_dev, false) : flux_impl<double, M>(c, input, fs_dev, false);
@@ -74,22 +84,31 @@ template <int M> cudaError_t launch_states(gks_ctx *c, int input, double *fs_dev
 
 template <int M> cudaError_t launch_flux(gks_ctx *c, int input, bool sums)
 {
-    return c->precision ? flux_impl<float, M>(c, input, nullptr, true, sums)
-                        : flux_impl<double, M>(c, input, nullptr, true, sums);
+    if constexpr (M >= 2) {
+        const bool ns = c->kp.fp.mu > 0.0;
+        if (sums && c->precision) return ns ? step_flux_impl<float, M, true>(c, input) : step_flux_impl<float, M, false>(c, input);
+        if (sums) return ns ? step_flux_impl<double, M, true>(c, input) : step_flux_impl<double, M, false>(c, input);
+    }
+    return c->precision ? flux_impl<float, M>(c, input, nullptr, true) : flux_impl<double, M>(c, input, nullptr, true);
+}
+
+template <typename R, int M, int STAGE> static void update_launch(gks_ctx *c)
+{
+    const unsigned nb = blocks_for(c->kp.ncell, 256);
+    const R *ff = (const R *)c->ff;
+    if constexpr (M == 1)
+        update_kernel<R, M, STAGE><<<nb, 256, 0, c->stream>>>(c->kp, ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0,
+                                                              c->s1, c->status, c->updc);
+    else
+        step_update_kernel<R, M, STAGE><<<nb, 256, 0, c->stream>>>(c->kp, ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc,
+                                                                   c->s0, c->s1, c->status, c->updc);
 }
 
 template <typename R, int M> static cudaError_t update_impl(gks_ctx *c, int stage)
 {
-    const KP &P = c->kp;
-    const unsigned nb = blocks_for(P.ncell, 256);
-    const R *ff = (const R *)c->ff;
     ProfScope ps(c, GKS_KC_UPDATE);
-    if (stage == 1)
-        update_kernel<R, M, 1><<<nb, 256, 0, c->stream>>>(P, ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1,
-                                                          c->status, c->updc);
-    else
-        update_kernel<R, M, 2><<<nb, 256, 0, c->stream>>>(P, ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1,
-                                                          c->status, c->updc);
+    if (stage == 1) update_launch<R, M, 1>(c);
+    else update_launch<R, M, 2>(c);
     return cudaGetLastError();
 }
 
