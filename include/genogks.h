@@ -332,15 +332,12 @@ int gks_batch_set_state(gks_batch_t b, int grid, const double *W, const double *
 int gks_batch_get_state(gks_batch_t b, int grid, double *W, double *G, int on_device);
 
 /* nsteps steps of every grid, grid b with dt_b = cfl h_b / (its max |u_d| + c)
- * computed on the device.  Mixed precision: per stage one persistent launch
- * of the fused stage kernel (reconstruction, flux and update through shared
- * memory), its blocks taking strips of a list spanning every grid from a
- * work counter; FP64: per stage three
- * persistent kernels (per-cell reconstruction, face flux, update) walk tile
- * lists spanning all grids.  The first call picks the tile sizes (rows per
- * strip) and block sizes by timing candidates (an autotuner; only scratch
- * buffers are written), then records one step into a CUDA graph; later calls
- * replay the graph (a new cfl re-records it).  The tuner's choices are cached
+ * computed on the device.  Per stage three kernels (per-cell reconstruction,
+ * face flux, update) over tile lists spanning all grids.  The first call picks
+ * the wave-speed kernel's tile and block size by timing candidates (an
+ * autotuner; only scratch is written), then records one step into a CUDA
+ * graph; later calls replay the graph (a new cfl re-records it).  The tuner's
+ * choices are cached
  * per (dimension, precision, limiter, size class of the batch, SM count): in
  * the process, and in the file named by the environment variable
  * GKS_TUNE_CACHE if set (one JSON object per line, appended); a batch whose
@@ -349,10 +346,10 @@ int gks_batch_get_state(gks_batch_t b, int grid, double *W, double *G, int on_de
  * that stream waits for it. */
 int gks_batch_run(gks_batch_t b, double cfl, int nsteps);
 
-/* JSON text of the launch shapes the tuner picked (per kernel class: block
- * size, items per tile or rows per strip, persistent blocks, measured ms;
- * "cached": true and no timings when they came from the cache, with the
- * size-class key); "" before the first gks_batch_run.  Owned by the handle. */
+/* JSON text of the launch shapes (per kernel class: block size, items per
+ * tile, blocks, and for a tuned class the measured ms; the mixed-precision
+ * stage kernels as one entry "stage"; "cached": true and no timings when the
+ * choices came from the cache, with the size-class key); "" before the first gks_batch_run.  Owned by the handle. */
 const char *gks_batch_tuning(gks_batch_t b);
 
 /* Synchronise and return the status word (as gks_status): the OR of every

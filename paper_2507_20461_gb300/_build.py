@@ -17,8 +17,7 @@ SOURCES = ["k1d.cu", "k2d.cu", "k3d.cu", "k2d_batch.cu", "api.cu", "batch.cu", "
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # FP32 division and square root compile to the approximate forms (at most 2
 # and about 1 ulp off; FP64 code is unaffected): the mixed-precision flux and
-# reconstruction issue fewer instructions and the 2048^2 step is 4% shorter,
-# the fused stage kernel 9%.  Denormals are kept (flushing them slowed the
+# reconstruction issue fewer instructions and the 2048^2 step is 4% shorter.  Denormals are kept (flushing them slowed the
 # double-float update).
 FLAGS = ["-std=c++17", "-O3", "-prec-div=false", "-prec-sqrt=false", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler",
          "-O2"]
@@ -40,12 +39,6 @@ def _newest_input() -> float:
     return t
 
 
-# extra flags per translation unit: the batched stage kernel flushes FP32
-# denormals (its double-float update never comes near them; 2.4% faster), the three-kernel update does not
-# (it ran 17% slower)
-UNIT_FLAGS: dict[str, list[str]] = {"k2d_batch.cu": ["-ftz=true"]}
-
-
 def build(force: bool = False, verbose: bool = False) -> str:
     srcs = [s for s in SOURCES if os.path.exists(os.path.join(CSRC, s))]
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_input():
@@ -56,7 +49,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
     def compile_one(src: str) -> str:
         obj = os.path.join(objdir, src.replace(".cu", ".o"))
-        cmd = [cc, *FLAGS, *UNIT_FLAGS.get(src, []), *ARCH, "-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [cc, *FLAGS, *ARCH, "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")

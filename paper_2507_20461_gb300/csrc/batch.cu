@@ -1,12 +1,10 @@
 /* C ABI of the batched 2D mode (gks_batch_*): many independent grids of
- * uneven sizes, persistent kernels over tile work lists, per-grid time steps
- * on the device, one step captured into a CUDA graph and replayed.  Mixed
- * precision runs each stage as one persistent launch of the fused stage
- * kernel over a list of strips of every grid (persistent blocks take the
- * strips from a work counter); FP64 runs the three kernel
- * classes (reconstruction, flux, update).  The tile size and block size of
- * every kernel class are picked by timing the candidates on the actual grids
- * before the graph is recorded; the choices are cached per (dimension,
+ * uneven sizes, kernels over tile work lists spanning every grid, per-grid time
+ * steps on the device, one step captured into a CUDA graph and replayed.  Each
+ * stage runs the three kernel classes of the single-grid step path
+ * (reconstruction, face flux, update), one block per tile.  The wave-speed
+ * kernel's tile and block size are picked by timing the candidates on the
+ * actual grids before the graph is recorded, and cached per (dimension,
  * precision, size class of the batch, SM count), in the process and, if the
  * environment variable GKS_TUNE_CACHE names a file, in that file (one JSON
  * object per line), so a batch of the same size class skips the timing. */
@@ -23,6 +21,7 @@
 #include <vector>
 
 #include "batch.h"
+#include "step_flux.cuh"
 
 using gks::BatchLaunch;
 using gks::GridDesc;
@@ -44,7 +43,7 @@ struct gks_batch_ctx {
     double *dt;
     unsigned long long *smax;
     int *status; /* per-grid status words status[g] (OR of the ST_* bits) */
-    int *queue;  /* work counters of the fused stage kernel (one per stage) */
+    float *updc; /* mixed precision: per-grid stage constants (UpdC, 10 floats each) */
     Tile *tiles[gks::BK_COUNT];
     int ntiles[gks::BK_COUNT];
     LaunchShape shape[gks::BK_COUNT];
@@ -122,27 +121,8 @@ long items(const gks::KP &P, int k, int dir)
     case gks::BK_SPEED:
     case gks::BK_UPDATE: return P.ncell;
     case gks::BK_POLY: return P.next;
-    /* face Gauss points, rounded up to whole 128-item groups (the FP32 flux
-     * maps each group to one block; items past the last face write nothing) */
-    default: return (P.nface[dir] * 2 + 127) / 128 * 128;
+    default: return P.nface[dir];
     }
-}
-
-/* the strips of the fused stage kernel: per grid, columns in strips of
- * kStageStrip, rows in chunks of `rows` */
-void stage_tiles(const gks_batch_ctx *b, long rows, std::vector<Tile> &v)
-{
-    for (int g = 0; g < b->nb; ++g) {
-        const gks::KP &P = b->hd[g].P;
-        for (int x0 = 0; x0 < P.n[0]; x0 += gks::kStageStrip)
-            for (long y0 = 0; y0 < P.n[1]; y0 += rows) v.push_back(Tile{g, x0, y0, y0 + rows < P.n[1] ? y0 + rows : P.n[1]});
-    }
-    /* largest strips first (columns x rows), so the work counter ends on small ones */
-    auto cost = [b](const Tile &t) {
-        const int w = std::min(gks::kStageStrip, b->hd[t.grid].P.n[0] - t.kind);
-        return (long)w * (t.end - t.begin);
-    };
-    std::stable_sort(v.begin(), v.end(), [&](const Tile &a, const Tile &c) { return cost(a) > cost(c); });
 }
 
 int build_tiles(gks_batch_ctx *b, int k, long tile)
@@ -150,17 +130,13 @@ int build_tiles(gks_batch_ctx *b, int k, long tile)
     /* the previous list may still be read by work on the internal stream */
     cudaError_t se = cudaStreamSynchronize(b->stream);
     if (se != cudaSuccess) return bcuda(b, se, "tile list");
-    /* flux tiles start on 128-item groups (one group = one 128-thread block
-     * of the FP32 face mapping, whose face sums synchronise the block) */
-    if (k == gks::BK_FLUX && tile % 128 != 0) return bfail(b, GKS_ERR_ARG, "flux tiles must be whole 128-item groups");
     std::vector<Tile> v;
-    if (k == gks::BK_STAGE) stage_tiles(b, tile, v);
-    for (int g = 0; g < b->nb && k != gks::BK_STAGE; ++g) {
+    for (int g = 0; g < b->nb; ++g) {
         const gks::KP &P = b->hd[g].P;
         const int ndir = (k == gks::BK_FLUX) ? 2 : 1;
         for (int d = 0; d < ndir; ++d) {
             const long n = items(P, k, d);
-            for (long s = 0; s < n; s += tile) v.push_back(Tile{g, d, s, s + tile < n ? s + tile : n});
+            for (long s = 0; s < n; s += tile) v.push_back(Tile{2u * (unsigned)g + (unsigned)d, (unsigned)s});
         }
     }
     if (b->tiles[k]) cudaFree(b->tiles[k]);
@@ -175,7 +151,7 @@ int build_tiles(gks_batch_ctx *b, int k, long tile)
 
 BatchLaunch launch_of(gks_batch_ctx *b, int k)
 {
-    return BatchLaunch{b->dd, b->tiles[k], b->ntiles[k], b->dt, b->smax, b->status, &b->hd[0].P, b->queue};
+    return BatchLaunch{b->dd, b->tiles[k], b->ntiles[k], b->dt, b->updc, b->smax, b->status, &b->hd[0].P};
 }
 
 cudaError_t run_class(gks_batch_ctx *b, int k, int stage)
@@ -185,12 +161,38 @@ cudaError_t run_class(gks_batch_ctx *b, int k, int stage)
     const bool f = b->precision == 1;
     switch (k) {
     case gks::BK_SPEED: return f ? gks::batch_speed<float>(L, S, b->stream) : gks::batch_speed<double>(L, S, b->stream);
-    /* the three stage kernels run the FP64 batches; mixed precision runs the fused stage kernel */
-    case gks::BK_POLY: return f ? cudaErrorInvalidValue : gks::batch_poly<double>(L, S, stage, b->stream);
-    case gks::BK_FLUX: return f ? cudaErrorInvalidValue : gks::batch_flux<double>(L, S, stage, b->stream);
-    case gks::BK_STAGE: return f ? gks::batch_stage(L, S, stage, b->stream) : cudaErrorInvalidValue;
-    default: return f ? cudaErrorInvalidValue : gks::batch_update<double>(L, S, stage, b->stream);
+    case gks::BK_POLY: return f ? gks::batch_poly<float>(L, S, stage, b->stream) : gks::batch_poly<double>(L, S, stage, b->stream);
+    case gks::BK_FLUX: return f ? gks::batch_flux<float>(L, S, stage, b->stream) : gks::batch_flux<double>(L, S, stage, b->stream);
+    case gks::BK_UPDATE: return f ? gks::batch_update<float>(L, S, stage, b->stream) : gks::batch_update<double>(L, S, stage, b->stream);
+    default: break;
     }
+    /* BK_STAGE: a whole stage */
+    for (int kk : {gks::BK_POLY, gks::BK_FLUX, gks::BK_UPDATE}) {
+        const cudaError_t e = run_class(b, kk, stage);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+/* Launch shape of class k.  Stage kernels: one block per tile, one item per
+ * thread (block threads a tile).  Wave speed: tiles of `tile` cells walked by
+ * a persistent grid of the resident blocks. */
+int set_shape(gks_batch_ctx *b, int k, int block, long tile)
+{
+    if (k == gks::BK_STAGE) {
+        for (int kk : {gks::BK_POLY, gks::BK_FLUX, gks::BK_UPDATE}) {
+            int r = set_shape(b, kk, 0, 0);
+            if (r) return r;
+        }
+        b->shape[k] = b->shape[gks::BK_FLUX];
+        return GKS_OK;
+    }
+    if (k != gks::BK_SPEED) tile = block = (k == gks::BK_FLUX) ? gks::kStepFluxBlock : 128;
+    int r = build_tiles(b, k, tile);
+    if (r) return r;
+    const int occ = (k == gks::BK_SPEED) ? gks::batch_occupancy(b->precision, block) : 0;
+    b->shape[k] = LaunchShape{block, tile, k == gks::BK_SPEED ? b->nsm * (occ > 0 ? occ : 1) : b->ntiles[k]};
+    return GKS_OK;
 }
 
 /* one full step on the internal stream */
@@ -198,16 +200,8 @@ int enqueue_step(gks_batch_ctx *b, double cfl)
 {
     cudaError_t e = cudaMemsetAsync(b->smax, 0, sizeof(unsigned long long) * b->nb, b->stream);
     if (e == cudaSuccess) e = run_class(b, gks::BK_SPEED, 1);
-    if (e == cudaSuccess) e = gks::batch_dt(b->dd, b->nb, cfl, b->smax, b->dt, b->stream);
-    for (int stage = 1; stage <= 2 && e == cudaSuccess; ++stage) {
-        if (b->precision == 1) {
-            e = run_class(b, gks::BK_STAGE, stage);
-            continue;
-        }
-        e = run_class(b, gks::BK_POLY, stage);
-        if (e == cudaSuccess) e = run_class(b, gks::BK_FLUX, stage);
-        if (e == cudaSuccess) e = run_class(b, gks::BK_UPDATE, stage);
-    }
+    if (e == cudaSuccess) e = gks::batch_dt(b->dd, b->nb, cfl, b->smax, b->dt, b->updc, b->stream);
+    for (int stage = 1; stage <= 2 && e == cudaSuccess; ++stage) e = run_class(b, gks::BK_STAGE, stage);
     return e == cudaSuccess ? GKS_OK : bcuda(b, e, "batched step");
 }
 
@@ -229,8 +223,8 @@ float time_class(gks_batch_ctx *b, int k)
     return ms;
 }
 
-/* The kernel classes a batch runs: mixed precision the wave speed and the
- * fused stage kernel, FP64 the wave speed and the three stage kernels. */
+/* The kernel classes a batch reports: the wave speed, which is tuned, and the
+ * three stage kernels, one by one in FP64 and as one entry in mixed precision. */
 std::vector<int> classes_of(const gks_batch_ctx *b)
 {
     if (b->precision == 1) return {gks::BK_SPEED, gks::BK_STAGE};
@@ -245,8 +239,8 @@ const char *class_name(int k)
 
 /* Size class of a batch: powers of two of the grid count, of the total cell
  * count and of the largest side, with the dimension, precision, limiter
- * the device's SM count and the fused stage kernel's block size (a cache file
- * written for another one is not used). */
+ * the device's SM count and the face flux's block size (a cache file written
+ * for other kernels is not used). */
 std::string size_class(const gks_batch_ctx *b)
 {
     long cells = 0;
@@ -258,7 +252,7 @@ std::string size_class(const gks_batch_ctx *b)
     auto lg = [](double x) { return (int)std::lround(std::log2(x > 1.0 ? x : 1.0)); };
     char k[160];
     snprintf(k, sizeof k, "2d/p%d/l%d/nb%d/cells%d/side%d/sm%d/t%d", b->precision, b->opts.limiter, lg(b->nb),
-             lg((double)cells), lg(side), b->nsm, gks::kStageThreads);
+             lg((double)cells), lg(side), b->nsm, gks::kStepFluxBlock);
     return k;
 }
 
@@ -320,24 +314,13 @@ void tune_file_append(const std::string &key, const TuneEntry &t)
     std::fclose(f);
 }
 
-/* the shapes of a cached entry: rebuild the tile lists */
-int apply_shapes(gks_batch_ctx *b, const TuneEntry &t)
-{
-    for (int k : classes_of(b)) {
-        int r = build_tiles(b, k, t.shape[k].tile);
-        if (r) return r;
-        b->shape[k] = t.shape[k];
-    }
-    return GKS_OK;
-}
-
-/* Autotuner: for every kernel class the batch runs, tile size x block size
- * candidates (the fused stage kernel: rows per strip), persistent grid = SMs
- * x resident blocks; keep the fastest.  Runs only kernels that write scratch
- * (wave speeds, coefficients, face fluxes, stage-1 outputs), so the state is
- * unchanged.  A batch of a size class tuned before (in this process or in
- * the GKS_TUNE_CACHE file) takes the cached shapes without timing. */
-int tune(gks_batch_ctx *b, double cfl)
+/* Autotuner of the wave-speed kernel: tile size x block size candidates,
+ * persistent grid = SMs x resident blocks; keep the fastest.  The stage
+ * kernels' shapes are fixed (set_shape).  Runs only the wave speed (and its
+ * time steps), so the state is unchanged.  A batch of a size class tuned
+ * before (in this process or in the GKS_TUNE_CACHE file) takes the cached
+ * shape without timing. */
+int tune(gks_batch_ctx *b)
 {
     const std::string key = size_class(b);
     {
@@ -345,7 +328,8 @@ int tune(gks_batch_ctx *b, double cfl)
         tune_file_read();
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
-            int r = apply_shapes(b, it->second);
+            const LaunchShape &sp = it->second.shape[gks::BK_SPEED];
+            int r = set_shape(b, gks::BK_SPEED, sp.block, sp.tile);
             if (r) return r;
             int pos = snprintf(b->tuning, sizeof(b->tuning), "{\"cached\": true, \"key\": \"%s\"", key.c_str());
             for (int k : classes_of(b))
@@ -357,51 +341,34 @@ int tune(gks_batch_ctx *b, double cfl)
         }
     }
     const long tiles[] = {512, 2048, 8192, 32768};
-    const long rows_c[] = {16, 32, 64, 128};
     int pos = 0;
     pos += snprintf(b->tuning + pos, sizeof(b->tuning) - pos, "{\"cached\": false, \"key\": \"%s\"", key.c_str());
-    for (int k : classes_of(b)) {
-        const int blocks_c[2] = {128, 256};
-        int nblk = (k == gks::BK_POLY || k == gks::BK_FLUX) ? 1 : 2;
-        const bool stg = k == gks::BK_STAGE;
-        if (stg) nblk = 1;
-        float best = 1e30f;
-        LaunchShape bs{128, 2048, b->nsm};
-        for (int bi = 0; bi < nblk; ++bi) {
-            const int block = stg ? gks::kStageThreads : blocks_c[bi];
-            const int occ = gks::batch_occupancy(k, b->precision, block);
-            for (int ci = 0; ci < 4; ++ci) {
-                const long t = stg ? rows_c[ci] : tiles[ci];
-                int r = build_tiles(b, k, t);
-                if (r) return r;
-                b->shape[k].block = block;
-                b->shape[k].blocks = b->nsm * (occ > 0 ? occ : 1);
-                if (k == gks::BK_SPEED) cudaMemsetAsync(b->smax, 0, sizeof(unsigned long long) * b->nb, b->stream);
-                const float ms = time_class(b, k);
-                if (ms < best) {
-                    best = ms;
-                    bs = b->shape[k];
-                    bs.tile = t;
-                }
+    float best = 1e30f;
+    LaunchShape bs{128, tiles[0], b->nsm};
+    for (int block : {128, 256}) {
+        for (long t : tiles) {
+            int r = set_shape(b, gks::BK_SPEED, block, t);
+            if (r) return r;
+            cudaMemsetAsync(b->smax, 0, sizeof(unsigned long long) * b->nb, b->stream);
+            const float ms = time_class(b, gks::BK_SPEED);
+            if (ms < best) {
+                best = ms;
+                bs = b->shape[gks::BK_SPEED];
             }
         }
-        int r = build_tiles(b, k, bs.tile);
-        if (r) return r;
-        b->shape[k] = bs;
-        if (k == gks::BK_SPEED) {
-            cudaMemsetAsync(b->smax, 0, sizeof(unsigned long long) * b->nb, b->stream);
-            run_class(b, gks::BK_SPEED, 1);
-            gks::batch_dt(b->dd, b->nb, cfl, b->smax, b->dt, b->stream);
-        }
-        if (k == gks::BK_POLY) run_class(b, gks::BK_POLY, 1);
-        pos += snprintf(b->tuning + pos, sizeof(b->tuning) - pos, ", \"%s\": {\"block\": %d, \"tile\": %ld, \"blocks\": %d, \"ms\": %.4f}",
-                        class_name(k), bs.block, bs.tile, bs.blocks, best);
+    }
+    int r = set_shape(b, gks::BK_SPEED, bs.block, bs.tile);
+    if (r) return r;
+    for (int k : classes_of(b)) {
+        const LaunchShape &sp = b->shape[k];
+        pos += snprintf(b->tuning + pos, sizeof(b->tuning) - pos, ", \"%s\": {\"block\": %d, \"tile\": %ld, \"blocks\": %d",
+                        class_name(k), sp.block, sp.tile, sp.blocks);
+        if (k == gks::BK_SPEED) pos += snprintf(b->tuning + pos, sizeof(b->tuning) - pos, ", \"ms\": %.4f", best);
+        pos += snprintf(b->tuning + pos, sizeof(b->tuning) - pos, "}");
     }
     snprintf(b->tuning + pos, sizeof(b->tuning) - pos, "}");
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "tuning");
-    /* tuning ran stage-1 kernels only; clear the status they may have set */
-    cudaMemset(b->status, 0, sizeof(int) * b->nb);
     b->tuned = 1;
     TuneEntry t;
     for (int k = 0; k < gks::BK_COUNT; ++k) t.shape[k] = b->shape[k];
@@ -437,8 +404,7 @@ int gks_batch_create(int nbatch, const int *nx, const int *ny, const double *hs,
     for (int g = 0; g < nbatch; ++g) {
         if (nx[g] < 1 || ny[g] < 1 || nx[g] > (1 << 20) || ny[g] > (1 << 20) || !(hs[g] > 0.0))
             return bfail(nullptr, GKS_ERR_ARG, "grid %d: invalid size or cell size", g);
-        /* the kernels decompose indices in 32-bit arithmetic; the flux's
-         * (face, Gauss point) index space is rounded up to 128-item groups */
+        /* the kernels decompose indices in 32-bit arithmetic */
         const long ext = (long)(nx[g] + 2) * (ny[g] + 2);
         const long gx = ((long)(nx[g] + 1) * ny[g] * 2 + 127) / 128 * 128;
         const long gy = ((long)nx[g] * (ny[g] + 1) * 2 + 127) / 128 * 128;
@@ -468,16 +434,17 @@ int gks_batch_create(int nbatch, const int *nx, const int *ny, const double *hs,
     const size_t rs = o.precision ? sizeof(float) : sizeof(double);
     b->hd.resize(nbatch);
     b->g_stale.assign(nbatch, 0);
-    size_t off = al(sizeof(double) * nbatch) + al(sizeof(unsigned long long) * nbatch) + al(sizeof(int) * 8) +
-                 al(sizeof(int) * nbatch);
+    size_t off = al(sizeof(double) * 2 * nbatch) + al(sizeof(unsigned long long) * nbatch) +
+                 al(sizeof(float) * 10 * nbatch) + al(sizeof(int) * nbatch);
     std::vector<size_t> base(nbatch);
     for (int g = 0; g < nbatch; ++g) {
         make_kp(b->hd[g].P, nx[g], ny[g], hs[g], gamma, (int)bc, o);
         const gks::KP &P = b->hd[g].P;
         base[g] = off;
-        off += al(sizeof(double) * 4 * P.ncell) * 3 + al(sizeof(double) * 8 * P.ncell) * 2 + al(rs * 4 * GENO_NC2 * P.next) +
-               al(rs * 3 * 4 * 2 * P.nftot);
+        off += al(sizeof(double) * 4 * P.ncell) * 2 + al(sizeof(double) * 8 * P.ncell) +
+               al(rs * gks::group_elems(P.next, gks::kCellFields<2>)) + al(rs * gks::group_elems(P.nftot, gks::kFaceFields<2>));
         if (o.precision == 1) off += 2 * al(sizeof(float) * 16 * P.ncell); /* shadows: hi, lo, g */
+        else off += al(sizeof(double) * 4 * P.ncell) + al(sizeof(double) * 8 * P.ncell); /* Ws, Gs */
     }
     b->ws_bytes = off;
     e = cudaMalloc(&b->ws, off);
@@ -489,25 +456,27 @@ int gks_batch_create(int nbatch, const int *nx, const int *ny, const double *hs,
     }
     char *w = (char *)b->ws;
     b->dt = (double *)w;
-    b->smax = (unsigned long long *)(w + al(sizeof(double) * nbatch));
-    b->queue = (int *)(w + al(sizeof(double) * nbatch) + al(sizeof(unsigned long long) * nbatch));
-    b->status = (int *)((char *)b->queue + al(sizeof(int) * 8));
+    b->smax = (unsigned long long *)(w + al(sizeof(double) * 2 * nbatch));
+    b->updc = (float *)((char *)b->smax + al(sizeof(unsigned long long) * nbatch));
+    b->status = (int *)((char *)b->updc + al(sizeof(float) * 10 * nbatch));
     for (int g = 0; g < nbatch; ++g) {
         GridDesc &D = b->hd[g];
         const gks::KP &P = D.P;
         size_t o2 = base[g];
         D.W = (double *)(w + o2); o2 += al(sizeof(double) * 4 * P.ncell);
-        D.Ws = (double *)(w + o2); o2 += al(sizeof(double) * 4 * P.ncell);
         D.Acc = (double *)(w + o2); o2 += al(sizeof(double) * 4 * P.ncell);
         D.G = (double *)(w + o2); o2 += al(sizeof(double) * 8 * P.ncell);
-        D.Gs = (double *)(w + o2); o2 += al(sizeof(double) * 8 * P.ncell);
-        D.B = w + o2; o2 += al(rs * 4 * GENO_NC2 * P.next);
-        D.ff = w + o2; o2 += al(rs * 3 * 4 * 2 * P.nftot);
+        D.B = w + o2; o2 += al(rs * gks::group_elems(P.next, gks::kCellFields<2>));
+        D.ff = w + o2; o2 += al(rs * gks::group_elems(P.nftot, gks::kFaceFields<2>));
+        D.Ws = D.Gs = nullptr;
         D.s0 = D.s1 = gks::Shadow{nullptr, nullptr, nullptr};
         if (o.precision == 1) {
             float *a = (float *)(w + o2), *c2 = (float *)(w + o2 + al(sizeof(float) * 16 * P.ncell));
             D.s0 = gks::Shadow{a, a + 4 * P.ncell, a + 8 * P.ncell};
             D.s1 = gks::Shadow{c2, c2 + 4 * P.ncell, c2 + 8 * P.ncell};
+        } else {
+            D.Ws = (double *)(w + o2); o2 += al(sizeof(double) * 4 * P.ncell);
+            D.Gs = (double *)(w + o2);
         }
     }
     e = cudaMalloc(&b->dd, sizeof(GridDesc) * nbatch);
@@ -519,10 +488,7 @@ int gks_batch_create(int nbatch, const int *nx, const int *ny, const double *hs,
         return r;
     }
     for (int k : classes_of(b)) {
-        const int block = (k == gks::BK_STAGE) ? gks::kStageThreads : 128;
-        const int occ = gks::batch_occupancy(k, b->precision, block);
-        b->shape[k] = LaunchShape{block, k == gks::BK_STAGE ? 32 : 4096, b->nsm * (occ > 0 ? occ : 1)};
-        int r = build_tiles(b, k, b->shape[k].tile);
+        int r = set_shape(b, k, 128, 4096);
         if (r) {
             std::memcpy(g_batch_err, b->err, sizeof(g_batch_err));
             gks_batch_destroy(b);
@@ -586,7 +552,7 @@ int gks_batch_run(gks_batch_t b, double cfl, int nsteps)
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_in, 0);
     if (e != cudaSuccess) return bcuda(b, e, "stream ordering");
     if (!b->tuned) {
-        int r = tune(b, cfl);
+        int r = tune(b);
         if (r) return r;
     }
     if (!b->exec || b->graph_cfl != cfl) {

@@ -1,8 +1,16 @@
-/* Persistent batched kernels of the 2D compact GKS: every block walks the tile
- * list (grid-stride over tiles), every thread walks the items of its tile.
- * The per-item arithmetic is the single-grid kernels' (kernels.cuh). */
+/* Batched kernels of the 2D compact GKS over tile lists spanning every grid:
+ * a block of a stage kernel takes one tile, a thread one item.  The per-item
+ * arithmetic is the single-grid step path's (kernels.cuh,
+ * step_flux.cuh), so a grid of a batch and the same grid alone run the same
+ * formulas.  Mixed precision ran each stage as one fused kernel sweeping
+ * strips through shared memory before the face flux took a thread per face;
+ * with that flux in both, 2 steps of 1.8 M cells in 12 grids, states copied in
+ * and out, take 2.96 ms against the sweep's 3.63 ms (registers and the
+ * sweep's barriers held it at 16 warps per SM); the FP64 batch of 6 grids 4.67
+ * ms against 5.54 ms with its tile loops over the per-point flux.
+ */
 #include "batch.h"
-#include "fused2d.cuh"
+#include "step_flux.cuh"
 
 namespace gks {
 
@@ -19,19 +27,21 @@ template <> __device__ __forceinline__ Src<float> stage_src_of<float>(const Grid
 
 template <typename R>
 __global__ void __launch_bounds__(256) bk_speed(const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles, int ntiles,
-                                                unsigned long long *__restrict__ smax)
+                                                long tile, unsigned long long *__restrict__ smax)
 {
     __shared__ double red[8];
     for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
         const Tile T = tiles[ti];
-        const KP &P = gd[T.grid].P;
+        const unsigned grid = T.grid_kind >> 1;
+        const KP &P = gd[grid].P;
+        const long end = T.begin + tile < P.ncell ? T.begin + tile : P.ncell;
         /* the FP64 state, or its FP32 shadow in mixed precision */
         const R *W;
-        if constexpr (sizeof(R) == sizeof(float)) W = gd[T.grid].s0.hi;
-        else W = gd[T.grid].W;
+        if constexpr (sizeof(R) == sizeof(float)) W = gd[grid].s0.hi;
+        else W = gd[grid].W;
         const R gam = R(P.gamma);
         R sr = R(0);
-        for (long c = T.begin + threadIdx.x; c < T.end; c += blockDim.x) {
+        for (long c = T.begin + threadIdx.x; c < end; c += blockDim.x) {
             const R rho = W[c];
             const R u = W[P.ncell + c] / rho, v = W[2 * P.ncell + c] / rho;
             const R p = (gam - R(1)) * (W[3 * P.ncell + c] - R(0.5) * rho * (u * u + v * v));
@@ -45,167 +55,129 @@ __global__ void __launch_bounds__(256) bk_speed(const GridDesc *__restrict__ gd,
         if (threadIdx.x == 0) {
             double m = 0.0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, red[w]);
-            atomicMax(&smax[T.grid], (unsigned long long)__double_as_longlong(isnan(m) ? 1e300 : m));
+            atomicMax(&smax[grid], (unsigned long long)__double_as_longlong(isnan(m) ? 1e300 : m));
         }
         __syncthreads();
     }
 }
 
 __global__ void bk_dt(const GridDesc *__restrict__ gd, int nb, double cfl, const unsigned long long *__restrict__ smax,
-                      double *__restrict__ dt)
+                      double *__restrict__ dt, float *__restrict__ updc)
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nb) dt[b] = cfl * gd[b].P.h / __longlong_as_double((long long)smax[b]);
+    if (b >= nb) return;
+    const KP &P = gd[b].P;
+    const double d = cfl * P.h / __longlong_as_double((long long)smax[b]);
+    dt[2 * b] = d;
+    dt[2 * b + 1] = 1.0 / d;
+    if (updc) store_updc(updc + 10 * b, make_updc(d, updc_cw(P, 2)));
 }
 
+/* The parameter block of one grid: the scheme constants and boundary types,
+ * which the grids of a batch share, from the launch parameter (constant
+ * bank), the geometry from the grid's descriptor. */
+__device__ __forceinline__ KP grid_kp(const KP &common, const KP &g)
+{
+    KP P = common;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        P.n[a] = g.n[a];
+        P.nface[a] = g.nface[a];
+        P.foff[a] = g.foff[a];
+        P.ext[a] = g.ext[a];
+        P.dn[a] = g.dn[a];
+        P.dface[a][0] = g.dface[a][0];
+        P.dface[a][1] = g.dface[a][1];
+    }
+    P.ncell = g.ncell;
+    P.nftot = g.nftot;
+    P.next = g.next;
+    P.h = g.h;
+    P.ih = g.ih;
+    P.fh = g.fh;
+    P.fih = g.fih;
+    P.dext[0] = g.dext[0];
+    P.dext[1] = g.dext[1];
+    return P;
+}
+
+/* One block per tile, one item per thread: no loop whose invariants (the
+ * grid's geometry, the addresses) would be held in registers across items. */
 template <typename R>
-__global__ void __launch_bounds__(128) bk_poly(const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles, int ntiles,
-                                               int stage)
+__global__ void __launch_bounds__(128) bk_poly(const KP common, const GridDesc *__restrict__ gd,
+                                               const Tile *__restrict__ tiles, int stage)
 {
-    for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
-        const Tile T = tiles[ti];
-        const GridDesc &g = gd[T.grid];
-        const Src<R> src = stage_src_of<R>(g, stage);
-        for (long t = T.begin + threadIdx.x; t < T.end; t += blockDim.x) cell_poly_item<R, 2>(g.P, src, (R *)g.B, t);
-    }
+    const Tile T = tiles[blockIdx.x];
+    const GridDesc &g = gd[T.grid_kind >> 1];
+    const KP P = grid_kp(common, g.P);
+    const unsigned t = T.begin + threadIdx.x;
+    if (t < P.next) cell_poly_item<R, 2, true>(P, stage_src_of<R>(g, stage), (R *)g.B, t);
 }
 
-/* same register cap as the single-grid 2D FP32 flux (8 blocks of 128 per SM) */
+/* block size and register cap of the single-grid face flux */
 template <typename R>
-__global__ void __launch_bounds__(128, (flux_blocks_per_sm<R, 2, false>())) bk_flux(const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles, int ntiles,
-                                               int stage, const double *__restrict__ dt, int *__restrict__ status)
+__global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, 2, false>))
+    bk_flux(const KP common, const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles,
+            const double *__restrict__ dt, int *__restrict__ status)
 {
-    for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
-        const Tile T = tiles[ti];
-        const GridDesc &g = gd[T.grid];
-        const Src<R> src = stage_src_of<R>(g, stage);
-        const double dtv = dt[T.grid];
-        /* FP32: per-face Gauss sums, as the single-grid step path (tiles are
-         * whole 128-item groups, so every thread runs the same iterations and
-         * t mod 128 is its thread index) */
-        constexpr bool fsum = sizeof(R) == sizeof(float);
-        if (T.kind == 0) {
-            for (long t = T.begin + threadIdx.x; t < T.end; t += blockDim.x)
-                face_flux_item<R, 2, 0, true, false, fsum>(g.P, src, (const R *)g.B, dtv, nullptr, (R *)g.ff, status + T.grid, t);
-        } else {
-            for (long t = T.begin + threadIdx.x; t < T.end; t += blockDim.x)
-                face_flux_item<R, 2, 1, true, false, fsum>(g.P, src, (const R *)g.B, dtv, nullptr, (R *)g.ff, status + T.grid, t);
-        }
+    __shared__ typename FaceV<R>::V slots[kFaceStash<R, 2> * kStepFluxBlock];
+    typename FaceV<R>::V *stash = slots + threadIdx.x;
+    const Tile T = tiles[blockIdx.x];
+    const unsigned grid = T.grid_kind >> 1;
+    const GridDesc &g = gd[grid];
+    const KP P = grid_kp(common, g.P);
+    const R d = R(dt[2 * grid]), id = R(dt[2 * grid + 1]);
+    const unsigned fl = T.begin + threadIdx.x;
+    if (T.grid_kind & 1u) {
+        if (fl < P.nface[1])
+            step_face_item<R, 2, 1, false, kStepFluxBlock>(P, (const R *)g.B, d, id, (R *)g.ff, status + grid, fl, stash);
+    } else {
+        if (fl < P.nface[0])
+            step_face_item<R, 2, 0, false, kStepFluxBlock>(P, (const R *)g.B, d, id, (R *)g.ff, status + grid, fl, stash);
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256) bk_update(const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles, int ntiles,
-                                                 int stage, const double *__restrict__ dt, int *__restrict__ status)
+template <typename R, int STAGE>
+__global__ void __launch_bounds__(128) bk_update(const KP common, const GridDesc *__restrict__ gd,
+                                                 const Tile *__restrict__ tiles, const double *__restrict__ dt,
+                                                 const float *__restrict__ updc, int *__restrict__ status)
 {
-    __shared__ UpdC uc;
-    for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
-        const Tile T = tiles[ti];
-        const GridDesc &g = gd[T.grid];
-        const double dtv = dt[T.grid];
-        if constexpr (sizeof(R) == sizeof(float)) {
-            /* the tile's grid's stage constants (the tile loop is uniform over the block) */
-            __syncthreads();
-            if (threadIdx.x == 0) uc = make_updc(dtv, g.P.ih / 2);
-            __syncthreads();
-        }
-        for (long c = T.begin + threadIdx.x; c < T.end; c += blockDim.x) {
-            if (stage == 1)
-                update_item<R, 2, 1>(g.P, (const R *)g.ff, dtv, g.W, g.G, g.Ws, g.Gs, g.Acc, g.s0, g.s1, status + T.grid, c, uc);
-            else
-                update_item<R, 2, 2>(g.P, (const R *)g.ff, dtv, g.W, g.G, g.Ws, g.Gs, g.Acc, g.s0, g.s1, status + T.grid, c, uc);
-        }
-    }
-}
-
-/* Mixed precision: one stage of every grid in one persistent launch.  Each
- * block takes the next strip of the list from a work counter (strips ordered
- * by size, largest first) and runs the fused reconstruction -> flux ->
- * update sweep (fused2d_strip) of it, until the list is done.  The grids
- * share every scheme constant and boundary type, so the kernel takes one
- * parameter block (its geometry fields unused) as a launch parameter, and
- * per strip only the grid's geometry, state pointers and time step. */
-constexpr int kStageMinBlocks = 4;
-
-template <int STAGE>
-__global__ void __launch_bounds__(kStageThreads, kStageMinBlocks)
-    bk_stage(const KP P, const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles, int ntiles,
-             const double *__restrict__ dt, int *__restrict__ queue, int *__restrict__ status)
-{
-    extern __shared__ __align__(16) float smem[];
-    __shared__ UpdC uc;
-    __shared__ int next;
-    for (;;) {
-        __syncthreads(); /* every thread has read `next`; the previous strip is done with uc and the rings */
-        if (threadIdx.x == 0) next = atomicAdd(queue, 1);
-        __syncthreads();
-        const int ti = next;
-        if (ti >= ntiles) break;
-        const Tile T = tiles[ti];
-        const GridDesc &g = gd[T.grid];
-        const FusedGeo geo{g.P.n[0], g.P.n[1], g.P.ncell, g.P.ih, g.P.fh, g.P.fih};
-        /* the shadows' lo and g planes follow hi at 4 and 8 planes of cells */
-        const long nc = geo.nc;
-        float *const h0 = g.s0.hi, *const h1 = g.s1.hi;
-        const Shadow s0{h0, h0 + 4 * nc, h0 + 8 * nc}, s1{h1, h1 + 4 * nc, h1 + 8 * nc};
-        fused2d_strip<STAGE, false, kStageStrip, kStageThreads>(P, geo, s0, s1, g.W, (float *)g.Acc, dt[T.grid],
-                                                               status + T.grid, T.kind, (int)T.begin, (int)(T.end - T.begin),
-                                                               smem, uc);
-    }
-}
-
-/* the dynamic shared memory opt-in of both stage kernels, once */
-cudaError_t stage_prepare()
-{
-    using Strip = SweepStrip<kStageStrip>;
-    static const cudaError_t prep = [] {
-        cudaError_t e = cudaFuncSetAttribute(bk_stage<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Strip::SMEM);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(bk_stage<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Strip::SMEM);
-        for (auto k : {bk_stage<1>, bk_stage<2>})
-            if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
-                (void)cudaGetLastError();
-        return e;
-    }();
-    return prep;
-}
-
-cudaError_t batch_stage(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
-{
-    using Strip = SweepStrip<kStageStrip>;
-    const cudaError_t prep = stage_prepare();
-    if (prep != cudaSuccess) return prep;
-    if (S.block != kStageThreads) return cudaErrorInvalidConfiguration;
-    if (L.ntiles < 1) return cudaSuccess;
-    int *q = L.queue + (stage - 1);
-    cudaError_t e = cudaMemsetAsync(q, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    if (stage == 1)
-        bk_stage<1><<<S.blocks, kStageThreads, Strip::SMEM, st>>>(*L.common, L.gd, L.tiles, L.ntiles, L.dt, q, L.status);
-    else
-        bk_stage<2><<<S.blocks, kStageThreads, Strip::SMEM, st>>>(*L.common, L.gd, L.tiles, L.ntiles, L.dt, q, L.status);
-    return cudaGetLastError();
+    const Tile T = tiles[blockIdx.x];
+    const unsigned grid = T.grid_kind >> 1;
+    const GridDesc &g = gd[grid];
+    const KP P = grid_kp(common, g.P);
+    UpdC uc;
+    if constexpr (sizeof(R) == sizeof(float)) uc = load_updc(updc + 10 * grid);
+    const unsigned c = T.begin + threadIdx.x;
+    if (c < P.ncell)
+        step_update_item<R, 2, STAGE>(P, (const R *)g.ff, dt[2 * grid], g.W, g.G, g.Ws, g.Gs, g.Acc, g.s0, g.s1,
+                                      status + grid, c, uc);
 }
 
 template <typename R> cudaError_t batch_speed(const BatchLaunch &L, const LaunchShape &S, cudaStream_t st)
 {
-    bk_speed<R><<<S.blocks, S.block, 0, st>>>(L.gd, L.tiles, L.ntiles, L.smax);
+    bk_speed<R><<<S.blocks, S.block, 0, st>>>(L.gd, L.tiles, L.ntiles, S.tile, L.smax);
     return cudaGetLastError();
 }
 template <typename R> cudaError_t batch_poly(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
 {
-    bk_poly<R><<<S.blocks, S.block, 0, st>>>(L.gd, L.tiles, L.ntiles, stage);
+    bk_poly<R><<<S.blocks, S.block, 0, st>>>(*L.common, L.gd, L.tiles, stage);
     return cudaGetLastError();
 }
 template <typename R> cudaError_t batch_flux(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
 {
-    if (S.block != 128) return cudaErrorInvalidConfiguration; /* the face mapping's group size */
-    bk_flux<R><<<S.blocks, S.block, 0, st>>>(L.gd, L.tiles, L.ntiles, stage, L.dt, L.status);
+    if (S.block != kStepFluxBlock) return cudaErrorInvalidConfiguration;
+    static const bool prep = (smem_carveout_for(bk_flux<R>, kStepFluxMinBlocks<R, 2, false>), true);
+    (void)prep;
+    bk_flux<R><<<S.blocks, S.block, 0, st>>>(*L.common, L.gd, L.tiles, L.dt, L.status);
     return cudaGetLastError();
 }
 template <typename R> cudaError_t batch_update(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
 {
-    bk_update<R><<<S.blocks, S.block, 0, st>>>(L.gd, L.tiles, L.ntiles, stage, L.dt, L.status);
+    if (stage == 1)
+        bk_update<R, 1><<<S.blocks, S.block, 0, st>>>(*L.common, L.gd, L.tiles, L.dt, L.updc, L.status);
+    else
+        bk_update<R, 2><<<S.blocks, S.block, 0, st>>>(*L.common, L.gd, L.tiles, L.dt, L.updc, L.status);
     return cudaGetLastError();
 }
 cudaError_t batch_shadow(const GridDesc &g, cudaStream_t st)
@@ -223,38 +195,19 @@ cudaError_t batch_widen_grad(const GridDesc &g, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t batch_dt(const GridDesc *gd, int nb, double cfl, const unsigned long long *smax, double *dt, cudaStream_t st)
+cudaError_t batch_dt(const GridDesc *gd, int nb, double cfl, const unsigned long long *smax, double *dt, float *updc,
+                     cudaStream_t st)
 {
-    bk_dt<<<(nb + 127) / 128, 128, 0, st>>>(gd, nb, cfl, smax, dt);
+    bk_dt<<<(nb + 127) / 128, 128, 0, st>>>(gd, nb, cfl, smax, dt, updc);
     return cudaGetLastError();
 }
 
-/* resident blocks per SM of one kernel class at a block size */
-int batch_occupancy(int kernel, int precision, int block)
+/* resident blocks per SM of the wave-speed kernel at a block size */
+int batch_occupancy(int precision, int block)
 {
     int n = 0;
-    switch (kernel) {
-    case BK_SPEED:
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, precision ? bk_speed<float> : bk_speed<double>, block, 0);
-        break;
-    case BK_POLY:
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bk_poly<double>, block, 0);
-        break;
-    case BK_FLUX:
-        smem_carveout_for(bk_flux<double>, flux_blocks_per_sm<double, 2, false>());
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bk_flux<double>, block, 0);
-        break;
-    case BK_STAGE:
-        /* the opt-in to the dynamic shared memory, then the occupancy with it */
-        if (stage_prepare() == cudaSuccess)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bk_stage<1>, kStageThreads, SweepStrip<kStageStrip>::SMEM);
-        else
-            (void)cudaGetLastError();
-        break;
-    default:
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bk_update<double>, block, 0);
-        break;
-    }
+    if (precision) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bk_speed<float>, block, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bk_speed<double>, block, 0);
     return n;
 }
 
@@ -263,7 +216,7 @@ int batch_occupancy(int kernel, int precision, int block)
     template cudaError_t batch_poly<R>(const BatchLaunch &, const LaunchShape &, int, cudaStream_t);   \
     template cudaError_t batch_flux<R>(const BatchLaunch &, const LaunchShape &, int, cudaStream_t);   \
     template cudaError_t batch_update<R>(const BatchLaunch &, const LaunchShape &, int, cudaStream_t);
-template cudaError_t batch_speed<float>(const BatchLaunch &, const LaunchShape &, cudaStream_t);
+GKS_BATCH_INST(float)
 GKS_BATCH_INST(double)
 
 } // namespace gks
