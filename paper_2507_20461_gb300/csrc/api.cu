@@ -8,6 +8,7 @@
 #include <new>
 
 #include "internal.h"
+#include "step_1d.cuh"
 #include "step_flux.cuh"
 
 namespace {
@@ -150,7 +151,6 @@ cudaError_t run_shadow(gks_ctx *c)
 cudaError_t run_update(gks_ctx *c, int stage)
 {
     switch (c->dim) {
-    case 1: return gks::launch_update<1>(c, stage);
     case 2: return gks::launch_update<2>(c, stage);
     default: return gks::launch_update<3>(c, stage);
     }
@@ -165,15 +165,42 @@ cudaError_t run_wavespeed(gks_ctx *c, double cfl)
     }
 }
 
-/* both stages with the time step already in c->dt */
+/* a 1D step, its stages with the given clocks */
+int step_1d(gks_ctx *c, const gks::StepClock &first, const gks::StepClock &mid, const gks::StepClock &last)
+{
+    const cudaError_t e = c->order == 8 ? gks::launch_step1d(c, first, last) : gks::nc_launch_step(c, first, mid, last);
+    return e == cudaSuccess ? GKS_OK : cuda_fail(c, e, "1D step");
+}
+
+/* nsteps 1D CFL steps: the wave speed of the current state in slot 0, then
+ * every step reads its time step from one slot, clears the other in its first
+ * stage and leaves the new state's wave speed there in its last */
+int steps_1d_cfl(gks_ctx *c, double cfl, int nsteps)
+{
+    const double visc = c->kp.fp.mu > 0.0 ? 2.0 * c->kp.fp.mu / c->h : 0.0;
+    if (nsteps < 1) return GKS_OK;
+    cudaError_t e = run_wavespeed(c, 0.0);
+    if (e != cudaSuccess) return cuda_fail(c, e, "time step");
+    for (int s = 0; s < nsteps; ++s) {
+        unsigned long long *in = c->smax + 2 * (s & 1), *out = c->smax + 2 * (~s & 1);
+        const bool more = s + 1 < nsteps;
+        const gks::StepClock mid{nullptr, in, nullptr, nullptr, cfl * c->h, visc};
+        gks::StepClock first = mid, last = mid;
+        if (more) {
+            first.clear = out;
+            last.out = out;
+        }
+        const int r = step_1d(c, first, mid, last);
+        if (r) return r;
+    }
+    return GKS_OK;
+}
+
+/* both stages of a multi-D step with the time step already in c->dt */
 int two_stages(gks_ctx *c)
 {
     cudaError_t e;
     if (c->shadows) c->g_stale = 1;
-    if (c->dim == 1 && c->order != 8) {
-        if ((e = gks::nc_launch_step(c)) != cudaSuccess) return cuda_fail(c, e, "RK4 step");
-        return GKS_OK;
-    }
     if ((e = run_flux(c, 0, true)) != cudaSuccess) return cuda_fail(c, e, "stage 1 flux");
     if ((e = run_update(c, 1)) != cudaSuccess) return cuda_fail(c, e, "stage 1 update");
     if ((e = run_flux(c, 1, true)) != cudaSuccess) return cuda_fail(c, e, "stage 2 flux");
@@ -476,6 +503,10 @@ int gks_step(gks_handle_t c, double dt)
     gks::set_dt_kernel<<<1, 1, 0, c->stream>>>(c->dt, dt, c->shadows ? c->updc : nullptr, gks::updc_cw(c->kp, c->dim));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "set dt");
+    if (c->dim == 1) {
+        const gks::StepClock k{c->dt, nullptr, nullptr, nullptr, 0.0, 0.0};
+        return step_1d(c, k, k, k);
+    }
     return two_stages(c);
 }
 
@@ -483,6 +514,7 @@ int gks_step_cfl(gks_handle_t c, double cfl, int nsteps)
 {
     if (!c) return fail(nullptr, GKS_ERR_ARG, "NULL handle");
     if (!(cfl > 0.0) || !std::isfinite(cfl) || nsteps < 0) return fail(c, GKS_ERR_ARG, "cfl > 0 and nsteps >= 0 required");
+    if (c->dim == 1) return steps_1d_cfl(c, cfl, nsteps);
     for (int s = 0; s < nsteps; ++s) {
         cudaError_t e = run_wavespeed(c, cfl);
         if (e != cudaSuccess) return cuda_fail(c, e, "time step");

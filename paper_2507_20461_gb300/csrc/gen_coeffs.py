@@ -165,8 +165,9 @@ def gen_noncompact(lines):
     {j-1,j,j+1}, {j,j+1,j+2} (the 5th-order WENO stencils);
     order 6: p^5 on {j-2..j+3}, quadratics on {j-2,j-1,j}, {j-1,j,j+1},
     cubics on {j-1..j+2}, {j..j+3}.  Inputs u[i] = average at offset i - 2
-    (minus any constant: every polynomial reproduces constants); the right
-    value is the same map applied to the mirrored stencil."""
+    minus the cell's own (every polynomial reproduces constants), so u[2] = 0
+    drops out of every expression; the right value is the same map applied to
+    the mirrored stencil."""
     for order, big, subs in (
         (5, list(range(-2, 3)), [((-2, -1, 0), 2), ((-1, 0, 1), 2), ((0, 1, 2), 2)]),
         (6, list(range(-2, 4)), [((-2, -1, 0), 2), ((-1, 0, 1), 2), ((-1, 0, 1, 2), 3), ((0, 1, 2, 3), 3)]),
@@ -186,11 +187,12 @@ def gen_noncompact(lines):
         lines.append(f"/* {order}th-order non-compact GENO (Sec. 4.1): left value at x_(j+1/2) of the")
         lines.append(f" * high-order polynomial (qH) and of the {len(subs)} sub-stencil polynomials (p), and")
         lines.append(" * the sub-stencils' Jiang-Shu indicators sum_l int (d^l p)^2 (IS), from the")
-        lines.append(" * averages u[i] at offsets i - 2 (cell units). */")
+        lines.append(" * averages u[i] at offsets i - 2 relative to the cell's (u[2] = 0, not read). */")
         lines.append("template <typename R>")
         lines.append(f"__host__ __device__ __forceinline__ void nc{order}_left(const R *__restrict__ u, R &qH, R *__restrict__ p, R *__restrict__ IS)")
         lines.append("{")
-        emit_assignments(lines, [sp.expand(e).xreplace(usyms) for e in exprs], names)
+        own = sp.Symbol("u2")
+        emit_assignments(lines, [sp.expand(sp.expand(e).subs(own, 0)).xreplace(usyms) for e in exprs], names)
         lines.append("}")
         lines.append("")
 

@@ -98,7 +98,10 @@ template <int M> cudaError_t launch_shadow(gks_ctx *c);
 /* 1D non-compact schemes (order 5 or 6): face states / HLLC fluxes of the
  * stage input (input 0: W, 1: Ws), and one classical RK4 step */
 cudaError_t nc_launch_faces(gks_ctx *c, int input, double *fs_dev, bool flux);
-cudaError_t nc_launch_step(gks_ctx *c);
+struct StepClock;
+cudaError_t nc_launch_step(gks_ctx *c, const StepClock &first, const StepClock &mid, const StepClock &last);
+/* one compact 1D step: its two stages with the clock of each */
+cudaError_t launch_step1d(gks_ctx *c, const StepClock &first, const StepClock &last);
 
 inline int ngauss(int m) { return m == 1 ? 1 : (m == 2 ? 2 : 4); }
 inline int ncubic(int m) { return m == 2 ? GENO_NC2 : (m == 3 ? GENO_NC3 : 0); }

@@ -20,6 +20,7 @@
  * extension with the normal derivative negated); no padded copies exist.
  */
 #pragma once
+#include <cmath>
 #include <cstdint>
 
 #include "fpsplit.cuh"
@@ -77,6 +78,9 @@ struct KP {
     FluxParams fp;
     /* FP32 copies for the mixed-precision kernels (fill with finalize_kp) */
     float fh, fih, fgm1, fC, fitanhC, feps, fC0, fadm, fd0, fct;
+    /* chi_is_one's thresholds, r = 2 and 3 (fill with finalize_kp) */
+    double chi1[2];
+    float fchi1[2];
     /* index decompositions (fill with finalize_kp; every index space of a
      * launch is below 2^32): cells per axis, extended box, per face
      * direction its two leading extents and its face count */
@@ -102,6 +106,11 @@ inline void finalize_kp(KP &P)
     P.fC0 = (float)P.C0;
     P.fd0 = (float)P.d0;
     P.fct = (float)P.ct;
+    const double e = 2.0 * P.C / 19.1 - 2.0, fe = 2.0 * P.C / 9.1 - 2.0;
+    P.chi1[0] = (e > 0.0 && P.itanhC == 1.0) ? std::sqrt(e) : -1.0;
+    P.chi1[1] = (e > 0.0 && P.itanhC == 1.0) ? std::cbrt(e) : -1.0;
+    P.fchi1[0] = (fe > 0.0 && P.fitanhC == 1.f) ? (float)std::sqrt(fe) : -1.f;
+    P.fchi1[1] = (fe > 0.0 && P.fitanhC == 1.f) ? (float)std::cbrt(fe) : -1.f;
     for (int a = 0; a < 3; ++a) P.dn[a] = make_fdiv((unsigned)P.n[a]);
     P.dext[0] = make_fdiv((unsigned)P.ext[0]);
     P.dext[1] = make_fdiv((unsigned)P.ext[1]);
@@ -239,6 +248,23 @@ __device__ __forceinline__ R chi_of(const KP &P, R ISt, R ISH, R ISL, int r)
     return RT<R>::tanh_(pick<R>(P.C, P.fC) * alpha) * pick<R>(P.itanhC, P.fitanhC);
 }
 
+/* Whether the path function is surely 1 to the last bit, from IS^tau and IS^L
+ * alone: tanh(x) rounds to 1 for x > 19.06 in FP64 and 9.01 in FP32 (2 exp(-2 x)
+ * below half an ulp), and alpha >= 2 / (2 + (IS^tau / IS^L)^r), so C alpha >= T holds
+ * if IS^tau <= chi1 IS^L, chi1 = (2 C / T - 2)^(1/r) (T = 19.1, 9.1; set by
+ * finalize_kp, -1 where tanh(C) itself is below 1).  That is where the data are
+ * resolved: there the low-order combination has weight 0, and the
+ * reconstructions skip IS^H, the path function and the weights (FP64: about
+ * 300 of the 400 FP64 instructions of a variable and 2D cell).
+ * GB300, a pass: noncompact 6th order 10^6 cells 10.6 to 4.5 ms, FP64 512^2
+ * reconstruction 0.55 to 0.29 ms a stage, mixed 2048^2 0.219 to
+ * 0.196 ms (a warp with one unresolved cell, as at every shock front, still takes
+ * the whole path). */
+template <typename R> __device__ __forceinline__ bool chi_is_one(const KP &P, R ISt, R ISL, int r)
+{
+    return ISt <= pick<R>(P.chi1[r - 2], P.fchi1[r - 2]) * (ISL + pick<R>(P.eps, P.feps));
+}
+
 /* WENO-Z (limiter 2, Eq. wgt-WENO-Z) or TENO (limiter 3, Eq. wgt-TENO-1 with
  * the exponent 7 and Eq. wgt-TENO-2) weights over K + 1 candidates: 0 is
  * the high-order polynomial (indicator IS^H), 1..K the sub-stencil
@@ -282,7 +308,7 @@ __device__ __forceinline__ void ao_weights(const KP &P, const R *d, const R *IS,
 }
 
 template <typename R, int M>
-__device__ __forceinline__ bool admissible(const R *w, const R *wc, R gm1, R delta)
+__device__ __forceinline__ bool admissible(const R *w, const R *wc, R, R delta)
 {
     R ke = R(0), kc = R(0);
 #pragma unroll
@@ -290,10 +316,12 @@ __device__ __forceinline__ bool admissible(const R *w, const R *wc, R gm1, R del
         ke += w[1 + a] * w[1 + a];
         kc += wc[1 + a] * wc[1 + a];
     }
-    if (!(w[0] > delta * wc[0])) return false;
-    const R p = gm1 * (w[M + 1] - R(0.5) * ke / w[0]);
-    const R pc = gm1 * (wc[M + 1] - R(0.5) * kc / wc[0]);
-    return p > delta * pc;
+    /* p > delta p_c without divisions: rho p / (gamma - 1) = q, so
+     * q rho_c > delta q_c rho (reversed where rho_c < 0; a rho <= 0 fails in the
+     * flux either way) */
+    const R q = w[0] * w[M + 1] - R(0.5) * ke, qc = wc[0] * wc[M + 1] - R(0.5) * kc;
+    const R t = q * wc[0] - delta * qc * w[0];
+    return w[0] > delta * wc[0] && (wc[0] >= R(0) ? t > R(0) : t < R(0));
 }
 
 /* ------------------------------------------------------------------ */
@@ -310,9 +338,14 @@ __device__ __forceinline__ void geno1d_blend(const KP &P, const R (*a)[2], const
     R IS[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) IS[k] = a[k][0] * a[k][0] + R(13.0 / 3.0) * a[k][1] * a[k][1];
-    const R ISH = fmax(IS[0], fmax(IS[1], IS[2]));
     const R ISL = fmin(IS[0], fmin(IS[1], IS[2]));
     const R ISt = RT<R>::abs_(R(0.5) * (IS[1] + IS[2]) - IS[0]);
+    if (P.limiter == 1 || (P.limiter == 0 && chi_is_one<R>(P, ISt, ISL, 2))) {
+        val = qv;
+        der = qd;
+        return;
+    }
+    const R ISH = fmax(IS[0], fmax(IS[1], IS[2]));
     if (P.limiter >= 2) {
         /* WENO-Z / TENO in the adaptive-order combination:
          * (w0/d0) q^H + sum_k (w_k - (w0/d0) d_k) p_k, the sub-stencils sharing
@@ -334,7 +367,7 @@ __device__ __forceinline__ void geno1d_blend(const KP &P, const R (*a)[2], const
         }
         return;
     }
-    const R chi = P.limiter ? R(1) : chi_of<R>(P, ISt, ISH, ISL, 2);
+    const R chi = chi_of<R>(P, ISt, ISH, ISL, 2);
     const R eps = pick<R>(P.eps, P.feps);
     const R w0 = R(1) / ((IS[0] + eps) * (IS[0] + eps));
     const R w1 = pick<R>(P.C0, P.fC0) / ((IS[1] + eps) * (IS[1] + eps));
@@ -344,6 +377,25 @@ __device__ __forceinline__ void geno1d_blend(const KP &P, const R (*a)[2], const
     const R ld = (w0 * pd[0] + w1 * pd[1] + w2 * pd[2]) * iws;
     val = chi * qv + (R(1) - chi) * lv;
     der = chi * qd + (R(1) - chi) * ld;
+}
+
+/* the three sub-stencil quadratics of a left reconstruction from averages
+ * relative to the cell (offsets -1, 1, 2) and the averaged derivative at -1:
+ * coefficients a[k] = (a1, a2), values pv and derivatives pd at the right face */
+template <typename R>
+__device__ __forceinline__ void sub_quadratics(R wm1, R w1, R w2, R dm1, R (*a)[2], R *pv, R *pd)
+{
+    a[0][1] = -(wm1 + dm1);
+    a[0][0] = -R(2) * wm1 - dm1;
+    a[1][0] = R(0.5) * (w1 - wm1);
+    a[1][1] = R(0.5) * (w1 + wm1);
+    a[2][1] = R(0.5) * (w2 - R(2) * w1);
+    a[2][0] = R(0.5) * (R(4) * w1 - w2);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        pv[k] = R(0.5) * a[k][0] + a[k][1] * R(1.0 / 6.0);
+        pd[k] = a[k][0] + a[k][1];
+    }
 }
 
 /* states[side][v][c]: c = 0 value, 1 physical derivative */
@@ -371,19 +423,8 @@ __device__ __forceinline__ void recon1d_face(const KP &P, const double *__restri
         R qv, qd;
         p7_face<R>(wm1, R(0), w1, w2, R(d[0][v]), R(d[1][v]), R(d[2][v]), R(d[3][v]), qv, qd);
         {
-            const R dm1 = R(d[0][v]);
             R a[3][2], pv[3], pd[3];
-            a[0][1] = -(wm1 + dm1);
-            a[0][0] = -R(2) * wm1 - dm1;
-            a[1][0] = R(0.5) * (w1 - wm1);
-            a[1][1] = R(0.5) * (w1 + wm1);
-            a[2][1] = R(0.5) * (w2 - R(2) * w1);
-            a[2][0] = R(0.5) * (R(4) * w1 - w2);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                pv[k] = R(0.5) * a[k][0] + a[k][1] * R(1.0 / 6.0);
-                pd[k] = a[k][0] + a[k][1];
-            }
+            sub_quadratics<R>(wm1, w1, w2, R(d[0][v]), a, pv, pd);
             R val, der;
             geno1d_blend<R>(P, a, pv, pd, qv, qd, val, der);
             st[0][v][0] = R(w[1][v]) + val;
@@ -416,19 +457,15 @@ __device__ __forceinline__ void recon1d_face(const KP &P, const double *__restri
     }
 }
 
-/* FLUX = false: write the interface states face_states[side][v][c][face] (double).
- * FLUX = true : write ff[q][v][face] (R), q = F, dF/dt, W(dt/2). */
-template <typename R, bool FLUX, bool NS = false>
-__global__ void __launch_bounds__(128) face1d_kernel(KP P, const double *__restrict__ W, const double *__restrict__ G,
-                                                     const double *__restrict__ dtp, double *__restrict__ fs,
-                                                     R *__restrict__ ff, int *__restrict__ status)
+/* both interface states of face f (physical derivatives), after the
+ * admissibility fallback */
+template <typename R>
+__device__ __forceinline__ void states1d_face(const KP &P, const double *__restrict__ W, const double *__restrict__ G, int f,
+                                              R *Wl, R *Wr, R (*dWl)[3], R (*dWr)[3])
 {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f > P.n[0]) return;
     R st[2][3][2], cw[2][3];
     recon1d_face<R>(P, W, G, f, st, cw);
     const R gm1 = pick<R>(P.fp.gm1, P.fgm1);
-    R Wl[3], Wr[3], dWl[1][3], dWr[1][3];
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
         R s[3];
@@ -443,8 +480,37 @@ __global__ void __launch_bounds__(128) face1d_kernel(KP P, const double *__restr
             else { Wr[v] = val; dWr[0][v] = der; }
         }
     }
+}
+
+/* F, dF/dt, W(dt/2) of face f */
+template <typename R, bool NS>
+__device__ __forceinline__ void flux1d_face(const KP &P, const double *__restrict__ W, const double *__restrict__ G, int f,
+                                            R dt, int *__restrict__ status, R *F, R *Ft, R *Wh)
+{
+    R Wl[3], Wr[3], dWl[1][3], dWr[1][3];
+    states1d_face<R>(P, W, G, f, Wl, Wr, dWl, dWr);
+    if (!gks_point<R, 1, NS>(P.fp, dt, Wl, Wr, dWl, dWr, F, Ft, Wh)) {
+        atomicOr(status, ST_FLUX);
+#pragma unroll
+        for (int v = 0; v < 3; ++v) F[v] = Ft[v] = Wh[v] = R(0);
+    }
+    /* walls (slip or no-slip) are at rest and adiabatic: neither mass nor energy crosses them */
+    if ((f == 0 && P.bcs[0][0] >= 2) || (f == P.n[0] && P.bcs[0][1] >= 2)) F[0] = F[2] = Ft[0] = Ft[2] = R(0);
+}
+
+/* FLUX = false: write the interface states face_states[side][v][c][face] (double).
+ * FLUX = true : write ff[q][v][face] (R), q = F, dF/dt, W(dt/2). */
+template <typename R, bool FLUX, bool NS = false>
+__global__ void __launch_bounds__(32) face1d_kernel(KP P, const double *__restrict__ W, const double *__restrict__ G,
+                                                    const double *__restrict__ dtp, double *__restrict__ fs,
+                                                    R *__restrict__ ff, int *__restrict__ status)
+{
+    const int f = blockIdx.x * blockDim.x + threadIdx.x;
+    if (f > P.n[0]) return;
+    const long nf = P.nftot;
     if (!FLUX) {
-        const long nf = P.nftot;
+        R Wl[3], Wr[3], dWl[1][3], dWr[1][3];
+        states1d_face<R>(P, W, G, f, Wl, Wr, dWl, dWr);
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
             fs[((long)(0 * 3 + v) * 2 + 0) * nf + f] = (double)Wl[v];
@@ -455,15 +521,7 @@ __global__ void __launch_bounds__(128) face1d_kernel(KP P, const double *__restr
         return;
     }
     R F[3], Ft[3], Wh[3];
-    const R dt = R(dtp[0]);
-    if (!gks_point<R, 1, NS>(P.fp, dt, Wl, Wr, dWl, dWr, F, Ft, Wh)) {
-        atomicOr(status, ST_FLUX);
-#pragma unroll
-        for (int v = 0; v < 3; ++v) F[v] = Ft[v] = Wh[v] = R(0);
-    }
-    /* walls (slip or no-slip) are at rest and adiabatic: neither mass nor energy crosses them */
-    if ((f == 0 && P.bcs[0][0] >= 2) || (f == P.n[0] && P.bcs[0][1] >= 2)) F[0] = F[2] = Ft[0] = Ft[2] = R(0);
-    const long nf = P.nftot;
+    flux1d_face<R, NS>(P, W, G, f, R(dtp[0]), status, F, Ft, Wh);
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
         ff[(0 * 3 + v) * nf + f] = F[v];
@@ -480,11 +538,13 @@ template <typename R> struct Cubic<R, 2> {
     static constexpr int NC = GENO_NC2, ND = GENO_ND2;
     __device__ __forceinline__ static void fit(const R *d, R *c) { cubic2d_fit<R>(d, c); }
     __device__ __forceinline__ static void ind(const R *c, R &h, R &t) { cubic2d_indicators<R>(c, h, t); }
+    __device__ __forceinline__ static R tau(const R *c) { R h, t; cubic2d_indicators<R>(c, h, t); return t; }
 };
 template <typename R> struct Cubic<R, 3> {
     static constexpr int NC = GENO_NC3, ND = GENO_ND3;
     __device__ __forceinline__ static void fit(const R *d, R *c) { cubic3d_fit<R>(d, c); }
     __device__ __forceinline__ static void ind(const R *c, R &h, R &t) { cubic3d_indicators<R>(c, h, t); }
+    __device__ __forceinline__ static R tau(const R *c) { R h, t; cubic3d_indicators<R>(c, h, t); return t; }
 };
 
 /* thread -> extended cell (-1..n along every active axis); false for corner
@@ -519,8 +579,6 @@ __device__ __forceinline__ void blend_cubic(const KP &P, const R *d, R *b)
 #pragma unroll
     for (int a = 0; a < M; ++a) lin[a] = R(0);
     if (P.limiter != 1) {
-        R ISH, ISt;
-        Cubic<R, M>::ind(c, ISH, ISt);
         /* linear sub-polynomials on {cell, neighbour q}: g_e = (s dW + D_e)/2, g_t = D_t */
         R IS[2 * M], g[2 * M][M];
 #pragma unroll
@@ -536,6 +594,7 @@ __device__ __forceinline__ void blend_cubic(const KP &P, const R *d, R *b)
             }
             IS[q] = sum;
         }
+        const R ISt = Cubic<R, M>::tau(c);
         if (P.limiter == 0) {
             R smin = IS[0], smax = IS[0], ssum = R(0);
 #pragma unroll
@@ -545,25 +604,30 @@ __device__ __forceinline__ void blend_cubic(const KP &P, const R *d, R *b)
                 ssum += IS[q];
             }
             const R ISL = (ssum - smin - smax) * R(1.0 / (2 * M - 2));
-            chi = chi_of<R>(P, ISt, ISH, ISL, 3);
-            const R eps = pick<R>(P.eps, P.feps);
-            R ws = R(0);
+            if (!chi_is_one<R>(P, ISt, ISL, 3)) {
+                R ISH, It;
+                Cubic<R, M>::ind(c, ISH, It);
+                chi = chi_of<R>(P, ISt, ISH, ISL, 3);
+                const R eps = pick<R>(P.eps, P.feps);
+                R ws = R(0);
 #pragma unroll
-            for (int q = 0; q < 2 * M; ++q) {
-                const R wq = R(1) / ((IS[q] + eps) * (IS[q] + eps));
-                ws += wq;
+                for (int q = 0; q < 2 * M; ++q) {
+                    const R wq = R(1) / ((IS[q] + eps) * (IS[q] + eps));
+                    ws += wq;
 #pragma unroll
-                for (int a = 0; a < M; ++a) lin[a] += wq * g[q][a];
+                    for (int a = 0; a < M; ++a) lin[a] += wq * g[q][a];
+                }
+                const R iws = R(1) / ws;
+#pragma unroll
+                for (int a = 0; a < M; ++a) lin[a] = (R(1) - chi) * (lin[a] * iws);
             }
-            const R iws = R(1) / ws;
-#pragma unroll
-            for (int a = 0; a < M; ++a) lin[a] = (R(1) - chi) * (lin[a] * iws);
         } else {
             /* WENO-Z / TENO, adaptive-order combination: (w0/d0) p^3 +
              * sum_q (w_q - (w0/d0) d_q) p_q, the 2m linear polynomials
              * sharing 1 - d0 equally */
             const R d0 = pick<R>(P.d0, P.fd0), dq = (R(1) - d0) * R(1.0 / (2 * M));
-            R d[2 * M + 1], I[2 * M + 1], w[2 * M + 1];
+            R d[2 * M + 1], I[2 * M + 1], w[2 * M + 1], ISH, It;
+            Cubic<R, M>::ind(c, ISH, It);
             d[0] = d0;
             I[0] = ISH;
 #pragma unroll
@@ -1171,7 +1235,8 @@ __device__ __forceinline__ void mixed_update_cell(const KP &P, const FaceSum &fs
 }
 
 /* The FP64 stage update of one cell from the face sums over the Gauss points
- * (weight wg each), fsum(q, v, d, plus) as in mixed_update_var.
+ * (weight wg each), fsum(q, v, d, plus) as in mixed_update_var; Wn receives
+ * the new averages.
  * STAGE 1: Ws = W - dt/2 L(F) - dt^2/8 L(Ft), Gs = Gauss(W(dt/2)), Acc = -dt L(F) - dt^2/6 L(Ft)
  * STAGE 2: W += Acc - dt^2/3 L(Ft*),        G  = Gauss(W*(dt/2))
  * with L(q)_j = (1/h) sum_d sum_g w_g (q(+d face) - q(-d face)). */
@@ -1179,11 +1244,10 @@ template <int M, int STAGE, typename FaceSum>
 __device__ __forceinline__ void fp64_update_cell(const KP &P, const FaceSum &fsum, double wg, double dt,
                                                  double *__restrict__ W, double *__restrict__ G, double *__restrict__ Ws,
                                                  double *__restrict__ Gs, double *__restrict__ Acc,
-                                                 int *__restrict__ status, long cell)
+                                                 int *__restrict__ status, long cell, double *Wn)
 {
     constexpr int NV = M + 2;
     const double cw = wg * P.ih;
-    double Wn[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         double DF = 0.0, DFt = 0.0;
@@ -1262,21 +1326,8 @@ __device__ __forceinline__ void update_item(const KP &P, const R *__restrict__ f
         for (int g = 0; g < NG; ++g) a += (double)ff[((long)(q * NV + v) * NG + g) * nft + (plus ? fp[d] : fm[d])];
         return a;
     };
-    fp64_update_cell<M, STAGE>(P, fsum, 1.0 / NG, dt, W, G, Ws, Gs, Acc, status, cell);
-}
-
-template <typename R, int M, int STAGE>
-__global__ void __launch_bounds__(256) update_kernel(KP P, const R *__restrict__ ff, const double *__restrict__ dtp,
-                                                    double *__restrict__ W, double *__restrict__ G,
-                                                    double *__restrict__ Ws, double *__restrict__ Gs,
-                                                    double *__restrict__ Acc, Shadow s0, Shadow s1,
-                                                    int *__restrict__ status, const float *__restrict__ updc)
-{
-    /* the mixed-precision stage constants of this time step (FP64 path: unused) */
-    UpdC uc;
-    if constexpr (sizeof(R) == sizeof(float) && M >= 2) uc = load_updc(updc);
-    const long cell = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell < P.ncell) update_item<R, M, STAGE>(P, ff, dtp[0], W, G, Ws, Gs, Acc, s0, s1, status, cell, uc);
+    double Wn[NV];
+    fp64_update_cell<M, STAGE>(P, fsum, 1.0 / NG, dt, W, G, Ws, Gs, Acc, status, cell, Wn);
 }
 
 /* FP64 gradients from the FP32 shadow (mixed precision keeps the gradients
@@ -1307,23 +1358,48 @@ __global__ void shadow_kernel(KP P, const double *__restrict__ W, const double *
 /* ------------------------------------------------------------------ */
 /* max over cells of max_d |u_d| + c, read from the FP64 state (T = double)
  * or from its FP32 shadow (T = float) */
+/* max_d |u_d| + c of the averages w */
+template <int M, typename T> __device__ __forceinline__ T speed_of(const T *w, T gam)
+{
+    T ke = T(0), um = T(0);
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+        const T u = w[1 + a] / w[0];
+        ke += u * u;
+        um = fmax(um, fabs(u));
+    }
+    const T p = (gam - T(1)) * (w[M + 1] - T(0.5) * w[0] * ke);
+    return um + sqrt(gam * p / w[0]);
+}
+
+/* largest of the warp's speeds s and inverse densities ir into smax[0], smax[1]
+ * (non-negative doubles order like their bit patterns; a NaN becomes 1e300,
+ * which the host reports) */
+template <typename T> __device__ __forceinline__ void speed_max(T s, T ir, unsigned long long *__restrict__ smax)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
+        ir = fmax(ir, __shfl_xor_sync(0xffffffffu, ir, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        const double sd = (double)s, id = (double)ir;
+        atomicMax(smax, (unsigned long long)__double_as_longlong(isnan(sd) ? 1e300 : sd));
+        atomicMax(smax + 1, (unsigned long long)__double_as_longlong(isnan(id) ? 1e300 : id));
+    }
+}
+
 template <int M, typename T>
 __global__ void wavespeed_kernel(KP P, const T *__restrict__ W, unsigned long long *__restrict__ smax)
 {
     T s = T(0), ir = T(0); /* max |u_d| + c and max 1 / rho */
     const T gam = pick<T>(P.gamma, (float)(P.fgm1 + 1.0f));
     for (long c = (long)blockIdx.x * blockDim.x + threadIdx.x; c < P.ncell; c += (long)gridDim.x * blockDim.x) {
-        const T rho = W[c];
-        T ke = T(0), um = T(0);
+        T w[M + 2];
 #pragma unroll
-        for (int a = 0; a < M; ++a) {
-            const T u = W[(1 + a) * P.ncell + c] / rho;
-            ke += u * u;
-            um = fmax(um, fabs(u));
-        }
-        const T p = (gam - T(1)) * (W[(M + 1) * P.ncell + c] - T(0.5) * rho * ke);
-        s = fmax(s, um + sqrt(gam * p / rho));
-        ir = fmax(ir, T(1) / rho);
+        for (int v = 0; v < M + 2; ++v) w[v] = W[v * P.ncell + c];
+        s = fmax(s, speed_of<M, T>(w, gam));
+        ir = fmax(ir, T(1) / w[0]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1357,15 +1433,18 @@ __global__ void wavespeed_kernel(KP P, const T *__restrict__ W, unsigned long lo
 /* dt = cfl h / max(|u_d| + c), and with viscosity mu > 0 also at most
  * cfl h^2 / (2 (m - 1) nu_max), nu_max = mu max(1 / rho) (Sec. 6; the factor
  * 2 (m - 1) is taken as 2 in 1D) */
+__device__ __forceinline__ double dt_of_speed(const unsigned long long *smax, double cfl_h, double visc)
+{
+    const double dt = cfl_h / __longlong_as_double((long long)smax[0]);
+    if (!(visc > 0.0)) return dt;
+    const double nu = visc * __longlong_as_double((long long)smax[1]);
+    return fmin(dt, cfl_h / nu);
+}
+
 static __global__ void dt_from_speed_kernel(const unsigned long long *__restrict__ smax, double cfl_h, double visc,
                                             double *__restrict__ dtp, float *__restrict__ updc, double cw)
 {
-    const double s = __longlong_as_double((long long)smax[0]);
-    double dt = cfl_h / s;
-    if (visc > 0.0) {
-        const double nu = visc * __longlong_as_double((long long)smax[1]);
-        dt = fmin(dt, cfl_h / nu);
-    }
+    const double dt = dt_of_speed(smax, cfl_h, visc);
     dtp[0] = dt;
     dtp[1] = 1.0 / dt;
     if (updc) store_updc(updc, make_updc(dt, cw));

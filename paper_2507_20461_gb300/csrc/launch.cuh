@@ -27,11 +27,11 @@ template <typename R, int M> static cudaError_t flux_impl(gks_ctx *c, int input,
     const double *G = input ? c->Gs : c->G;
     if constexpr (M == 1) {
         if (c->order != 8) return nc_launch_faces(c, input, fs_dev, flux);
-        const unsigned nb = blocks_for(P.n[0] + 1);
+        const unsigned nb = blocks_for(P.n[0] + 1, 32);
         ProfScope ps(c, GKS_KC_FACE);
-        if (flux && P.fp.mu > 0.0) face1d_kernel<R, true, true><<<nb, kBlock, 0, c->stream>>>(P, W, G, c->dt, nullptr, ff, c->status);
-        else if (flux) face1d_kernel<R, true><<<nb, kBlock, 0, c->stream>>>(P, W, G, c->dt, nullptr, ff, c->status);
-        else face1d_kernel<R, false><<<nb, kBlock, 0, c->stream>>>(P, W, G, c->dt, fs_dev, nullptr, c->status);
+        if (flux && P.fp.mu > 0.0) face1d_kernel<R, true, true><<<nb, 32, 0, c->stream>>>(P, W, G, c->dt, nullptr, ff, c->status);
+        else if (flux) face1d_kernel<R, true><<<nb, 32, 0, c->stream>>>(P, W, G, c->dt, nullptr, ff, c->status);
+        else face1d_kernel<R, false><<<nb, 32, 0, c->stream>>>(P, W, G, c->dt, fs_dev, nullptr, c->status);
     } else {
         constexpr int NG = (M == 2) ? 2 : 4;
         R *B = (R *)c->B;
@@ -94,14 +94,8 @@ template <int M> cudaError_t launch_flux(gks_ctx *c, int input, bool sums)
 
 template <typename R, int M, int STAGE> static void update_launch(gks_ctx *c)
 {
-    const unsigned nb = blocks_for(c->kp.ncell, 256);
-    const R *ff = (const R *)c->ff;
-    if constexpr (M == 1)
-        update_kernel<R, M, STAGE><<<nb, 256, 0, c->stream>>>(c->kp, ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0,
-                                                              c->s1, c->status, c->updc);
-    else
-        step_update_kernel<R, M, STAGE><<<nb, 256, 0, c->stream>>>(c->kp, ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc,
-                                                                   c->s0, c->s1, c->status, c->updc);
+    step_update_kernel<R, M, STAGE><<<blocks_for(c->kp.ncell, 256), 256, 0, c->stream>>>(
+        c->kp, (const R *)c->ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1, c->status, c->updc);
 }
 
 template <typename R, int M> static cudaError_t update_impl(gks_ctx *c, int stage)
@@ -114,7 +108,8 @@ template <typename R, int M> static cudaError_t update_impl(gks_ctx *c, int stag
 
 template <int M> cudaError_t launch_update(gks_ctx *c, int stage)
 {
-    return c->precision ? update_impl<float, M>(c, stage) : update_impl<double, M>(c, stage);
+    if constexpr (M == 1) return cudaErrorInvalidValue; /* the 1D stages update in the kernel that evaluates the fluxes */
+    else return c->precision ? update_impl<float, M>(c, stage) : update_impl<double, M>(c, stage);
 }
 
 template <int M> cudaError_t launch_wavespeed(gks_ctx *c, double cfl)

@@ -372,8 +372,10 @@ __device__ __forceinline__ void step_update_item(const KP &P, const R *__restric
     auto fsum = [&](int q, int v, int d, int plus) -> R { return (plus ? fp[d] : fm[d])[(q * NV + v) * 32]; };
     if constexpr (sizeof(R) == sizeof(float))
         mixed_update_cell<M, STAGE>(P, fsum, uc, W, (float *)Acc, s0, s1, status, cell);
-    else
-        fp64_update_cell<M, STAGE>(P, fsum, 1.0 / (M == 2 ? 2 : 4), dt, W, G, Ws, Gs, Acc, status, cell);
+    else {
+        double Wn[NV];
+        fp64_update_cell<M, STAGE>(P, fsum, 1.0 / (M == 2 ? 2 : 4), dt, W, G, Ws, Gs, Acc, status, cell, Wn);
+    }
 }
 
 template <typename R, int M, int STAGE>
