@@ -248,9 +248,27 @@ def gen_md(lines, m):
     lines.append("template <typename R>")
     lines.append(f"__host__ __device__ __forceinline__ void cubic{m}d_fit(const R *__restrict__ d, R *__restrict__ c)")
     lines.append("{")
-    dsyms = {d[j]: sp.Symbol(f"d[{j}]") for j in range(nd)}
-    emit_linear(lines, [ce.xreplace(dsyms) for ce in c_exprs], [f"c[{k}]" for k in range(nc)],
-                [dsyms[d[j]] for j in range(nd)])
+    # the fit is symmetric: every coefficient depends on a pair of opposite
+    # neighbours through their sum or their difference only, which are formed
+    # once (2D 40 operations instead of 50, 3D 84 instead of 108)
+    pairs, subs = [], {}
+    for e in range(m):
+        lo, hi = 2 * e * (1 + m), (2 * e + 1) * (1 + m)
+        for k in range(1 + m):
+            S, D = sp.Symbol(f"s{lo + k}"), sp.Symbol(f"t{lo + k}")
+            pairs.append((S, D, lo + k, hi + k))
+            subs[d[lo + k]] = (S - D) / 2
+            subs[d[hi + k]] = (S + D) / 2
+    own = [sp.Symbol(f"d[{2 * m * (1 + m) + a}]") for a in range(m)]
+    subs.update({d[2 * m * (1 + m) + a]: own[a] for a in range(m)})
+    c_exprs = [sp.expand(ce.xreplace(subs)) for ce in c_exprs]
+    used = set().union(*(ce.free_symbols for ce in c_exprs))
+    for S, D, i, j in pairs:
+        if S in used:
+            lines.append(f"    const R {S} = d[{j}] + d[{i}];")
+        if D in used:
+            lines.append(f"    const R {D} = d[{j}] - d[{i}];")
+    emit_linear(lines, c_exprs, [f"c[{k}]" for k in range(nc)], [x for S, D, _, _ in pairs for x in (S, D)] + own)
     lines.append("}")
     lines.append("")
 

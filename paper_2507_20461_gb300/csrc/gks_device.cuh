@@ -48,38 +48,78 @@
 
 #include <type_traits>
 
+#include "erfc_table.cuh"
+#include "fpsplit.cuh"
 #include "lr2.cuh"
 
 namespace gks {
 
+/* The half-space moments take h = erfc(a) and e = exp(-a^2) of the same
+ * argument.
+ * FP64, |a| < 3 (Mach 3.5 normal to the face): degree-8 polynomials about the
+ * nearest k/32 from a 14 KB table (gen_erfc.py; truncation below 2^-55), 21 FP64
+ * instructions for both where the library's erfc and exp take about 71; the
+ * table's loads run beside the FP64 pipe, which bounds the kernel (2D 512^2 face
+ * flux 1.52 to 1.27 ms a stage).  The interval comes from an exact add of 1.5 2^47, whose unit is 1/32.  Above, the library.
+ * FP32: the library's erfc; e is the hardware exponential (__expf, about 2 + 1.2 x
+ * ulp, x = a^2; it multiplies terms that vanish as x grows).  A polynomial in
+ * 1 / (1 + |a|/2) times e, lanes together, raised the error of W(dt/2) by a third
+ * and is not taken. */
 template <typename R> struct RT;
 template <> struct RT<double> {
-    __device__ static double erfc_(double x) { return erfc(x); }
     __device__ static double exp_(double x) { return exp(x); }
     __device__ static double sqrt_(double x) { return sqrt(x); }
     __device__ static double rsqrt_(double x) { return rsqrt(x); }
     __device__ static double tanh_(double x) { return tanh(x); }
     __device__ static double abs_(double x) { return fabs(x); }
+    __device__ __forceinline__ static void erfc_exp(double a, double &h, double &e)
+    {
+        const uint64_t bits = fps::dbits(a);
+        const uint32_t hi = (uint32_t)(bits >> 32) & 0x7fffffffu;
+        const double x = fps::bitsd(bits & 0x7fffffffffffffffull);
+        if (hi < 0x40080000u) { /* |a| < 3 */
+            const double m = 211106232532992.0; /* 1.5 2^47 */
+            const double t = x + m, d = x - (t - m);
+            const double *row = erfc_rows[(uint32_t)fps::dbits(t) & 127u];
+            double p = row[ERFC_DEG], q = row[2 * ERFC_DEG + 1];
+#pragma unroll
+            for (int j = ERFC_DEG - 1; j >= 0; --j) {
+                p = p * d + row[j];
+                q = q * d + row[ERFC_DEG + 1 + j];
+            }
+            h = p;
+            e = q;
+        } else {
+            h = erfc(x);
+            e = exp(-x * x);
+        }
+        if (bits >> 63) h = 2.0 - h;
+    }
 };
-/* FP32: the exponentials of the flux (the half-space moments' exp(-lambda
- * U^2) and the relaxation factor) take the hardware exponential (__expf,
- * about 2 + 1.2 |x| ulp); both multiply terms that vanish as |x| grows, and
- * the 2048^2 mixed step is 1.3% shorter */
+/* FP32: the exponentials of the flux (erfc_exp and the relaxation factor) take
+ * the hardware exponential; the 2048^2 mixed step is 1.3% shorter */
 template <> struct RT<float> {
-    __device__ static float erfc_(float x) { return erfcf(x); }
     __device__ static float exp_(float x) { return __expf(x); }
     __device__ static float sqrt_(float x) { return sqrtf(x); }
     __device__ static float rsqrt_(float x) { return rsqrtf(x); }
     __device__ static float tanh_(float x) { return tanhf(x); }
     __device__ static float abs_(float x) { return fabsf(x); }
+    __device__ __forceinline__ static void erfc_exp(float a, float &h, float &e)
+    {
+        e = __expf(-a * a);
+        h = erfcf(a);
+    }
 };
 
 /* left/right pairs: the transcendentals per lane */
 template <> struct RT<LR> {
-    __device__ static LR erfc_(LR x) { return LR(erfcf(x.l()), erfcf(x.r())); }
-    __device__ static LR exp_(LR x) { return LR(__expf(x.l()), __expf(x.r())); }
-    __device__ static LR sqrt_(LR x) { return LR(sqrtf(x.l()), sqrtf(x.r())); }
     __device__ static LR rsqrt_(LR x) { return LR(rsqrtf(x.l()), rsqrtf(x.r())); }
+    __device__ __forceinline__ static void erfc_exp(LR a, LR &h, LR &e)
+    {
+        const LR x = LR(a * a);
+        e = LR(__expf(-x.l()), __expf(-x.r()));
+        h = LR(erfcf(a.l()), erfcf(a.r()));
+    }
 };
 
 /* x > 0 (every lane of a pair) */
@@ -140,8 +180,10 @@ __device__ __forceinline__ bool half_stream(const R *W, const R (*dW)[M + 2], R 
     R u[7];
     {
         const R x = R(0.70710678118654752) * y * U0;
-        u[0] = R(0.5) * W[0] * RT<R>::erfc_(-s * x);
-        u[1] = U0 * u[0] + s * (R(0.39894228040143268) * W[0] * th * y) * RT<R>::exp_(-x * x);
+        R h, e;
+        RT<R>::erfc_exp(-s * x, h, e);
+        u[0] = R(0.5) * W[0] * h;
+        u[1] = U0 * u[0] + s * (R(0.39894228040143268) * W[0] * th * y) * e;
 #pragma unroll
         for (int k = 0; k < 5; ++k) u[k + 2] = U0 * u[k + 1] + R(k + 1) * th * u[k];
     }
@@ -471,14 +513,21 @@ __device__ __forceinline__ bool flux_of_streams(const FluxParams &fp, R dt, R id
     F0[M + 1] = U[0] * (W0[M + 1] + p0);
 
     /* relaxation time over dt, kappa = tau_n / dt, and the time integrals */
-    R kap = pick<R>(fp.c1, fp.fc1) + pick<R>(fp.c2, fp.fc2) * RT<R>::abs_(pl - pr) / (pl + pr), tau = R(0);
-    if constexpr (NS) {
-        tau = pick<R>(fp.mu, fp.fmu) / p0;
-        kap += tau * idt;
-        tau *= ih;
+    R kap, eh = R(0), tau = R(0);
+    if constexpr (std::is_same_v<R, double> && !NS) {
+        /* kappa = y / S and 1 / (2 kappa) from one reciprocal of S y */
+        const double S = pl + pr, y = fp.c1 * S + fp.c2 * fabs(pl - pr), q = 1.0 / (S * y);
+        kap = y > 0.0 ? y * y * q : 0.0;
+        if (y > 0.0) eh = exp(-0.5 * S * S * q);
+    } else {
+        kap = pick<R>(fp.c1, fp.fc1) + pick<R>(fp.c2, fp.fc2) * RT<R>::abs_(pl - pr) / (pl + pr);
+        if constexpr (NS) {
+            tau = pick<R>(fp.mu, fp.fmu) / p0;
+            kap += tau * idt;
+            tau *= ih;
+        }
+        if (kap > R(0)) eh = RT<R>::exp_(R(-0.5) / kap);
     }
-    R eh = R(0);
-    if (kap > R(0)) eh = RT<R>::exp_(R(-0.5) / kap);
     const R e1 = eh * eh; /* exp(-dt/tn) */
     const R ie_h = kap * (R(1) - eh), ie_1 = kap * (R(1) - e1);
     const R ite_h = kap * (kap - (R(0.5) + kap) * eh), ite_1 = kap * (kap - (R(1) + kap) * e1);
