@@ -721,7 +721,7 @@ def main():
         if ex:
             r["executed_flops_per_unit"] = ex
             r["frac_executed"] = r["frac"] * ex / FACE_GP_2D
-    launches_per_step = 1 + 1 + 2 * (1 + 1 + 1)  # wavespeed, dt, 2 x (poly, face flux, update)
+    launches = 1 + args.steps * (1 + 2 * (1 + 1 + 1))  # wave speed once, then per step dt, 2 x (poly, face flux, update)
     value = ws * N * N / (ms_mixed * 1e-3)
     value64 = ws * N * N / (ms_fp64 * 1e-3)
     hbm_frac = BYTES_PER_CELL_UPDATE * value / ws / (peaks.get("hbm_gbs", 6800.0) * 1e9)
@@ -766,7 +766,7 @@ def main():
                       ((B.KC_RECON, "cell_poly"), (B.KC_FACE, "face_flux"), (B.KC_UPDATE, "update"), (B.KC_DT, "dt"))},
         "status": {"mixed": st_mixed, "fp64": st_fp64, "error_run": st_l1},
         "e2e": {"value": ws * e2e_val, "unit": "cell-updates/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-        "gpu_launches": launches_per_step * args.steps,
+        "gpu_launches": launches,
         "batched_256_grids": batch,
         "three_d_256": three_d,
         "navier_stokes_tgv_256": tgv,

@@ -148,20 +148,28 @@ cudaError_t run_shadow(gks_ctx *c)
     }
 }
 
-cudaError_t run_update(gks_ctx *c, int stage)
+cudaError_t run_update(gks_ctx *c, int stage, unsigned long long *smax)
 {
     switch (c->dim) {
-    case 2: return gks::launch_update<2>(c, stage);
-    default: return gks::launch_update<3>(c, stage);
+    case 2: return gks::launch_update<2>(c, stage, smax);
+    default: return gks::launch_update<3>(c, stage, smax);
     }
 }
 
-cudaError_t run_wavespeed(gks_ctx *c, double cfl)
+cudaError_t run_wavespeed(gks_ctx *c)
 {
     switch (c->dim) {
-    case 1: return gks::launch_wavespeed<1>(c, cfl);
-    case 2: return gks::launch_wavespeed<2>(c, cfl);
-    default: return gks::launch_wavespeed<3>(c, cfl);
+    case 1: return gks::launch_wavespeed<1>(c);
+    case 2: return gks::launch_wavespeed<2>(c);
+    default: return gks::launch_wavespeed<3>(c);
+    }
+}
+
+cudaError_t run_dt(gks_ctx *c, double cfl, const unsigned long long *in, unsigned long long *clear)
+{
+    switch (c->dim) {
+    case 2: return gks::launch_dt<2>(c, cfl, in, clear);
+    default: return gks::launch_dt<3>(c, cfl, in, clear);
     }
 }
 
@@ -179,7 +187,7 @@ int steps_1d_cfl(gks_ctx *c, double cfl, int nsteps)
 {
     const double visc = c->kp.fp.mu > 0.0 ? 2.0 * c->kp.fp.mu / c->h : 0.0;
     if (nsteps < 1) return GKS_OK;
-    cudaError_t e = run_wavespeed(c, 0.0);
+    cudaError_t e = run_wavespeed(c);
     if (e != cudaSuccess) return cuda_fail(c, e, "time step");
     for (int s = 0; s < nsteps; ++s) {
         unsigned long long *in = c->smax + 2 * (s & 1), *out = c->smax + 2 * (~s & 1);
@@ -196,15 +204,16 @@ int steps_1d_cfl(gks_ctx *c, double cfl, int nsteps)
     return GKS_OK;
 }
 
-/* both stages of a multi-D step with the time step already in c->dt */
-int two_stages(gks_ctx *c)
+/* both stages of a multi-D step with the time step already in c->dt; smax: where
+ * the new state's wave speed goes, or nullptr */
+int two_stages(gks_ctx *c, unsigned long long *smax)
 {
     cudaError_t e;
     if (c->shadows) c->g_stale = 1;
     if ((e = run_flux(c, 0, true)) != cudaSuccess) return cuda_fail(c, e, "stage 1 flux");
-    if ((e = run_update(c, 1)) != cudaSuccess) return cuda_fail(c, e, "stage 1 update");
+    if ((e = run_update(c, 1, nullptr)) != cudaSuccess) return cuda_fail(c, e, "stage 1 update");
     if ((e = run_flux(c, 1, true)) != cudaSuccess) return cuda_fail(c, e, "stage 2 flux");
-    if ((e = run_update(c, 2)) != cudaSuccess) return cuda_fail(c, e, "stage 2 update");
+    if ((e = run_update(c, 2, smax)) != cudaSuccess) return cuda_fail(c, e, "stage 2 update");
     return GKS_OK;
 }
 
@@ -507,7 +516,7 @@ int gks_step(gks_handle_t c, double dt)
         const gks::StepClock k{c->dt, nullptr, nullptr, nullptr, 0.0, 0.0};
         return step_1d(c, k, k, k);
     }
-    return two_stages(c);
+    return two_stages(c, nullptr);
 }
 
 int gks_step_cfl(gks_handle_t c, double cfl, int nsteps)
@@ -515,10 +524,17 @@ int gks_step_cfl(gks_handle_t c, double cfl, int nsteps)
     if (!c) return fail(nullptr, GKS_ERR_ARG, "NULL handle");
     if (!(cfl > 0.0) || !std::isfinite(cfl) || nsteps < 0) return fail(c, GKS_ERR_ARG, "cfl > 0 and nsteps >= 0 required");
     if (c->dim == 1) return steps_1d_cfl(c, cfl, nsteps);
+    /* the wave speed of the current state in slot 0, then every step takes its
+     * time step from one slot and leaves the new state's wave speed in the other,
+     * so a step is seven launches (nine with a memory set and a pass over the
+     * state each step) */
+    if (nsteps < 1) return GKS_OK;
+    cudaError_t e = run_wavespeed(c);
     for (int s = 0; s < nsteps; ++s) {
-        cudaError_t e = run_wavespeed(c, cfl);
+        unsigned long long *in = c->smax + 2 * (s & 1), *out = s + 1 < nsteps ? c->smax + 2 * (~s & 1) : nullptr;
+        if (e == cudaSuccess) e = run_dt(c, cfl, in, out);
         if (e != cudaSuccess) return cuda_fail(c, e, "time step");
-        int r = two_stages(c);
+        int r = two_stages(c, out);
         if (r) return r;
     }
     return GKS_OK;
@@ -528,7 +544,7 @@ int gks_max_wavespeed(gks_handle_t c, double *out)
 {
     if (!c) return fail(nullptr, GKS_ERR_ARG, "NULL handle");
     if (!out) return fail(c, GKS_ERR_ARG, "out is NULL");
-    cudaError_t e = run_wavespeed(c, 0.0);
+    cudaError_t e = run_wavespeed(c);
     if (e != cudaSuccess) return cuda_fail(c, e, "wavespeed");
     unsigned long long bits = 0;
     e = cudaMemcpyAsync(&bits, c->smax, sizeof(bits), cudaMemcpyDeviceToHost, c->stream);

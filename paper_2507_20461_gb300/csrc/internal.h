@@ -92,8 +92,11 @@ template <int M> cudaError_t launch_states(gks_ctx *c, int input, double *fs_dev
 /* sums: the step path (multi-D: per-face Gauss sums, read by the update);
  * false: per-Gauss-point fluxes (gks_flux) */
 template <int M> cudaError_t launch_flux(gks_ctx *c, int input, bool sums);
-template <int M> cudaError_t launch_update(gks_ctx *c, int stage);
-template <int M> cudaError_t launch_wavespeed(gks_ctx *c, double cfl);
+/* smax: the slot of the new state's wave speed (stage 2), or nullptr */
+template <int M> cudaError_t launch_update(gks_ctx *c, int stage, unsigned long long *smax);
+/* the wave speed of the current state into slot 0 */
+template <int M> cudaError_t launch_wavespeed(gks_ctx *c);
+template <int M> cudaError_t launch_dt(gks_ctx *c, double cfl, const unsigned long long *in, unsigned long long *clear);
 template <int M> cudaError_t launch_shadow(gks_ctx *c);
 /* 1D non-compact schemes (order 5 or 6): face states / HLLC fluxes of the
  * stage input (input 0: W, 1: Ws), and one classical RK4 step */

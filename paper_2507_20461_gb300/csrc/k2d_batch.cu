@@ -149,9 +149,10 @@ __global__ void __launch_bounds__(128) bk_update(const KP common, const GridDesc
     UpdC uc;
     if constexpr (sizeof(R) == sizeof(float)) uc = load_updc(updc + 10 * grid);
     const unsigned c = T.begin + threadIdx.x;
+    R wn[4];
     if (c < P.ncell)
         step_update_item<R, 2, STAGE>(P, (const R *)g.ff, dt[2 * grid], g.W, g.G, g.Ws, g.Gs, g.Acc, g.s0, g.s1,
-                                      status + grid, c, uc);
+                                      status + grid, c, uc, wn);
 }
 
 template <typename R> cudaError_t batch_speed(const BatchLaunch &L, const LaunchShape &S, cudaStream_t st)

@@ -1165,7 +1165,7 @@ __device__ __forceinline__ long face_of(const KP &P, int d, int i, int j, int k,
  * come from FP32 differences of the interface states and live in the shadow
  * only (Eq. slope).  mixed_update_var updates variable v (nc cells, fih =
  * 1/h in FP32) and returns its new FP32 value; mixed_update_cell all
- * variables and the admissibility flags. */
+ * variables (new FP32 values in wn) and the admissibility flags. */
 template <int M, int STAGE, typename FaceSum>
 __device__ __forceinline__ float mixed_update_var(long nc, float fih, const FaceSum &fsum, const UpdC &uc,
                                                  double *__restrict__ W, float *__restrict__ acc, const Shadow &s0,
@@ -1225,10 +1225,9 @@ template <int M> __device__ __forceinline__ void mixed_state_flags(const KP &P, 
 template <int M, int STAGE, typename FaceSum>
 __device__ __forceinline__ void mixed_update_cell(const KP &P, const FaceSum &fsum, const UpdC &uc,
                                                   double *__restrict__ W, float *__restrict__ acc, const Shadow &s0,
-                                                  const Shadow &s1, int *__restrict__ status, long cell)
+                                                  const Shadow &s1, int *__restrict__ status, long cell, float *wn)
 {
     constexpr int NV = M + 2;
-    float wn[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) wn[v] = mixed_update_var<M, STAGE>(P.ncell, P.fih, fsum, uc, W, acc, s0, s1, cell, v);
     mixed_state_flags<M>(P, wn, status);
@@ -1305,7 +1304,8 @@ __device__ __forceinline__ void update_item(const KP &P, const R *__restrict__ f
         auto fsum = [&](int q, int v, int d, int plus) -> float {
             return ff[(long)(q * NV + v) * nft + (plus ? fp[d] : fm[d])];
         };
-        mixed_update_cell<M, STAGE>(P, fsum, uc, W, (float *)Acc, s0, s1, status, cell);
+        float wn[NV];
+        mixed_update_cell<M, STAGE>(P, fsum, uc, W, (float *)Acc, s0, s1, status, cell, wn);
         return;
     }
     unsigned q0, q1 = 0;
@@ -1389,18 +1389,11 @@ template <typename T> __device__ __forceinline__ void speed_max(T s, T ir, unsig
     }
 }
 
-template <int M, typename T>
-__global__ void wavespeed_kernel(KP P, const T *__restrict__ W, unsigned long long *__restrict__ smax)
+/* the same over a block of whole warps, which all call it: one atomic per
+ * block and word, and none where the word is already as large (a stale read
+ * only adds an atomic) */
+template <typename T> __device__ __forceinline__ void block_speed_max(T s, T ir, unsigned long long *__restrict__ smax)
 {
-    T s = T(0), ir = T(0); /* max |u_d| + c and max 1 / rho */
-    const T gam = pick<T>(P.gamma, (float)(P.fgm1 + 1.0f));
-    for (long c = (long)blockIdx.x * blockDim.x + threadIdx.x; c < P.ncell; c += (long)gridDim.x * blockDim.x) {
-        T w[M + 2];
-#pragma unroll
-        for (int v = 0; v < M + 2; ++v) w[v] = W[v * P.ncell + c];
-        s = fmax(s, speed_of<M, T>(w, gam));
-        ir = fmax(ir, T(1) / w[0]);
-    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
@@ -1421,13 +1414,28 @@ __global__ void wavespeed_kernel(KP P, const T *__restrict__ W, unsigned long lo
             s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
             ir = fmax(ir, __shfl_xor_sync(0xffffffffu, ir, o));
         }
-        /* non-negative doubles order like their bit patterns; NaN is caught on the host */
-        const double sd = (double)s, id = (double)ir;
-        if (threadIdx.x == 0) {
-            atomicMax(smax, (unsigned long long)__double_as_longlong(isnan(sd) ? 1e300 : sd));
-            atomicMax(smax + 1, (unsigned long long)__double_as_longlong(isnan(id) ? 1e300 : id));
+        if (threadIdx.x < 2) {
+            /* non-negative doubles order like their bit patterns; NaN is caught on the host */
+            const double x = (double)(threadIdx.x ? ir : s);
+            const unsigned long long b = (unsigned long long)__double_as_longlong(isnan(x) ? 1e300 : x);
+            if (b > *(volatile unsigned long long *)(smax + threadIdx.x)) atomicMax(smax + threadIdx.x, b);
         }
     }
+}
+
+template <int M, typename T>
+__global__ void wavespeed_kernel(KP P, const T *__restrict__ W, unsigned long long *__restrict__ smax)
+{
+    T s = T(0), ir = T(0); /* max |u_d| + c and max 1 / rho */
+    const T gam = pick<T>(P.gamma, (float)(P.fgm1 + 1.0f));
+    for (long c = (long)blockIdx.x * blockDim.x + threadIdx.x; c < P.ncell; c += (long)gridDim.x * blockDim.x) {
+        T w[M + 2];
+#pragma unroll
+        for (int v = 0; v < M + 2; ++v) w[v] = W[v * P.ncell + c];
+        s = fmax(s, speed_of<M, T>(w, gam));
+        ir = fmax(ir, T(1) / w[0]);
+    }
+    block_speed_max<T>(s, ir, smax);
 }
 
 /* dt = cfl h / max(|u_d| + c), and with viscosity mu > 0 also at most
@@ -1442,8 +1450,10 @@ __device__ __forceinline__ double dt_of_speed(const unsigned long long *smax, do
 }
 
 static __global__ void dt_from_speed_kernel(const unsigned long long *__restrict__ smax, double cfl_h, double visc,
-                                            double *__restrict__ dtp, float *__restrict__ updc, double cw)
+                                            double *__restrict__ dtp, float *__restrict__ updc, double cw,
+                                            unsigned long long *__restrict__ clear)
 {
+    if (clear) clear[0] = clear[1] = 0ull;
     const double dt = dt_of_speed(smax, cfl_h, visc);
     dtp[0] = dt;
     dtp[1] = 1.0 / dt;

@@ -92,27 +92,28 @@ template <int M> cudaError_t launch_flux(gks_ctx *c, int input, bool sums)
     return c->precision ? flux_impl<float, M>(c, input, nullptr, true) : flux_impl<double, M>(c, input, nullptr, true);
 }
 
-template <typename R, int M, int STAGE> static void update_launch(gks_ctx *c)
+template <typename R, int M, int STAGE, bool SPEED> static void update_launch(gks_ctx *c, unsigned long long *smax)
 {
-    step_update_kernel<R, M, STAGE><<<blocks_for(c->kp.ncell, 256), 256, 0, c->stream>>>(
-        c->kp, (const R *)c->ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1, c->status, c->updc);
+    step_update_kernel<R, M, STAGE, SPEED><<<blocks_for(c->kp.ncell, 256), 256, 0, c->stream>>>(
+        c->kp, (const R *)c->ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1, c->status, c->updc, smax);
 }
 
-template <typename R, int M> static cudaError_t update_impl(gks_ctx *c, int stage)
+template <typename R, int M> static cudaError_t update_impl(gks_ctx *c, int stage, unsigned long long *smax)
 {
     ProfScope ps(c, GKS_KC_UPDATE);
-    if (stage == 1) update_launch<R, M, 1>(c);
-    else update_launch<R, M, 2>(c);
+    if (stage == 1) update_launch<R, M, 1, false>(c, nullptr);
+    else if (smax) update_launch<R, M, 2, true>(c, smax);
+    else update_launch<R, M, 2, false>(c, nullptr);
     return cudaGetLastError();
 }
 
-template <int M> cudaError_t launch_update(gks_ctx *c, int stage)
+template <int M> cudaError_t launch_update(gks_ctx *c, int stage, unsigned long long *smax)
 {
     if constexpr (M == 1) return cudaErrorInvalidValue; /* the 1D stages update in the kernel that evaluates the fluxes */
-    else return c->precision ? update_impl<float, M>(c, stage) : update_impl<double, M>(c, stage);
+    else return c->precision ? update_impl<float, M>(c, stage, smax) : update_impl<double, M>(c, stage, smax);
 }
 
-template <int M> cudaError_t launch_wavespeed(gks_ctx *c, double cfl)
+template <int M> cudaError_t launch_wavespeed(gks_ctx *c)
 {
     cudaError_t e = cudaMemsetAsync(c->smax, 0, 2 * sizeof(unsigned long long), c->stream);
     if (e != cudaSuccess) return e;
@@ -125,13 +126,18 @@ template <int M> cudaError_t launch_wavespeed(gks_ctx *c, double cfl)
     ProfScope ps(c, GKS_KC_DT);
     if (c->shadows) wavespeed_kernel<M, float><<<nb, 256, 0, c->stream>>>(c->kp, c->s0.hi, c->smax);
     else wavespeed_kernel<M, double><<<nb, 256, 0, c->stream>>>(c->kp, c->W, c->smax);
-    if (cfl > 0.0) {
-        /* viscous limit cfl h^2 / (2 (m - 1) nu): passed as the factor
-         * 2 (m - 1) mu / h that turns max(1 / rho) into the rate cfl h / dt */
-        const double visc = c->kp.fp.mu > 0.0 ? 2.0 * (M > 1 ? M - 1 : 1) * c->kp.fp.mu / c->h : 0.0;
-        dt_from_speed_kernel<<<1, 1, 0, c->stream>>>(c->smax, cfl * c->h, visc, c->dt, c->shadows ? c->updc : nullptr,
-                                                     updc_cw(c->kp, M));
-    }
+    return cudaGetLastError();
+}
+
+/* the time step of wave speed slot in; clears the slot that the step's last stage adds to */
+template <int M> cudaError_t launch_dt(gks_ctx *c, double cfl, const unsigned long long *in, unsigned long long *clear)
+{
+    /* viscous limit cfl h^2 / (2 (m - 1) nu): passed as the factor
+     * 2 (m - 1) mu / h that turns max(1 / rho) into the rate cfl h / dt */
+    const double visc = c->kp.fp.mu > 0.0 ? 2.0 * (M > 1 ? M - 1 : 1) * c->kp.fp.mu / c->h : 0.0;
+    ProfScope ps(c, GKS_KC_DT);
+    dt_from_speed_kernel<<<1, 1, 0, c->stream>>>(in, cfl * c->h, visc, c->dt, c->shadows ? c->updc : nullptr,
+                                                 updc_cw(c->kp, M), clear);
     return cudaGetLastError();
 }
 
@@ -147,8 +153,9 @@ template <int M> cudaError_t launch_shadow(gks_ctx *c)
 #define GKS_INSTANTIATE(M)                                                                                \
     template cudaError_t launch_states<M>(gks_ctx *, int, double *);                                      \
     template cudaError_t launch_flux<M>(gks_ctx *, int, bool);                                            \
-    template cudaError_t launch_update<M>(gks_ctx *, int);                                                \
-    template cudaError_t launch_wavespeed<M>(gks_ctx *, double);                                          \
+    template cudaError_t launch_update<M>(gks_ctx *, int, unsigned long long *);                          \
+    template cudaError_t launch_wavespeed<M>(gks_ctx *);                                                  \
+    template cudaError_t launch_dt<M>(gks_ctx *, double, const unsigned long long *, unsigned long long *); \
     template cudaError_t launch_shadow<M>(gks_ctx *);
 
 } // namespace gks

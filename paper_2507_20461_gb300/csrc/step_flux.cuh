@@ -351,12 +351,12 @@ __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, M, NS>)
     }
 }
 
-/* the stage update from the face sums of step_face_item */
+/* the stage update from the face sums of step_face_item; wn receives the new averages */
 template <typename R, int M, int STAGE>
 __device__ __forceinline__ void step_update_item(const KP &P, const R *__restrict__ ff, double dt, double *__restrict__ W,
                                                  double *__restrict__ G, double *__restrict__ Ws, double *__restrict__ Gs,
                                                  double *__restrict__ Acc, const Shadow &s0, const Shadow &s1,
-                                                 int *__restrict__ status, long cell, const UpdC &uc)
+                                                 int *__restrict__ status, long cell, const UpdC &uc, R *wn)
 {
     constexpr int NV = M + 2;
     unsigned q0, q1;
@@ -371,24 +371,33 @@ __device__ __forceinline__ void step_update_item(const KP &P, const R *__restric
     }
     auto fsum = [&](int q, int v, int d, int plus) -> R { return (plus ? fp[d] : fm[d])[(q * NV + v) * 32]; };
     if constexpr (sizeof(R) == sizeof(float))
-        mixed_update_cell<M, STAGE>(P, fsum, uc, W, (float *)Acc, s0, s1, status, cell);
-    else {
-        double Wn[NV];
-        fp64_update_cell<M, STAGE>(P, fsum, 1.0 / (M == 2 ? 2 : 4), dt, W, G, Ws, Gs, Acc, status, cell, Wn);
-    }
+        mixed_update_cell<M, STAGE>(P, fsum, uc, W, (float *)Acc, s0, s1, status, cell, wn);
+    else
+        fp64_update_cell<M, STAGE>(P, fsum, 1.0 / (M == 2 ? 2 : 4), dt, W, G, Ws, Gs, Acc, status, cell, wn);
 }
 
-template <typename R, int M, int STAGE>
+/* SPEED: the new state's wave speed into smax as well (the last stage of a CFL
+ * step that another follows), from the values that wavespeed_kernel would read */
+template <typename R, int M, int STAGE, bool SPEED>
 __global__ void __launch_bounds__(256) step_update_kernel(KP P, const R *__restrict__ ff, const double *__restrict__ dtp,
                                                           double *__restrict__ W, double *__restrict__ G,
                                                           double *__restrict__ Ws, double *__restrict__ Gs,
                                                           double *__restrict__ Acc, Shadow s0, Shadow s1,
-                                                          int *__restrict__ status, const float *__restrict__ updc)
+                                                          int *__restrict__ status, const float *__restrict__ updc,
+                                                          unsigned long long *__restrict__ smax)
 {
     UpdC uc;
     if constexpr (sizeof(R) == sizeof(float)) uc = load_updc(updc);
     const long cell = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell < P.ncell) step_update_item<R, M, STAGE>(P, ff, dtp[0], W, G, Ws, Gs, Acc, s0, s1, status, cell, uc);
+    R wn[M + 2], s = R(0), ir = R(0);
+    if (cell < P.ncell) {
+        step_update_item<R, M, STAGE>(P, ff, dtp[0], W, G, Ws, Gs, Acc, s0, s1, status, cell, uc, wn);
+        if constexpr (SPEED) {
+            s = fmax(R(0), speed_of<M, R>(wn, pick<R>(P.gamma, (float)(P.fgm1 + 1.0f)))); /* a NaN counts as 0 */
+            ir = fmax(R(0), R(1) / wn[0]);
+        }
+    }
+    if constexpr (SPEED) block_speed_max<R>(s, ir, smax);
 }
 
 } // namespace gks
