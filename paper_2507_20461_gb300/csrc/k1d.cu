@@ -10,10 +10,10 @@ template <typename R, bool NS> static cudaError_t step1d(gks_ctx *c, const StepC
     const unsigned nb = blocks_for(c->kp.n[0], kCells1d);
     {
         ProfScope ps(c, GKS_KC_FACE);
-        step1d_kernel<R, NS, 1><<<nb, 32, 0, c->stream>>>(c->kp, c->W, c->G, c->W, c->G, c->Ws, c->Gs, c->Acc, c->status, first);
+        launch_chained(step1d_kernel<R, NS, 1>, nb, 32, c->stream, c->kp, c->W, c->G, c->W, c->G, c->Ws, c->Gs, c->Acc, c->status, first);
     }
     ProfScope ps(c, GKS_KC_FACE);
-    step1d_kernel<R, NS, 2><<<nb, 32, 0, c->stream>>>(c->kp, c->Ws, c->Gs, c->W, c->G, c->Ws, c->Gs, c->Acc, c->status, last);
+    launch_chained(step1d_kernel<R, NS, 2>, nb, 32, c->stream, c->kp, c->Ws, c->Gs, c->W, c->G, c->Ws, c->Gs, c->Acc, c->status, last);
     return cudaGetLastError();
 }
 
@@ -22,10 +22,10 @@ template <bool NS> static cudaError_t step1d_short(gks_ctx *c, const StepClock &
     const unsigned nb = blocks_for(c->kp.n[0], kCellsShort);
     {
         ProfScope ps(c, GKS_KC_FACE);
-        step1d_short_kernel<NS, 1><<<nb, 128, 0, c->stream>>>(c->kp, c->W, c->G, c->W, c->G, c->Ws, c->Gs, c->Acc, c->status, first);
+        launch_chained(step1d_short_kernel<NS, 1>, nb, 128, c->stream, c->kp, c->W, c->G, c->W, c->G, c->Ws, c->Gs, c->Acc, c->status, first);
     }
     ProfScope ps(c, GKS_KC_FACE);
-    step1d_short_kernel<NS, 2><<<nb, 128, 0, c->stream>>>(c->kp, c->Ws, c->Gs, c->W, c->G, c->Ws, c->Gs, c->Acc, c->status, last);
+    launch_chained(step1d_short_kernel<NS, 2>, nb, 128, c->stream, c->kp, c->Ws, c->Gs, c->W, c->G, c->Ws, c->Gs, c->Acc, c->status, last);
     return cudaGetLastError();
 }
 

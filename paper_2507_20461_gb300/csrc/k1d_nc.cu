@@ -227,6 +227,7 @@ __global__ void __launch_bounds__(32) nc_stage_kernel(KP P, const double *__rest
                                                       double *__restrict__ Wout, double *__restrict__ Acc,
                                                       int *__restrict__ status, StepClock clk)
 {
+    after_previous(Win, clk.dt, clk.in);
     const int lane = threadIdx.x, n = P.n[0];
     const int f = min((int)blockIdx.x * kCells1d + lane, n); /* lanes past the last face repeat it */
     const double dt = clock_dt(clk);
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(128) nc_short_kernel(KP P, const double *__res
                                                        double *__restrict__ Wout, double *__restrict__ Acc,
                                                        int *__restrict__ status, StepClock clk)
 {
+    after_previous(Win, clk.dt, clk.in);
     __shared__ double q[kShortFaces][3];
     const int n = P.n[0], sub = threadIdx.x & 7, face = threadIdx.x >> 3;
     const int f = min((int)blockIdx.x * kCellsShort + face, n); /* past the last face: the last face again */
@@ -308,9 +310,9 @@ void nc_stage(gks_ctx *c, const double *in, double *out, const StepClock &clk)
     const KP &P = c->kp;
     ProfScope ps(c, GKS_KC_FACE);
     if (short_1d(P.n[0]))
-        nc_short_kernel<ORDER, STAGE><<<blocks_for(P.n[0], kCellsShort), 128, 0, c->stream>>>(P, in, c->W, out, c->Acc, c->status, clk);
+        launch_chained(nc_short_kernel<ORDER, STAGE>, blocks_for(P.n[0], kCellsShort), 128, c->stream, P, in, c->W, out, c->Acc, c->status, clk);
     else
-        nc_stage_kernel<ORDER, STAGE><<<blocks_for(P.n[0], kCells1d), 32, 0, c->stream>>>(P, in, c->W, out, c->Acc, c->status, clk);
+        launch_chained(nc_stage_kernel<ORDER, STAGE>, blocks_for(P.n[0], kCells1d), 32, c->stream, P, in, c->W, out, c->Acc, c->status, clk);
 }
 
 template <int ORDER> cudaError_t nc_step(gks_ctx *c, const StepClock &first, const StepClock &mid, const StepClock &last)

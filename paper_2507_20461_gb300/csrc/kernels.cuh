@@ -23,6 +23,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "chain.cuh"
 #include "fpsplit.cuh"
 #include "geno_coeffs.cuh"
 #include "gks_device.cuh"
@@ -747,6 +748,7 @@ __device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R
 template <typename R, int M, bool GROUPED = false>
 __global__ void __launch_bounds__(128) cell_poly_kernel(KP P, Src<R> src, R *__restrict__ B)
 {
+    after_previous();
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < P.next) cell_poly_item<R, M, GROUPED>(P, src, B, t);
 }
@@ -1426,6 +1428,7 @@ template <typename T> __device__ __forceinline__ void block_speed_max(T s, T ir,
 template <int M, typename T>
 __global__ void wavespeed_kernel(KP P, const T *__restrict__ W, unsigned long long *__restrict__ smax)
 {
+    after_previous(W);
     T s = T(0), ir = T(0); /* max |u_d| + c and max 1 / rho */
     const T gam = pick<T>(P.gamma, (float)(P.fgm1 + 1.0f));
     for (long c = (long)blockIdx.x * blockDim.x + threadIdx.x; c < P.ncell; c += (long)gridDim.x * blockDim.x) {
@@ -1453,6 +1456,7 @@ static __global__ void dt_from_speed_kernel(const unsigned long long *__restrict
                                             double *__restrict__ dtp, float *__restrict__ updc, double cw,
                                             unsigned long long *__restrict__ clear)
 {
+    after_previous(smax);
     if (clear) clear[0] = clear[1] = 0ull;
     const double dt = dt_of_speed(smax, cfl_h, visc);
     dtp[0] = dt;

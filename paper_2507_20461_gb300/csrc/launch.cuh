@@ -68,12 +68,12 @@ template <typename R, int M, bool NS> static cudaError_t step_flux_impl(gks_ctx 
     (void)prep;
     {
         ProfScope ps(c, GKS_KC_RECON);
-        cell_poly_kernel<R, M, true><<<blocks_for(P.next), kBlock, 0, c->stream>>>(P, stage_src<R>(c, input), B);
+        launch_chained(cell_poly_kernel<R, M, true>, blocks_for(P.next), kBlock, c->stream, P, stage_src<R>(c, input), B);
     }
     const unsigned nb0 = blocks_for(P.nface[0], BT), nb1 = nb0 + blocks_for(P.nface[1], BT);
     const unsigned nb = M == 3 ? nb1 + blocks_for(P.nface[2], BT) : nb1;
     ProfScope ps(c, GKS_KC_FACE);
-    step_flux_kernel<R, M, NS><<<nb, BT, 0, c->stream>>>(P, B, c->dt, (R *)c->ff, c->status, nb0, nb1);
+    launch_chained(step_flux_kernel<R, M, NS>, nb, BT, c->stream, P, B, c->dt, (R *)c->ff, c->status, nb0, nb1);
     return cudaGetLastError();
 }
 
@@ -94,8 +94,7 @@ template <int M> cudaError_t launch_flux(gks_ctx *c, int input, bool sums)
 
 template <typename R, int M, int STAGE, bool SPEED> static void update_launch(gks_ctx *c, unsigned long long *smax)
 {
-    step_update_kernel<R, M, STAGE, SPEED><<<blocks_for(c->kp.ncell, 256), 256, 0, c->stream>>>(
-        c->kp, (const R *)c->ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1, c->status, c->updc, smax);
+    launch_chained(step_update_kernel<R, M, STAGE, SPEED>, blocks_for(c->kp.ncell, 256), 256, c->stream, c->kp, (const R *)c->ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1, c->status, c->updc, smax);
 }
 
 template <typename R, int M> static cudaError_t update_impl(gks_ctx *c, int stage, unsigned long long *smax)
@@ -136,7 +135,7 @@ template <int M> cudaError_t launch_dt(gks_ctx *c, double cfl, const unsigned lo
      * 2 (m - 1) mu / h that turns max(1 / rho) into the rate cfl h / dt */
     const double visc = c->kp.fp.mu > 0.0 ? 2.0 * (M > 1 ? M - 1 : 1) * c->kp.fp.mu / c->h : 0.0;
     ProfScope ps(c, GKS_KC_DT);
-    dt_from_speed_kernel<<<1, 1, 0, c->stream>>>(in, cfl * c->h, visc, c->dt, c->shadows ? c->updc : nullptr,
+    launch_chained(dt_from_speed_kernel, 1, 1, c->stream, in, cfl * c->h, visc, c->dt, c->shadows ? c->updc : nullptr,
                                                  updc_cw(c->kp, M), clear);
     return cudaGetLastError();
 }

@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(128) step1d_short_kernel(KP P, const double *_
                                                            double *__restrict__ Ws, double *__restrict__ Gs,
                                                            double *__restrict__ Acc, int *__restrict__ status, StepClock clk)
 {
+    after_previous(Win, Gin, clk.dt, clk.in);
     __shared__ double q[kShortFaces][9];
     const int n = P.n[0], sub = threadIdx.x & 7, face = threadIdx.x >> 3;
     const int f = min((int)blockIdx.x * kCellsShort + face, n); /* past the last face: the last face again */
@@ -172,6 +173,7 @@ __global__ void __launch_bounds__(32) step1d_kernel(KP P, const double *__restri
                                                     double *__restrict__ Gs, double *__restrict__ Acc,
                                                     int *__restrict__ status, StepClock clk)
 {
+    after_previous(Win, Gin, clk.dt, clk.in);
     const int lane = threadIdx.x, n = P.n[0];
     const int f = min((int)blockIdx.x * kCells1d + lane, n); /* lanes past the last face repeat it */
     const double dt = clock_dt(clk);

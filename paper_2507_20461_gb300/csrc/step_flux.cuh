@@ -335,6 +335,7 @@ __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, M, NS>)
     constexpr int BT = kStepFluxBlock;
     __shared__ typename FaceV<R>::V slots[kFaceStash<R, M> * BT];
     typename FaceV<R>::V *stash = slots + threadIdx.x;
+    after_previous(B, dtp);
     const R dt = R(dtp[0]), idt = R(dtp[1]);
     const unsigned b = blockIdx.x;
     if (b < nb0) {
@@ -369,7 +370,7 @@ __device__ __forceinline__ void step_update_item(const KP &P, const R *__restric
         fm[d] = ff + group_off<kFaceFields<M>>((unsigned)face_of<M>(P, d, i, j, k, 0));
         fp[d] = ff + group_off<kFaceFields<M>>((unsigned)face_of<M>(P, d, i, j, k, 1));
     }
-    auto fsum = [&](int q, int v, int d, int plus) -> R { return (plus ? fp[d] : fm[d])[(q * NV + v) * 32]; };
+    auto fsum = [&](int q, int v, int d, int plus) -> R { return load_ro((plus ? fp[d] : fm[d]) + (q * NV + v) * 32); };
     if constexpr (sizeof(R) == sizeof(float))
         mixed_update_cell<M, STAGE>(P, fsum, uc, W, (float *)Acc, s0, s1, status, cell, wn);
     else
@@ -386,6 +387,7 @@ __global__ void __launch_bounds__(256) step_update_kernel(KP P, const R *__restr
                                                           int *__restrict__ status, const float *__restrict__ updc,
                                                           unsigned long long *__restrict__ smax)
 {
+    after_previous(ff, dtp, updc);
     UpdC uc;
     if constexpr (sizeof(R) == sizeof(float)) uc = load_updc(updc);
     const long cell = (long)blockIdx.x * blockDim.x + threadIdx.x;
