@@ -8,6 +8,7 @@
 #include <new>
 
 #include "internal.h"
+#include "state_io.cuh"
 #include "step_1d.cuh"
 #include "step_flux.cuh"
 
@@ -104,10 +105,8 @@ Layout layout(const gks_grid_t *g, int precision)
 
 int sync_status(gks_ctx *c)
 {
-    cudaError_t e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "stream synchronize");
     int st = 0;
-    e = cudaMemcpy(&st, c->status, sizeof(int), cudaMemcpyDeviceToHost);
+    const cudaError_t e = gks::read_status(c->status, &st, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "status read");
     return st;
 }
@@ -145,6 +144,25 @@ cudaError_t run_shadow(gks_ctx *c)
     case 1: return gks::launch_shadow<1>(c);
     case 2: return gks::launch_shadow<2>(c);
     default: return gks::launch_shadow<3>(c);
+    }
+}
+
+cudaError_t run_state_in(gks_ctx *c, const double *W, const double *G, long n)
+{
+    switch (c->dim) {
+    case 1: return gks::state_in<1>(W, G, c->W, c->G, c->s0, n, c->status, c->stream);
+    case 2: return gks::state_in<2>(W, G, c->W, c->G, c->s0, n, c->status, c->stream);
+    default: return gks::state_in<3>(W, G, c->W, c->G, c->s0, n, c->status, c->stream);
+    }
+}
+
+cudaError_t run_state_out(gks_ctx *c, double *W, double *G, long n)
+{
+    const float *g = c->g_stale ? c->s0.g : nullptr;
+    switch (c->dim) {
+    case 1: return gks::state_out<1>(c->W, c->G, g, W, G, n, c->stream);
+    case 2: return gks::state_out<2>(c->W, c->G, g, W, G, n, c->stream);
+    default: return gks::state_out<3>(c->W, c->G, g, W, G, n, c->stream);
     }
 }
 
@@ -416,11 +434,16 @@ int gks_set_state(gks_handle_t c, const double *W, const double *G, int on_devic
     if (!W || !G) return fail(c, GKS_ERR_ARG, "W and G are required");
     const size_t nW = (size_t)c->nv * c->kp.ncell, nG = (size_t)c->dim * nW;
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    cudaError_t e = cudaMemcpyAsync(c->W, W, nW * sizeof(double), k, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->G, G, nG * sizeof(double), k, c->stream);
-    if (e == cudaSuccess) e = run_shadow(c);
+    cudaError_t e;
+    if (on_device && gks::in_device_memory(W, nW * sizeof(double)) && gks::in_device_memory(G, nG * sizeof(double)))
+        e = run_state_in(c, W, G, (long)nW);
+    else {
+        e = cudaMemcpyAsync(c->W, W, nW * sizeof(double), k, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(c->G, G, nG * sizeof(double), k, c->stream);
+        if (e == cudaSuccess) e = run_shadow(c);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->status, 0, sizeof(int), c->stream);
+    }
     c->g_stale = 0;
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->status, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "set_state");
     c->err[0] = 0;
@@ -433,14 +456,16 @@ int gks_get_state(gks_handle_t c, double *W, double *G, int on_device)
     const size_t nW = (size_t)c->nv * c->kp.ncell, nG = (size_t)c->dim * nW;
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     cudaError_t e = cudaSuccess;
-    if (G && c->g_stale) {
+    const bool direct = on_device && W && G && gks::in_device_memory(W, nW * sizeof(double)) && gks::in_device_memory(G, nG * sizeof(double));
+    if (direct) e = run_state_out(c, W, G, (long)nW);
+    else if (G && c->g_stale) {
         gks::widen_grad_kernel<<<gks::blocks_for((long)nG, 256) > 4096 ? 4096 : gks::blocks_for((long)nG, 256), 256, 0,
                                  c->stream>>>(c->s0.g, c->G, (long)nG);
         e = cudaGetLastError();
         if (e == cudaSuccess) c->g_stale = 0;
     }
-    if (e == cudaSuccess && W) e = cudaMemcpyAsync(W, c->W, nW * sizeof(double), k, c->stream);
-    if (e == cudaSuccess && G) e = cudaMemcpyAsync(G, c->G, nG * sizeof(double), k, c->stream);
+    if (!direct && e == cudaSuccess && W) e = cudaMemcpyAsync(W, c->W, nW * sizeof(double), k, c->stream);
+    if (!direct && e == cudaSuccess && G) e = cudaMemcpyAsync(G, c->G, nG * sizeof(double), k, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "get_state");
     const int st = sync_status(c);
     if (st < 0) return st;

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "batch.h"
+#include "state_io.cuh"
 #include "step_flux.cuh"
 
 using gks::BatchLaunch;
@@ -509,11 +510,13 @@ int gks_batch_set_state(gks_batch_t b, int grid, const double *W, const double *
     /* the caller's buffers may still be written by work on its stream */
     cudaError_t e = cudaEventRecord(b->ev_in, b->user_stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_in, 0);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(D.W, W, n * sizeof(double), k, b->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(D.G, G, 2 * n * sizeof(double), k, b->stream);
-    if (e == cudaSuccess && b->precision == 1) e = gks::batch_shadow(D, b->stream);
+    const bool direct = on_device && gks::in_device_memory(W, n * sizeof(double)) && gks::in_device_memory(G, 2 * n * sizeof(double));
+    if (direct && e == cudaSuccess) e = gks::state_in<2>(W, G, D.W, D.G, D.s0, (long)n, b->status + grid, b->stream);
+    if (!direct && e == cudaSuccess) e = cudaMemcpyAsync(D.W, W, n * sizeof(double), k, b->stream);
+    if (!direct && e == cudaSuccess) e = cudaMemcpyAsync(D.G, G, 2 * n * sizeof(double), k, b->stream);
+    if (!direct && e == cudaSuccess && b->precision == 1) e = gks::batch_shadow(D, b->stream);
     b->g_stale[grid] = 0;
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->status + grid, 0, sizeof(int), b->stream);
+    if (!direct && e == cudaSuccess) e = cudaMemsetAsync(b->status + grid, 0, sizeof(int), b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     return e == cudaSuccess ? GKS_OK : bcuda(b, e, "batch set_state");
 }
@@ -528,17 +531,19 @@ int gks_batch_get_state(gks_batch_t b, int grid, double *W, double *G, int on_de
     /* the caller's stream may still use the destination buffers */
     cudaError_t e = cudaEventRecord(b->ev_in, b->user_stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_in, 0);
-    if (e == cudaSuccess && G && b->precision && b->g_stale[grid]) {
+    const bool direct = on_device && W && G && gks::in_device_memory(W, n * sizeof(double)) &&
+                        gks::in_device_memory(G, 2 * n * sizeof(double));
+    if (direct && e == cudaSuccess)
+        e = gks::state_out<2>(D.W, D.G, b->precision && b->g_stale[grid] ? D.s0.g : nullptr, W, G, (long)n, b->stream);
+    if (!direct && e == cudaSuccess && G && b->precision && b->g_stale[grid]) {
         e = gks::batch_widen_grad(D, b->stream);
         if (e == cudaSuccess) b->g_stale[grid] = 0;
     }
-    if (e == cudaSuccess && W) e = cudaMemcpyAsync(W, D.W, n * sizeof(double), k, b->stream);
-    if (e == cudaSuccess && G) e = cudaMemcpyAsync(G, D.G, 2 * n * sizeof(double), k, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return bcuda(b, e, "batch get_state");
+    if (!direct && e == cudaSuccess && W) e = cudaMemcpyAsync(W, D.W, n * sizeof(double), k, b->stream);
+    if (!direct && e == cudaSuccess && G) e = cudaMemcpyAsync(G, D.G, 2 * n * sizeof(double), k, b->stream);
     int st = 0;
-    e = cudaMemcpy(&st, b->status + grid, sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return bcuda(b, e, "status read");
+    if (e == cudaSuccess) e = gks::read_status(b->status + grid, &st, b->stream);
+    if (e != cudaSuccess) return bcuda(b, e, "batch get_state");
     if (st) return bfail(b, GKS_ERR_NONPHYSICAL, "grid %d: non-physical state (status bits 0x%x)", grid, st);
     return GKS_OK;
 }
