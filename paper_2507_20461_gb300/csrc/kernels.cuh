@@ -317,6 +317,8 @@ __device__ __forceinline__ bool admissible(const R *w, const R *wc, R, R delta)
         ke += w[1 + a] * w[1 + a];
         kc += wc[1 + a] * wc[1 + a];
     }
+    if constexpr (sizeof(R) == sizeof(float)) /* products of three factors would leave FP32's range early */
+        return w[0] > delta * wc[0] && w[M + 1] - R(0.5) * ke / w[0] > delta * (wc[M + 1] - R(0.5) * kc / wc[0]);
     /* p > delta p_c without divisions: rho p / (gamma - 1) = q, so
      * q rho_c > delta q_c rho (reversed where rho_c < 0; a rho <= 0 fails in the
      * flux either way) */

@@ -157,16 +157,18 @@ template <typename R> __device__ __forceinline__ const R *opaque(const R *p)
 /* The flux of one Gauss point from the face-frame states and derivatives
  * W[g][v], dW[g][e][v] (cell units) of both sides, after the admissibility
  * fallback: a side whose density or pressure is not above adm times its cell's
- * takes the cell average (average(g, v)) with zero slopes.  Without divisions:
- * rho p / (gamma - 1) = q = rho E - |m|^2 / 2, so p > adm p_c is q rho_c > adm q_c rho
- * (reversed where rho_c < 0; a rho <= 0 fails in the flux either way).  rc, dqc:
- * rho_c and adm q_c per side.  False: a state the flux could not use. */
+ * takes the cell average (average(g, v)) with zero slopes.  Without divisions
+ * here: rho p / (gamma - 1) = q = rho E - |m|^2 / 2, so p > adm p_c is q > dpc rho,
+ * rc = rho_c, dpc = adm p_c / (gamma - 1) (FP32: products of two factors only, the
+ * range of the test with divisions; 64-bit: q rho_c > dpc rho with dpc = adm q_c,
+ * reversed where rho_c < 0, which spares a division a face).  A rho <= 0 fails in
+ * the flux either way.  False: a state the flux could not use. */
 template <typename R, int M, bool NS, typename Average>
 __device__ __forceinline__ bool face_point(const FluxParams &fp, R adm, R dt, R idt, R ih,
                                            typename FaceV<R>::V (&W)[FaceV<R>::G][M + 2],
                                            typename FaceV<R>::V (&dW)[FaceV<R>::G][M][M + 2],
                                            const typename FaceV<R>::V (&rc)[FaceV<R>::G],
-                                           const typename FaceV<R>::V (&dqc)[FaceV<R>::G], const Average &average, R *F,
+                                           const typename FaceV<R>::V (&dpc)[FaceV<R>::G], const Average &average, R *F,
                                            R *Ft, R *Wh)
 {
     using V = typename FaceV<R>::V;
@@ -177,10 +179,11 @@ __device__ __forceinline__ bool face_point(const FluxParams &fp, R adm, R dt, R 
 #pragma unroll
         for (int i = 0; i < M; ++i) ke += W[g][1 + i] * W[g][1 + i];
         const V q = W[g][0] * W[g][M + 1] - V(0.5) * ke;
-        const V t = q * rc[g] - dqc[g] * W[g][0], lo = V(adm) * rc[g];
+        const V lo = V(adm) * rc[g];
         if constexpr (G == 1) {
-            const bool okl = W[g][0].l() > lo.l() && (rc[g].l() >= 0.f ? t.l() > 0.f : t.l() < 0.f);
-            const bool okr = W[g][0].r() > lo.r() && (rc[g].r() >= 0.f ? t.r() > 0.f : t.r() < 0.f);
+            const V t = q - dpc[g] * W[g][0];
+            const bool okl = W[g][0].l() > lo.l() && t.l() > 0.f;
+            const bool okr = W[g][0].r() > lo.r() && t.r() > 0.f;
             if (!okl || !okr) {
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
@@ -191,6 +194,7 @@ __device__ __forceinline__ bool face_point(const FluxParams &fp, R adm, R dt, R 
                 }
             }
         } else {
+            const V t = q * rc[g] - dpc[g] * W[g][0];
             if (!(W[g][0] > lo && (rc[g] >= 0.0 ? t > 0.0 : t < 0.0))) {
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
@@ -242,8 +246,8 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
         const V sa = V(b ? 0.28867513459481287 : -0.28867513459481287);
         pl = opaque(pl);
         pr = opaque(pr);
-        /* face frame: W[g][v], dW[g][e][v]; rc, dqc: the cell averages' side of the admissibility test */
-        V W[G][NV], dW[G][M][NV], rc[G], dqc[G];
+        /* face frame: W[g][v], dW[g][e][v]; rc, dpc: the cell averages' side of the admissibility test */
+        V W[G][NV], dW[G][M][NV], rc[G], dpc[G];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             V kc = V(0), Ec = V(0), r0 = V(0);
@@ -267,7 +271,8 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
                 }
             }
             rc[g] = r0;
-            dqc[g] = V(adm) * (r0 * Ec - V(0.5) * kc);
+            if constexpr (G == 1) dpc[g] = V(adm) * (Ec - V(0.5) * (kc / r0));
+            else dpc[g] = V(adm) * (r0 * Ec - V(0.5) * kc);
         }
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
@@ -286,7 +291,7 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
                 return FV::load(opaque(pl), opaque(pr), g, (gv * (NC + 1) + NC) * 32);
             };
             R f[NV], ft[NV], wh[NV];
-            const bool ok = face_point<R, M, NS>(P.fp, adm, dt, idt, ih, W, dW, rc, dqc, average, f, ft, wh);
+            const bool ok = face_point<R, M, NS>(P.fp, adm, dt, idt, ih, W, dW, rc, dpc, average, f, ft, wh);
             if (ok) {
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
