@@ -43,13 +43,13 @@ template <typename T> __device__ __forceinline__ T load_ro(const T *p)
 
 #ifdef __CUDACC__
 template <typename... K, typename... A>
-cudaError_t launch_chained(void (*kernel)(K...), unsigned blocks, unsigned threads, cudaStream_t stream, A... args)
+cudaError_t launch_chained(void (*kernel)(K...), dim3 blocks, unsigned threads, cudaStream_t stream, A... args)
 {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(blocks);
+    cfg.gridDim = blocks;
     cfg.blockDim = dim3(threads);
     cfg.stream = stream;
     cfg.attrs = &at;

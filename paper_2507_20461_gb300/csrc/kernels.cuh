@@ -658,8 +658,8 @@ __device__ __forceinline__ void blend_cubic(const KP &P, const R *d, R *b)
 /* GROUPED = false: B[v][k][ext cell]; true: the step path's layout, the fields
  * of 32 consecutive cells in rows of 32, v (NC + 1) + k with k = NC the
  * (mirrored) average itself (step_flux.cuh). */
-template <typename R, int M, bool GROUPED = false>
-__device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R *__restrict__ B, long t)
+template <typename R, int M, bool GROUPED = false, bool ONE = false>
+__device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R *__restrict__ B, long t, int only = -1)
 {
     constexpr int NV = M + 2, NC = Cubic<R, M>::NC, ND = Cubic<R, M>::ND;
     int i, j, k;
@@ -700,7 +700,7 @@ __device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R
 #pragma unroll
     for (int q = 0; q <= 2 * M; ++q) anyflip |= sm[q];
 #pragma unroll 1
-    for (int v = 0; v < NV; ++v) {
+    for (int v = ONE ? only : 0; v < (ONE ? only + 1 : NV); ++v) {
         R d[ND];
         const R hr = pick<R>(P.h, P.fh);
         if (anyflip == 0) {
@@ -747,12 +747,12 @@ __device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R
     }
 }
 
-template <typename R, int M, bool GROUPED = false>
+template <typename R, int M, bool GROUPED = false, bool SPREAD = false>
 __global__ void __launch_bounds__(128) cell_poly_kernel(KP P, Src<R> src, R *__restrict__ B)
 {
     after_previous();
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < P.next) cell_poly_item<R, M, GROUPED>(P, src, B, t);
+    if (t < P.next) cell_poly_item<R, M, GROUPED, SPREAD>(P, src, B, t, (int)blockIdx.y);
 }
 
 template <int M>

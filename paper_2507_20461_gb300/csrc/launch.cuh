@@ -58,23 +58,55 @@ template <typename R, int M> static cudaError_t flux_impl(gks_ctx *c, int input,
     return cudaGetLastError();
 }
 
+template <typename R, int M, bool NS, bool SPLIT> static cudaError_t step_flux_launch(gks_ctx *c)
+{
+    const KP &P = c->kp;
+    constexpr int BT = kStepFluxBlock, FB = SPLIT ? BT / (M == 3 ? 4 : 2) : BT;
+    static const bool prep = SPLIT || (smem_carveout_for(step_flux_kernel<R, M, NS, SPLIT>, kStepFluxMinBlocks<R, M, NS>), true);
+    (void)prep;
+    const unsigned nb0 = blocks_for(P.nface[0], FB), nb1 = nb0 + blocks_for(P.nface[1], FB);
+    const unsigned nb = M == 3 ? nb1 + blocks_for(P.nface[2], FB) : nb1;
+    ProfScope ps(c, GKS_KC_FACE);
+    launch_chained(step_flux_kernel<R, M, NS, SPLIT>, nb, BT, c->stream, P, (const R *)c->B, c->dt, (R *)c->ff, c->status, nb0, nb1);
+    return cudaGetLastError();
+}
+
+inline int sm_count()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    return n;
+}
+/* Small grids, as blocks per SM: a thread per (cell, variable) in the
+ * reconstruction, a lane per Gauss point in the flux.  With too few blocks to
+ * hide a thread's chain of instructions the work of one is spread over several;
+ * past the lines below the repeated index work and evaluations cost more.
+ * Measured (GB300, us a step, plain / spread, then plain / split):
+ *   FP32 2D: 160^2 (1.4 recon, 5.3 flux blocks per SM) 44.9 / 40.5, 44.9 / 37.2;
+ *     224^2 (2.6, 10.4) 47.7 / 45.1, 47.7 / 44.9; 320^2 (5.3, 21) 63.9 / 60.3, 63.7 / 65.1;
+ *     448^2 (10.4, 41) 97.9 / 98.4, equal;
+ *   FP32 3D: 26^3 (1.1, 5.6) 88 / 71, 88 / 68; 32^3 (2.0, 10.4) 97 / 93, 97 / 90;
+ *     40 x 36^2 (3.1, 16) 117.6 / 117.1, 117.3 / 115.1; 48 x 40^2 (4.5, 24) 139 / 151, 139 / 152;
+ *   FP64 2D: 160^2 565 / 454, 565 / 590; 3D: 20^3 (0.6, 2.6) 986 / 669, 986 / 707;
+ *     26^3 1360 / 1110, 1360 / 1507; 64 x 50^2 (9.2, 50) 8451 / 8354. */
+template <typename R, int M> inline bool spread_cells(unsigned blocks)
+{
+    return blocks <= (sizeof(R) == sizeof(double) ? 10 : (M == 2 ? 6 : 3)) * sm_count();
+}
+template <typename R> inline bool split_faces(unsigned blocks) { return blocks <= (sizeof(R) == sizeof(double) ? 3 : 12) * sm_count(); }
+
 /* the multi-D step path: reconstruction and face sums (step_flux.cuh) */
 template <typename R, int M, bool NS> static cudaError_t step_flux_impl(gks_ctx *c, int input)
 {
     const KP &P = c->kp;
     R *B = (R *)c->B;
-    constexpr int BT = kStepFluxBlock;
-    static const bool prep = (smem_carveout_for(step_flux_kernel<R, M, NS>, kStepFluxMinBlocks<R, M, NS>), true);
-    (void)prep;
     {
         ProfScope ps(c, GKS_KC_RECON);
-        launch_chained(cell_poly_kernel<R, M, true>, blocks_for(P.next), kBlock, c->stream, P, stage_src<R>(c, input), B);
+        const unsigned nb = blocks_for(P.next);
+        if (spread_cells<R, M>(nb)) launch_chained(cell_poly_kernel<R, M, true, true>, dim3(nb, M + 2), kBlock, c->stream, P, stage_src<R>(c, input), B);
+        else launch_chained(cell_poly_kernel<R, M, true>, nb, kBlock, c->stream, P, stage_src<R>(c, input), B);
     }
-    const unsigned nb0 = blocks_for(P.nface[0], BT), nb1 = nb0 + blocks_for(P.nface[1], BT);
-    const unsigned nb = M == 3 ? nb1 + blocks_for(P.nface[2], BT) : nb1;
-    ProfScope ps(c, GKS_KC_FACE);
-    launch_chained(step_flux_kernel<R, M, NS>, nb, BT, c->stream, P, B, c->dt, (R *)c->ff, c->status, nb0, nb1);
-    return cudaGetLastError();
+    return split_faces<R>(blocks_for(P.nftot, kStepFluxBlock)) ? step_flux_launch<R, M, NS, true>(c) : step_flux_launch<R, M, NS, false>(c);
 }
 
 template <int M> cudaError_t launch_states(gks_ctx *c, int input, double *fs_dev)

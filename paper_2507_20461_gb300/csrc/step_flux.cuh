@@ -215,10 +215,13 @@ __device__ __forceinline__ bool face_point(const FluxParams &fp, R adm, R dt, R 
 }
 
 /* One face of direction D: fl its index among that direction's faces; stash the
- * thread's first shared slot, SS the slot stride. */
-template <typename R, int M, int D, bool NS, int SS>
+ * thread's first shared slot, SS the slot stride.
+ * SPLIT: each of 2 (3D: 4) neighbouring lanes takes one Gauss point of the face,
+ * all lanes of the warp call it, and the sums go over shuffles (no stash); lanes
+ * past the last face pass it again with store = false. */
+template <typename R, int M, int D, bool NS, int SS, bool SPLIT = false>
 __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict__ B, R dt, R idt, R *__restrict__ ff,
-                                               int *__restrict__ status, unsigned fl, typename FaceV<R>::V *stash)
+                                               int *__restrict__ status, unsigned fl, typename FaceV<R>::V *stash, bool store = true)
 {
     using FV = FaceV<R>;
     using V = typename FV::V;
@@ -241,8 +244,11 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
 #pragma unroll
     for (int v = 0; v < NV; ++v) F[v] = Ft[v] = Wh[v] = R(0);
     bool bad = false;
+    constexpr int NG = M == 3 ? 4 : 2;
+    const int point = SPLIT ? (int)(threadIdx.x % NG) : 0; /* SPLIT: this lane's Gauss point */
+    const int b0 = SPLIT ? point >> 1 : 0, b1 = SPLIT ? b0 + 1 : NG / 2;
 #pragma unroll 1
-    for (int b = 0; b < (M == 3 ? 2 : 1); ++b) {
+    for (int b = b0; b < b1; ++b) {
         const V sa = V(b ? 0.28867513459481287 : -0.28867513459481287);
         pl = opaque(pl);
         pr = opaque(pr);
@@ -262,12 +268,18 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
                 else if (v <= M) kc += w * w;
                 else Ec = w;
                 face_pair<V, M, D>(c, w, FV::sign(g), sa, o0, o1);
-                W[g][v] = o0[0];
-                stash[(g * NV + v) * (M + 1) * SS] = o1[0];
+                if constexpr (SPLIT) {
+                    W[g][v] = point & 1 ? o1[0] : o0[0];
 #pragma unroll
-                for (int e = 0; e < M; ++e) {
-                    dW[g][e][v] = o0[1 + e];
-                    stash[((g * NV + v) * (M + 1) + 1 + e) * SS] = o1[1 + e];
+                    for (int e = 0; e < M; ++e) dW[g][e][v] = point & 1 ? o1[1 + e] : o0[1 + e];
+                } else {
+                    W[g][v] = o0[0];
+                    stash[(g * NV + v) * (M + 1) * SS] = o1[0];
+#pragma unroll
+                    for (int e = 0; e < M; ++e) {
+                        dW[g][e][v] = o0[1 + e];
+                        stash[((g * NV + v) * (M + 1) + 1 + e) * SS] = o1[1 + e];
+                    }
                 }
             }
             rc[g] = r0;
@@ -275,7 +287,7 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
             else dpc[g] = V(adm) * (r0 * Ec - V(0.5) * kc);
         }
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
+        for (int p = 0; p < (SPLIT ? 1 : 2); ++p) {
             if (p) {
 #pragma unroll
                 for (int g = 0; g < G; ++g)
@@ -304,6 +316,17 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
         }
     }
     if (bad) atomicOr(status, ST_FLUX);
+    if constexpr (SPLIT) {
+#pragma unroll
+        for (int o = 1; o < NG; o <<= 1)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                F[v] += __shfl_xor_sync(0xffffffffu, F[v], o);
+                Ft[v] += __shfl_xor_sync(0xffffffffu, Ft[v], o);
+                Wh[v] += __shfl_xor_sync(0xffffffffu, Wh[v], o);
+            }
+        if (!store || point != 0) return;
+    }
     /* walls (slip or no-slip) are at rest and adiabatic: neither mass nor
      * energy crosses them (exactly, whatever the rounding of the two sides) */
     if ((idx[D] == 0 && P.bcs[D][0] >= 2) || (idx[D] == P.n[D] && P.bcs[D][1] >= 2))
@@ -332,29 +355,27 @@ constexpr int kStepFluxBlock = 64;
 template <typename R, int M, bool NS>
 constexpr int kStepFluxMinBlocks = sizeof(R) == sizeof(float) ? (M == 2 && !NS ? 12 : 8) : (M == 2 ? 6 : 4);
 
-template <typename R, int M, bool NS>
+/* SPLIT: a lane per Gauss point, 64 / NG faces a block */
+template <typename R, int M, bool NS, bool SPLIT>
 __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, M, NS>))
     step_flux_kernel(KP P, const R *__restrict__ B, const double *__restrict__ dtp, R *__restrict__ ff,
                      int *__restrict__ status, unsigned nb0, unsigned nb1)
 {
-    constexpr int BT = kStepFluxBlock;
-    __shared__ typename FaceV<R>::V slots[kFaceStash<R, M> * BT];
-    typename FaceV<R>::V *stash = slots + threadIdx.x;
+    constexpr int BT = kStepFluxBlock, PER = SPLIT ? (M == 3 ? 4 : 2) : 1, FB = BT / PER;
+    __shared__ typename FaceV<R>::V slots[SPLIT ? 1 : kFaceStash<R, M> * BT];
+    typename FaceV<R>::V *stash = SPLIT ? slots : slots + threadIdx.x;
     after_previous(B, dtp);
     const R dt = R(dtp[0]), idt = R(dtp[1]);
     const unsigned b = blockIdx.x;
-    if (b < nb0) {
-        const unsigned fl = b * BT + threadIdx.x;
-        if (fl < (unsigned)P.nface[0]) step_face_item<R, M, 0, NS, BT>(P, B, dt, idt, ff, status, fl, stash);
-    } else if (M == 2 || b < nb1) {
-        const unsigned fl = (b - nb0) * BT + threadIdx.x;
-        if (fl < (unsigned)P.nface[1]) step_face_item<R, M, 1, NS, BT>(P, B, dt, idt, ff, status, fl, stash);
-    } else {
-        if constexpr (M == 3) {
-            const unsigned fl = (b - nb1) * BT + threadIdx.x;
-            if (fl < (unsigned)P.nface[2]) step_face_item<R, M, 2, NS, BT>(P, B, dt, idt, ff, status, fl, stash);
-        }
-    }
+    auto face = [&](auto dir, unsigned block) {
+        constexpr int D = decltype(dir)::value;
+        const unsigned fl = block * FB + threadIdx.x / PER, n = (unsigned)P.nface[D];
+        if constexpr (SPLIT) step_face_item<R, M, D, NS, BT, true>(P, B, dt, idt, ff, status, fl < n ? fl : n - 1, stash, fl < n);
+        else if (fl < n) step_face_item<R, M, D, NS, BT>(P, B, dt, idt, ff, status, fl, stash);
+    };
+    if (b < nb0) face(std::integral_constant<int, 0>{}, b);
+    else if (M == 2 || b < nb1) face(std::integral_constant<int, 1>{}, b - nb0);
+    else if constexpr (M == 3) face(std::integral_constant<int, 2>{}, b - nb1);
 }
 
 /* the stage update from the face sums of step_face_item; wn receives the new averages */
