@@ -777,7 +777,7 @@ template <int M> __device__ __forceinline__ float *flux_stage()
 /* one (face, Gauss point) of direction D.  FLUX = false writes the states
  * face_states[side][v][c][g][face] (double, global axes); FLUX = true the
  * fluxes ff[q][v][g][face] (R, global momentum order). */
-template <typename R, int M, int D, bool FLUX, bool NS = false, bool FSUM = false>
+template <typename R, int M, int D, bool FLUX, bool NS = false>
 __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, const R *__restrict__ B, double dtv,
                                                double *__restrict__ fs, R *__restrict__ ff, int *__restrict__ status,
                                                long t)
@@ -804,8 +804,7 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
     }
     const bool valid = fl < nf && g < NG;
     /* a masked item evaluates the last face; in FP32 it keeps its warp's
-     * Gauss point (always < NG), which also places it in the face sums'
-     * shared tile below */
+     * Gauss point (always < NG) */
     if (!valid) {
         fl = nf - 1;
         if constexpr (!gfast) g = 0;
@@ -820,8 +819,7 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
      * are staged in shared memory, stage[side][v * NC + k][face in block].
      * Each face's NG threads copy a share of its 2 NV NC values with cp.async
      * (all copies in flight at once, each value read once per face instead
-     * of once per Gauss point, no registers held while they land); the face
-     * sums below reuse the buffer. */
+     * of once per Gauss point, no registers held while they land). */
     constexpr int FB = 128 / NG, NVC = NV * NC;
     float *stage = nullptr;
     if constexpr (gfast) stage = flux_stage<M>();
@@ -933,61 +931,18 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
      * energy crosses them (exactly, whatever the rounding of the two sides) */
     if ((idx[D] == 0 && P.bcs[D][0] >= 2) || (idx[D] == P.n[D] && P.bcs[D][1] >= 2))
         F[0] = F[NV - 1] = Ft[0] = Ft[NV - 1] = R(0);
-    if constexpr (FSUM) {
-        /* step path in FP32: sum the face's NG Gauss points (the NG warps of
-         * its group, through shared memory; every thread of the block takes
-         * part) in the order (F0 + F1) [+ (F2 + F3)], and store one value per
-         * face and quantity, ff[q][v][face] (q = F, dF/dt, W(dt/2)) */
-        static_assert(gfast, "face sums need the warp-group mapping");
-        static_assert(3 * NV * 128 <= 2 * NVC * FB, "the face sums fit in the staging buffer");
-        R(*xs)[128] = reinterpret_cast<R(*)[128]>(stage);
-        const int lt = threadIdx.x;
-        __syncthreads(); /* every thread has read its coefficients */
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            xs[v][lt] = F[v];
-            xs[NV + v][lt] = Ft[v];
-            xs[2 * NV + v][lt] = Wh[v];
+    for (int v = 0; v < NV; ++v) {
+        int fv = v;
+        if (v >= 1 && v <= M) {
+#pragma unroll
+            for (int kk = 0; kk < M; ++kk)
+                if (ax[kk] == v - 1) fv = 1 + kk;
         }
-        __syncthreads();
-        const int l0 = lt - g * 32; /* this face's Gauss point 0 */
-#pragma unroll
-        for (int q = 0; q < 3 * NV; ++q) {
-            R a = xs[q][l0] + xs[q][l0 + 32];
-            if constexpr (NG == 4) a = a + (xs[q][l0 + 64] + xs[q][l0 + 96]);
-            if (q < NV) F[q] = a;
-            else if (q < 2 * NV) Ft[q - NV] = a;
-            else Wh[q - 2 * NV] = a;
-        }
-        __syncthreads();
-        if (g == 0 && valid) {
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                int fv = v;
-                if (v >= 1 && v <= M) {
-#pragma unroll
-                    for (int kk = 0; kk < M; ++kk)
-                        if (ax[kk] == v - 1) fv = 1 + kk;
-                }
-                ff[(long)(0 * NV + v) * nft + face] = F[fv];
-                ff[(long)(1 * NV + v) * nft + face] = Ft[fv];
-                ff[(long)(2 * NV + v) * nft + face] = Wh[fv];
-            }
-        }
-    } else {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            int fv = v;
-            if (v >= 1 && v <= M) {
-#pragma unroll
-                for (int kk = 0; kk < M; ++kk)
-                    if (ax[kk] == v - 1) fv = 1 + kk;
-            }
-            if (!valid) continue;
-            ff[((long)(0 * NV + v) * NG + g) * nft + face] = F[fv];
-            ff[((long)(1 * NV + v) * NG + g) * nft + face] = Ft[fv];
-            ff[((long)(2 * NV + v) * NG + g) * nft + face] = Wh[fv];
-        }
+        if (!valid) continue;
+        ff[((long)(0 * NV + v) * NG + g) * nft + face] = F[fv];
+        ff[((long)(1 * NV + v) * NG + g) * nft + face] = Ft[fv];
+        ff[((long)(2 * NV + v) * NG + g) * nft + face] = Wh[fv];
     }
 }
 
@@ -1001,7 +956,7 @@ template <typename R, int M, bool NS> constexpr int flux_blocks_per_sm()
     return sizeof(R) == sizeof(float) ? (NS ? 5 : (M == 2 ? 8 : 7)) : 1;
 }
 
-template <typename R, int M, int D, bool FLUX, bool NS = false, bool FSUM = false>
+template <typename R, int M, int D, bool FLUX, bool NS = false>
 __global__ void __launch_bounds__(128, (flux_blocks_per_sm<R, M, NS>())) face_flux_kernel(KP P, Src<R> src, const R *__restrict__ B,
                                                         const double *__restrict__ dtp, double *__restrict__ fs,
                                                         R *__restrict__ ff, int *__restrict__ status)
@@ -1009,11 +964,11 @@ __global__ void __launch_bounds__(128, (flux_blocks_per_sm<R, M, NS>())) face_fl
     constexpr int NG = (M == 2) ? 2 : 4;
     /* 128 threads per block.  FP32: the grid covers whole 128-item groups
      * (ceil(nface / (128 / NG)) blocks) and every thread runs the item, which
-     * masks the items past the last face (its face sums synchronise the
+     * masks the items past the last face (its staged copies synchronise the
      * block).  FP64: one thread per (face, Gauss point). */
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (sizeof(R) == sizeof(float) || t < P.nface[D] * NG)
-        face_flux_item<R, M, D, FLUX, NS, FSUM>(P, src, B, FLUX ? dtp[0] : 0.0, fs, ff, status, t);
+        face_flux_item<R, M, D, FLUX, NS>(P, src, B, FLUX ? dtp[0] : 0.0, fs, ff, status, t);
 }
 
 /* Shared-memory carveout of a kernel with static shared memory: the smallest
@@ -1040,9 +995,9 @@ template <typename K> inline void smem_carveout_for(K kernel, int blocks)
 }
 
 /* once per instantiation, before its first launch */
-template <typename R, int M, int D, bool FLUX, bool NS = false, bool FSUM = false> inline void face_flux_prepare()
+template <typename R, int M, int D, bool FLUX, bool NS = false> inline void face_flux_prepare()
 {
-    static const bool done = (smem_carveout_for(face_flux_kernel<R, M, D, FLUX, NS, FSUM>, flux_blocks_per_sm<R, M, NS>()), true);
+    static const bool done = (smem_carveout_for(face_flux_kernel<R, M, D, FLUX, NS>, flux_blocks_per_sm<R, M, NS>()), true);
     (void)done;
 }
 

@@ -17,60 +17,6 @@ template <> inline Src<float> stage_src<float>(gks_ctx *c, int input)
     return Src<float>{s.hi, s.lo, s.g};
 }
 
-/* flux = false: interface states into fs_dev; flux = true: fluxes per Gauss
- * point into c->ff */
-template <typename R, int M> static cudaError_t flux_impl(gks_ctx *c, int input, double *fs_dev, bool flux)
-{
-    const KP &P = c->kp;
-    R *ff = (R *)c->ff;
-    const double *W = input ? c->Ws : c->W;
-    const double *G = input ? c->Gs : c->G;
-    if constexpr (M == 1) {
-        if (c->order != 8) return nc_launch_faces(c, input, fs_dev, flux);
-        const unsigned nb = blocks_for(P.n[0] + 1, 32);
-        ProfScope ps(c, GKS_KC_FACE);
-        if (flux && P.fp.mu > 0.0) face1d_kernel<R, true, true><<<nb, 32, 0, c->stream>>>(P, W, G, c->dt, nullptr, ff, c->status);
-        else if (flux) face1d_kernel<R, true><<<nb, 32, 0, c->stream>>>(P, W, G, c->dt, nullptr, ff, c->status);
-        else face1d_kernel<R, false><<<nb, 32, 0, c->stream>>>(P, W, G, c->dt, fs_dev, nullptr, c->status);
-    } else {
-        constexpr int NG = (M == 2) ? 2 : 4;
-        R *B = (R *)c->B;
-        const Src<R> src = stage_src<R>(c, input);
-        {
-            ProfScope ps(c, GKS_KC_RECON);
-            cell_poly_kernel<R, M><<<blocks_for(P.next), kBlock, 0, c->stream>>>(P, src, B);
-        }
-        for (int d = 0; d < M; ++d) {
-            const unsigned nb = blocks_for(P.nface[d] * NG);
-            ProfScope ps(c, GKS_KC_FACE);
-#define GKS_FACE(D)                                                                                           \
-    if (d == D) {                                                                                             \
-        if (!flux) { face_flux_prepare<R, M, D, false>(); face_flux_kernel<R, M, D, false><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, fs_dev, nullptr, c->status); } \
-        else if (P.fp.mu > 0.0) { face_flux_prepare<R, M, D, true, true>(); face_flux_kernel<R, M, D, true, true><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, nullptr, ff, c->status); } \
-        else { face_flux_prepare<R, M, D, true>(); face_flux_kernel<R, M, D, true><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, nullptr, ff, c->status); } \
-    }
-            GKS_FACE(0)
-            GKS_FACE(1)
-            if constexpr (M == 3) { GKS_FACE(2) }
-#undef GKS_FACE
-        }
-    }
-    return cudaGetLastError();
-}
-
-template <typename R, int M, bool NS, bool SPLIT> static cudaError_t step_flux_launch(gks_ctx *c)
-{
-    const KP &P = c->kp;
-    constexpr int BT = kStepFluxBlock, FB = SPLIT ? BT / (M == 3 ? 4 : 2) : BT;
-    static const bool prep = SPLIT || (smem_carveout_for(step_flux_kernel<R, M, NS, SPLIT>, kStepFluxMinBlocks<R, M, NS>), true);
-    (void)prep;
-    const unsigned nb0 = blocks_for(P.nface[0], FB), nb1 = nb0 + blocks_for(P.nface[1], FB);
-    const unsigned nb = M == 3 ? nb1 + blocks_for(P.nface[2], FB) : nb1;
-    ProfScope ps(c, GKS_KC_FACE);
-    launch_chained(step_flux_kernel<R, M, NS, SPLIT>, nb, BT, c->stream, P, (const R *)c->B, c->dt, (R *)c->ff, c->status, nb0, nb1);
-    return cudaGetLastError();
-}
-
 inline int sm_count()
 {
     int dev = 0, n = 0;
@@ -95,8 +41,55 @@ template <typename R, int M> inline bool spread_cells(unsigned blocks)
 }
 template <typename R> inline bool split_faces(unsigned blocks) { return blocks <= (sizeof(R) == sizeof(double) ? 3 : 12) * sm_count(); }
 
-/* the multi-D step path: reconstruction and face sums (step_flux.cuh) */
-template <typename R, int M, bool NS> static cudaError_t step_flux_impl(gks_ctx *c, int input)
+/* interface states into fs_dev */
+template <typename R, int M> static cudaError_t states_impl(gks_ctx *c, int input, double *fs_dev)
+{
+    const KP &P = c->kp;
+    if constexpr (M == 1) {
+        if (c->order != 8) return nc_launch_faces(c, input, fs_dev, false);
+        ProfScope ps(c, GKS_KC_FACE);
+        face1d_kernel<R, false><<<blocks_for(P.n[0] + 1, 32), 32, 0, c->stream>>>(P, input ? c->Ws : c->W, input ? c->Gs : c->G, c->dt, fs_dev, nullptr, c->status);
+    } else {
+        constexpr int NG = (M == 2) ? 2 : 4;
+        R *B = (R *)c->B;
+        const Src<R> src = stage_src<R>(c, input);
+        {
+            ProfScope ps(c, GKS_KC_RECON);
+            cell_poly_kernel<R, M><<<blocks_for(P.next), kBlock, 0, c->stream>>>(P, src, B);
+        }
+        for (int d = 0; d < M; ++d) {
+            const unsigned nb = blocks_for(P.nface[d] * NG);
+            ProfScope ps(c, GKS_KC_FACE);
+#define GKS_FACE(D)                                                                                           \
+    if (d == D) {                                                                                             \
+        face_flux_prepare<R, M, D, false>();                                                                  \
+        face_flux_kernel<R, M, D, false><<<nb, kBlock, 0, c->stream>>>(P, src, B, c->dt, fs_dev, nullptr, c->status); \
+    }
+            GKS_FACE(0)
+            GKS_FACE(1)
+            if constexpr (M == 3) { GKS_FACE(2) }
+#undef GKS_FACE
+        }
+    }
+    return cudaGetLastError();
+}
+
+template <typename R, int M, bool NS, bool SPLIT, bool POINTS> static cudaError_t face_flux_launch(gks_ctx *c)
+{
+    const KP &P = c->kp;
+    constexpr int BT = kStepFluxBlock, FB = SPLIT ? BT / (M == 3 ? 4 : 2) : BT;
+    static const bool prep = SPLIT || (smem_carveout_for(step_flux_kernel<R, M, NS, SPLIT, POINTS>, kStepFluxMinBlocks<R, M, NS>), true);
+    (void)prep;
+    const unsigned nb0 = blocks_for(P.nface[0], FB), nb1 = nb0 + blocks_for(P.nface[1], FB);
+    const unsigned nb = M == 3 ? nb1 + blocks_for(P.nface[2], FB) : nb1;
+    ProfScope ps(c, GKS_KC_FACE);
+    launch_chained(step_flux_kernel<R, M, NS, SPLIT, POINTS>, nb, BT, c->stream, P, (const R *)c->B, c->dt, (R *)c->ff, c->status, nb0, nb1);
+    return cudaGetLastError();
+}
+
+/* reconstruction and face fluxes (step_flux.cuh): summed over the Gauss points
+ * (the step), or per point (gks_flux) */
+template <typename R, int M, bool NS, bool POINTS> static cudaError_t flux_impl(gks_ctx *c, int input)
 {
     const KP &P = c->kp;
     R *B = (R *)c->B;
@@ -106,22 +99,36 @@ template <typename R, int M, bool NS> static cudaError_t step_flux_impl(gks_ctx 
         if (spread_cells<R, M>(nb)) launch_chained(cell_poly_kernel<R, M, true, true>, dim3(nb, M + 2), kBlock, c->stream, P, stage_src<R>(c, input), B);
         else launch_chained(cell_poly_kernel<R, M, true>, nb, kBlock, c->stream, P, stage_src<R>(c, input), B);
     }
-    return split_faces<R>(blocks_for(P.nftot, kStepFluxBlock)) ? step_flux_launch<R, M, NS, true>(c) : step_flux_launch<R, M, NS, false>(c);
+    return split_faces<R>(blocks_for(P.nftot, kStepFluxBlock)) ? face_flux_launch<R, M, NS, true, POINTS>(c)
+                                                            : face_flux_launch<R, M, NS, false, POINTS>(c);
 }
 
 template <int M> cudaError_t launch_states(gks_ctx *c, int input, double *fs_dev)
 {
-    return c->precision ? flux_impl<float, M>(c, input, fs_dev, false) : flux_impl<double, M>(c, input, fs_dev, false);
+    return c->precision ? states_impl<float, M>(c, input, fs_dev) : states_impl<double, M>(c, input, fs_dev);
+}
+
+template <typename R, int M> static cudaError_t flux_of(gks_ctx *c, int input, bool sums)
+{
+    const KP &P = c->kp;
+    const bool ns = P.fp.mu > 0.0;
+    if constexpr (M == 1) {
+        if (c->order != 8) return nc_launch_faces(c, input, nullptr, true);
+        const unsigned nb = blocks_for(P.n[0] + 1, 32);
+        const double *W = input ? c->Ws : c->W, *G = input ? c->Gs : c->G;
+        ProfScope ps(c, GKS_KC_FACE);
+        if (ns) face1d_kernel<R, true, true><<<nb, 32, 0, c->stream>>>(P, W, G, c->dt, nullptr, (R *)c->ff, c->status);
+        else face1d_kernel<R, true><<<nb, 32, 0, c->stream>>>(P, W, G, c->dt, nullptr, (R *)c->ff, c->status);
+        return cudaGetLastError();
+    } else {
+        if (sums) return ns ? flux_impl<R, M, true, false>(c, input) : flux_impl<R, M, false, false>(c, input);
+        return ns ? flux_impl<R, M, true, true>(c, input) : flux_impl<R, M, false, true>(c, input);
+    }
 }
 
 template <int M> cudaError_t launch_flux(gks_ctx *c, int input, bool sums)
 {
-    if constexpr (M >= 2) {
-        const bool ns = c->kp.fp.mu > 0.0;
-        if (sums && c->precision) return ns ? step_flux_impl<float, M, true>(c, input) : step_flux_impl<float, M, false>(c, input);
-        if (sums) return ns ? step_flux_impl<double, M, true>(c, input) : step_flux_impl<double, M, false>(c, input);
-    }
-    return c->precision ? flux_impl<float, M>(c, input, nullptr, true) : flux_impl<double, M>(c, input, nullptr, true);
+    return c->precision ? flux_of<float, M>(c, input, sums) : flux_of<double, M>(c, input, sums);
 }
 
 template <typename R, int M, int STAGE, bool SPEED> static void update_launch(gks_ctx *c, unsigned long long *smax)

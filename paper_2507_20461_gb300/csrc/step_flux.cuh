@@ -218,8 +218,10 @@ __device__ __forceinline__ bool face_point(const FluxParams &fp, R adm, R dt, R 
  * thread's first shared slot, SS the slot stride.
  * SPLIT: each of 2 (3D: 4) neighbouring lanes takes one Gauss point of the face,
  * all lanes of the warp call it, and the sums go over shuffles (no stash); lanes
- * past the last face pass it again with store = false. */
-template <typename R, int M, int D, bool NS, int SS, bool SPLIT = false>
+ * past the last face pass it again with store = false.
+ * POINTS: the fluxes of every Gauss point into ff[q][v][g][face] (gks_flux)
+ * instead of their sums. */
+template <typename R, int M, int D, bool NS, int SS, bool SPLIT = false, bool POINTS = false>
 __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict__ B, R dt, R idt, R *__restrict__ ff,
                                                int *__restrict__ status, unsigned fl, typename FaceV<R>::V *stash, bool store = true)
 {
@@ -243,6 +245,9 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
     R F[NV], Ft[NV], Wh[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) F[v] = Ft[v] = Wh[v] = R(0);
+    /* walls (slip or no-slip) are at rest and adiabatic: neither mass nor
+     * energy crosses them (exactly, whatever the rounding of the two sides) */
+    const bool wall = (idx[D] == 0 && P.bcs[D][0] >= 2) || (idx[D] == P.n[D] && P.bcs[D][1] >= 2);
     bool bad = false;
     constexpr int NG = M == 3 ? 4 : 2;
     const int point = SPLIT ? (int)(threadIdx.x % NG) : 0; /* SPLIT: this lane's Gauss point */
@@ -304,7 +309,20 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
             };
             R f[NV], ft[NV], wh[NV];
             const bool ok = face_point<R, M, NS>(P.fp, adm, dt, idt, ih, W, dW, rc, dpc, average, f, ft, wh);
-            if (ok) {
+            if constexpr (POINTS) {
+                const int point_at = SPLIT ? point : p + 2 * b;
+                if (store) {
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) {
+                        const int gv = (v >= 1 && v <= M) ? 1 + ax[v - 1] : v;
+                        const bool none = !ok || (wall && (v == 0 || v == NV - 1));
+                        R *o = ff + ((long)gv * NG + point_at) * P.nftot + (unsigned)P.foff[D] + fl;
+                        o[0] = none ? R(0) : f[v];
+                        o[(long)NV * NG * P.nftot] = none ? R(0) : ft[v];
+                        o[2l * NV * NG * P.nftot] = ok ? wh[v] : R(0);
+                    }
+                }
+            } else if (ok) {
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
                     F[v] += f[v];
@@ -316,6 +334,7 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
         }
     }
     if (bad) atomicOr(status, ST_FLUX);
+    if constexpr (POINTS) return;
     if constexpr (SPLIT) {
 #pragma unroll
         for (int o = 1; o < NG; o <<= 1)
@@ -327,9 +346,7 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
             }
         if (!store || point != 0) return;
     }
-    /* walls (slip or no-slip) are at rest and adiabatic: neither mass nor
-     * energy crosses them (exactly, whatever the rounding of the two sides) */
-    if ((idx[D] == 0 && P.bcs[D][0] >= 2) || (idx[D] == P.n[D] && P.bcs[D][1] >= 2))
+    if (wall)
         F[0] = F[NV - 1] = Ft[0] = Ft[NV - 1] = R(0);
     R *o = ff + group_off<kFaceFields<M>>((unsigned)P.foff[D] + fl);
 #pragma unroll
@@ -356,7 +373,7 @@ template <typename R, int M, bool NS>
 constexpr int kStepFluxMinBlocks = sizeof(R) == sizeof(float) ? (M == 2 && !NS ? 12 : 8) : (M == 2 ? 6 : 4);
 
 /* SPLIT: a lane per Gauss point, 64 / NG faces a block */
-template <typename R, int M, bool NS, bool SPLIT>
+template <typename R, int M, bool NS, bool SPLIT, bool POINTS = false>
 __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, M, NS>))
     step_flux_kernel(KP P, const R *__restrict__ B, const double *__restrict__ dtp, R *__restrict__ ff,
                      int *__restrict__ status, unsigned nb0, unsigned nb1)
@@ -370,8 +387,8 @@ __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, M, NS>)
     auto face = [&](auto dir, unsigned block) {
         constexpr int D = decltype(dir)::value;
         const unsigned fl = block * FB + threadIdx.x / PER, n = (unsigned)P.nface[D];
-        if constexpr (SPLIT) step_face_item<R, M, D, NS, BT, true>(P, B, dt, idt, ff, status, fl < n ? fl : n - 1, stash, fl < n);
-        else if (fl < n) step_face_item<R, M, D, NS, BT>(P, B, dt, idt, ff, status, fl, stash);
+        if constexpr (SPLIT) step_face_item<R, M, D, NS, BT, true, POINTS>(P, B, dt, idt, ff, status, fl < n ? fl : n - 1, stash, fl < n);
+        else if (fl < n) step_face_item<R, M, D, NS, BT, false, POINTS>(P, B, dt, idt, ff, status, fl, stash);
     };
     if (b < nb0) face(std::integral_constant<int, 0>{}, b);
     else if (M == 2 || b < nb1) face(std::integral_constant<int, 1>{}, b - nb0);
