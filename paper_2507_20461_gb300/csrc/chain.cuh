@@ -41,6 +41,11 @@ template <typename T> __device__ __forceinline__ T load_ro(const T *p)
 #endif
 }
 
+/* Blocks from the last to the first (rev) or in order: the kernels of a step
+ * alternate, so each begins with what the one before it wrote last, which L2
+ * still holds. */
+__device__ __forceinline__ unsigned block_in_order(bool rev) { return rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x; }
+
 #ifdef __CUDACC__
 template <typename... K, typename... A>
 cudaError_t launch_chained(void (*kernel)(K...), dim3 blocks, unsigned threads, cudaStream_t stream, A... args)

@@ -107,7 +107,8 @@ template <typename R>
 __global__ void __launch_bounds__(128) bk_poly(const KP common, const GridDesc *__restrict__ gd,
                                                const Tile *__restrict__ tiles, int stage)
 {
-    const Tile T = tiles[blockIdx.x];
+    after_previous();
+    const Tile T = tiles[block_in_order(stage == 2)];
     const GridDesc &g = gd[T.grid_kind >> 1];
     const KP P = grid_kp(common, g.P);
     const unsigned t = T.begin + threadIdx.x;
@@ -118,11 +119,12 @@ __global__ void __launch_bounds__(128) bk_poly(const KP common, const GridDesc *
 template <typename R>
 __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, 2, false>))
     bk_flux(const KP common, const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles,
-            const double *__restrict__ dt, int *__restrict__ status)
+            const double *__restrict__ dt, int *__restrict__ status, bool rev)
 {
+    after_previous(dt);
     __shared__ typename FaceV<R>::V slots[kFaceStash<R, 2> * kStepFluxBlock];
     typename FaceV<R>::V *stash = slots + threadIdx.x;
-    const Tile T = tiles[blockIdx.x];
+    const Tile T = tiles[block_in_order(rev)];
     const unsigned grid = T.grid_kind >> 1;
     const GridDesc &g = gd[grid];
     const KP P = grid_kp(common, g.P);
@@ -142,7 +144,8 @@ __global__ void __launch_bounds__(128) bk_update(const KP common, const GridDesc
                                                  const Tile *__restrict__ tiles, const double *__restrict__ dt,
                                                  const float *__restrict__ updc, int *__restrict__ status)
 {
-    const Tile T = tiles[blockIdx.x];
+    after_previous(dt, updc);
+    const Tile T = tiles[block_in_order(STAGE == 2)];
     const unsigned grid = T.grid_kind >> 1;
     const GridDesc &g = gd[grid];
     const KP P = grid_kp(common, g.P);
@@ -162,24 +165,19 @@ template <typename R> cudaError_t batch_speed(const BatchLaunch &L, const Launch
 }
 template <typename R> cudaError_t batch_poly(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
 {
-    bk_poly<R><<<S.blocks, S.block, 0, st>>>(*L.common, L.gd, L.tiles, stage);
-    return cudaGetLastError();
+    return launch_chained(bk_poly<R>, S.blocks, S.block, st, *L.common, L.gd, L.tiles, stage);
 }
 template <typename R> cudaError_t batch_flux(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
 {
     if (S.block != kStepFluxBlock) return cudaErrorInvalidConfiguration;
     static const bool prep = (smem_carveout_for(bk_flux<R>, kStepFluxMinBlocks<R, 2, false>), true);
     (void)prep;
-    bk_flux<R><<<S.blocks, S.block, 0, st>>>(*L.common, L.gd, L.tiles, L.dt, L.status);
-    return cudaGetLastError();
+    return launch_chained(bk_flux<R>, S.blocks, S.block, st, *L.common, L.gd, L.tiles, L.dt, L.status, stage == 1);
 }
 template <typename R> cudaError_t batch_update(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
 {
-    if (stage == 1)
-        bk_update<R, 1><<<S.blocks, S.block, 0, st>>>(*L.common, L.gd, L.tiles, L.dt, L.updc, L.status);
-    else
-        bk_update<R, 2><<<S.blocks, S.block, 0, st>>>(*L.common, L.gd, L.tiles, L.dt, L.updc, L.status);
-    return cudaGetLastError();
+    return launch_chained(stage == 1 ? bk_update<R, 1> : bk_update<R, 2>, S.blocks, S.block, st, *L.common, L.gd, L.tiles, L.dt, L.updc,
+                          L.status);
 }
 cudaError_t batch_shadow(const GridDesc &g, cudaStream_t st)
 {

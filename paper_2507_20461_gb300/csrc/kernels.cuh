@@ -7,15 +7,18 @@
  *   1D   face1d        one thread per face: p^7 on {j-1..j+2} (shared by both
  *                      sides), the three sub-stencil quadratics of each side,
  *                      GENO blend, admissibility fallback, GKS flux.
- *   M-D  cell_poly     one thread per cell (plus the ghost ring): least-squares
- *                      cubic, linear sub-polynomials, GENO blend -> blended
- *                      cubic coefficients B[v][k].
- *        face_flux     one thread per (face, Gauss point) of one direction:
- *                      both interface states from B, admissibility fallback,
- *                      GKS flux, F / dF/dt / W(dt/2) to the face arrays.
- *   all  update        one thread per cell: FP64 two-stage update of the
+ *   M-D  cell_poly     one thread per cell (plus the ghost ring), or per cell and
+ *                      variable: least-squares cubic, linear sub-polynomials,
+ *                      GENO blend -> blended cubic coefficients B.
+ *        step_flux     one thread per face (step_flux.cuh): interface states
+ *                      from B, admissibility fallback, GKS flux, F / dF/dt /
+ *                      W(dt/2) to the face arrays.  face_flux: one thread per
+ *                      (face, Gauss point) of one direction, for the interface
+ *                      states and gks_flux_2d_static.
+ *        step_update   one thread per cell: FP64 two-stage update of the
  *                      averages (Eq. semifvs) and of the averaged gradients by
  *                      the Gauss theorem (Eq. slope).
+ *   The 1D step path is step_1d.cuh and k1d_nc.cu: a stage in one kernel.
  * Ghost cells are index mappings (periodic wrap, or transmissive even
  * extension with the normal derivative negated); no padded copies exist.
  */
@@ -748,10 +751,10 @@ __device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R
 }
 
 template <typename R, int M, bool GROUPED = false, bool SPREAD = false>
-__global__ void __launch_bounds__(128) cell_poly_kernel(KP P, Src<R> src, R *__restrict__ B)
+__global__ void __launch_bounds__(128) cell_poly_kernel(KP P, Src<R> src, R *__restrict__ B, bool rev = false)
 {
     after_previous();
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long t = (long)block_in_order(rev) * blockDim.x + threadIdx.x;
     if (t < P.next) cell_poly_item<R, M, GROUPED, SPREAD>(P, src, B, t, (int)blockIdx.y);
 }
 
@@ -1071,8 +1074,7 @@ __device__ __forceinline__ UpdC make_updc(double dt, double cw)
 /* The stage constants live in a 10-float device buffer, written once per
  * time step by the kernel that sets dt, so the update kernel (one cell per
  * thread) neither recomputes them per block in FP64 nor waits on a barrier
- * for them.  The fused stage kernels compute them once per strip, which
- * their rows amortise. */
+ * for them. */
 __device__ __forceinline__ void store_updc(float *p, const UpdC &u)
 {
 #pragma unroll

@@ -37,9 +37,9 @@ inline int sm_count()
  *     26^3 1360 / 1110, 1360 / 1507; 64 x 50^2 (9.2, 50) 8451 / 8354. */
 template <typename R, int M> inline bool spread_cells(unsigned blocks)
 {
-    return blocks <= (sizeof(R) == sizeof(double) ? 10 : (M == 2 ? 6 : 3)) * sm_count();
+    return blocks <= (unsigned)((sizeof(R) == sizeof(double) ? 10 : (M == 2 ? 6 : 3)) * sm_count());
 }
-template <typename R> inline bool split_faces(unsigned blocks) { return blocks <= (sizeof(R) == sizeof(double) ? 3 : 12) * sm_count(); }
+template <typename R> inline bool split_faces(unsigned blocks) { return blocks <= (unsigned)((sizeof(R) == sizeof(double) ? 3 : 12) * sm_count()); }
 
 /* interface states into fs_dev */
 template <typename R, int M> static cudaError_t states_impl(gks_ctx *c, int input, double *fs_dev)
@@ -74,16 +74,21 @@ template <typename R, int M> static cudaError_t states_impl(gks_ctx *c, int inpu
     return cudaGetLastError();
 }
 
-template <typename R, int M, bool NS, bool SPLIT, bool POINTS> static cudaError_t face_flux_launch(gks_ctx *c)
+template <typename R, int M, bool NS, bool SPLIT, bool POINTS> static cudaError_t face_flux_launch(gks_ctx *c, int input)
 {
     const KP &P = c->kp;
     constexpr int BT = kStepFluxBlock, FB = SPLIT ? BT / (M == 3 ? 4 : 2) : BT;
     static const bool prep = SPLIT || (smem_carveout_for(step_flux_kernel<R, M, NS, SPLIT, POINTS>, kStepFluxMinBlocks<R, M, NS>), true);
     (void)prep;
-    const unsigned nb0 = blocks_for(P.nface[0], FB), nb1 = nb0 + blocks_for(P.nface[1], FB);
-    const unsigned nb = M == 3 ? nb1 + blocks_for(P.nface[2], FB) : nb1;
+    unsigned nb[3], total = 0, runs = M == 2 ? ~0u : 0u;
+    for (int d = 0; d < M; ++d) {
+        nb[d] = blocks_for(P.nface[d], FB);
+        total += nb[d];
+        if (nb[d] / kFaceRun < runs) runs = nb[d] / kFaceRun;
+    }
+    const FaceOrder order{runs, {nb[0] - runs * kFaceRun, nb[1] - runs * kFaceRun}};
     ProfScope ps(c, GKS_KC_FACE);
-    launch_chained(step_flux_kernel<R, M, NS, SPLIT, POINTS>, nb, BT, c->stream, P, (const R *)c->B, c->dt, (R *)c->ff, c->status, nb0, nb1);
+    launch_chained(step_flux_kernel<R, M, NS, SPLIT, POINTS>, total, BT, c->stream, P, (const R *)c->B, c->dt, (R *)c->ff, c->status, order, input == 0);
     return cudaGetLastError();
 }
 
@@ -96,11 +101,13 @@ template <typename R, int M, bool NS, bool POINTS> static cudaError_t flux_impl(
     {
         ProfScope ps(c, GKS_KC_RECON);
         const unsigned nb = blocks_for(P.next);
-        if (spread_cells<R, M>(nb)) launch_chained(cell_poly_kernel<R, M, true, true>, dim3(nb, M + 2), kBlock, c->stream, P, stage_src<R>(c, input), B);
-        else launch_chained(cell_poly_kernel<R, M, true>, nb, kBlock, c->stream, P, stage_src<R>(c, input), B);
+        if (spread_cells<R, M>(nb))
+            launch_chained(cell_poly_kernel<R, M, true, true>, dim3(nb, M + 2), kBlock, c->stream, P, stage_src<R>(c, input), B, input != 0);
+        else
+            launch_chained(cell_poly_kernel<R, M, true>, nb, kBlock, c->stream, P, stage_src<R>(c, input), B, input != 0);
     }
-    return split_faces<R>(blocks_for(P.nftot, kStepFluxBlock)) ? face_flux_launch<R, M, NS, true, POINTS>(c)
-                                                            : face_flux_launch<R, M, NS, false, POINTS>(c);
+    return split_faces<R>(blocks_for(P.nftot, kStepFluxBlock)) ? face_flux_launch<R, M, NS, true, POINTS>(c, input)
+                                                            : face_flux_launch<R, M, NS, false, POINTS>(c, input);
 }
 
 template <int M> cudaError_t launch_states(gks_ctx *c, int input, double *fs_dev)
@@ -133,7 +140,7 @@ template <int M> cudaError_t launch_flux(gks_ctx *c, int input, bool sums)
 
 template <typename R, int M, int STAGE, bool SPEED> static void update_launch(gks_ctx *c, unsigned long long *smax)
 {
-    launch_chained(step_update_kernel<R, M, STAGE, SPEED>, blocks_for(c->kp.ncell, 256), 256, c->stream, c->kp, (const R *)c->ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1, c->status, c->updc, smax);
+    launch_chained(step_update_kernel<R, M, STAGE, SPEED>, blocks_for(c->kp.ncell, 256), 256, c->stream, c->kp, (const R *)c->ff, c->dt, c->W, c->G, c->Ws, c->Gs, c->Acc, c->s0, c->s1, c->status, c->updc, smax, STAGE == 2);
 }
 
 template <typename R, int M> static cudaError_t update_impl(gks_ctx *c, int stage, unsigned long long *smax)
