@@ -112,7 +112,9 @@ __global__ void __launch_bounds__(128) bk_poly(const KP common, const GridDesc *
     const GridDesc &g = gd[T.grid_kind >> 1];
     const KP P = grid_kp(common, g.P);
     const unsigned t = T.begin + threadIdx.x;
-    if (t < P.next) cell_poly_item<R, 2, true>(P, stage_src_of<R>(g, stage), (R *)g.B, t);
+    /* FP64: a thread per variable too (spread_cells) */
+    if (t < P.next)
+        cell_poly_item<R, 2, true, sizeof(R) == sizeof(double)>(P, stage_src_of<R>(g, stage), (R *)g.B, t, (int)blockIdx.y);
 }
 
 /* block size and register cap of the single-grid face flux */
@@ -165,7 +167,7 @@ template <typename R> cudaError_t batch_speed(const BatchLaunch &L, const Launch
 }
 template <typename R> cudaError_t batch_poly(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
 {
-    return launch_chained(bk_poly<R>, S.blocks, S.block, st, *L.common, L.gd, L.tiles, stage);
+    return launch_chained(bk_poly<R>, dim3(S.blocks, sizeof(R) == sizeof(double) ? 4 : 1), S.block, st, *L.common, L.gd, L.tiles, stage);
 }
 template <typename R> cudaError_t batch_flux(const BatchLaunch &L, const LaunchShape &S, int stage, cudaStream_t st)
 {

@@ -26,7 +26,8 @@ inline int sm_count()
 /* Small grids, as blocks per SM: a thread per (cell, variable) in the
  * reconstruction, a lane per Gauss point in the flux.  With too few blocks to
  * hide a thread's chain of instructions the work of one is spread over several;
- * past the lines below the repeated index work and evaluations cost more.
+ * past the lines below the repeated index work and evaluations cost more.  The
+ * FP64 reconstruction is always spread: its index work runs beside the FP64 pipe.
  * Measured (GB300, us a step, plain / spread, then plain / split):
  *   FP32 2D: 160^2 (1.4 recon, 5.3 flux blocks per SM) 44.9 / 40.5, 44.9 / 37.2;
  *     224^2 (2.6, 10.4) 47.7 / 45.1, 47.7 / 44.9; 320^2 (5.3, 21) 63.9 / 60.3, 63.7 / 65.1;
@@ -34,10 +35,11 @@ inline int sm_count()
  *   FP32 3D: 26^3 (1.1, 5.6) 88 / 71, 88 / 68; 32^3 (2.0, 10.4) 97 / 93, 97 / 90;
  *     40 x 36^2 (3.1, 16) 117.6 / 117.1, 117.3 / 115.1; 48 x 40^2 (4.5, 24) 139 / 151, 139 / 152;
  *   FP64 2D: 160^2 565 / 454, 565 / 590; 3D: 20^3 (0.6, 2.6) 986 / 669, 986 / 707;
- *     26^3 1360 / 1110, 1360 / 1507; 64 x 50^2 (9.2, 50) 8451 / 8354. */
+ *     26^3 1360 / 1110, 1360 / 1507; 64 x 50^2 (9.2, 50) 8451 / 8354; 512^2 (13.6) 3210 / 3148. */
 template <typename R, int M> inline bool spread_cells(unsigned blocks)
 {
-    return blocks <= (unsigned)((sizeof(R) == sizeof(double) ? 10 : (M == 2 ? 6 : 3)) * sm_count());
+    if constexpr (sizeof(R) == sizeof(double)) return true;
+    else return blocks <= (unsigned)((M == 2 ? 6 : 3) * sm_count());
 }
 template <typename R> inline bool split_faces(unsigned blocks) { return blocks <= (unsigned)((sizeof(R) == sizeof(double) ? 3 : 12) * sm_count()); }
 
@@ -103,7 +105,7 @@ template <typename R, int M, bool NS, bool POINTS> static cudaError_t flux_impl(
         const unsigned nb = blocks_for(P.next);
         if (spread_cells<R, M>(nb))
             launch_chained(cell_poly_kernel<R, M, true, true>, dim3(nb, M + 2), kBlock, c->stream, P, stage_src<R>(c, input), B, input != 0);
-        else
+        else if constexpr (sizeof(R) == sizeof(float))
             launch_chained(cell_poly_kernel<R, M, true>, nb, kBlock, c->stream, P, stage_src<R>(c, input), B, input != 0);
     }
     return split_faces<R>(blocks_for(P.nftot, kStepFluxBlock)) ? face_flux_launch<R, M, NS, true, POINTS>(c, input)

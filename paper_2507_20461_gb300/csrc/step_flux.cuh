@@ -247,7 +247,11 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
     for (int v = 0; v < NV; ++v) F[v] = Ft[v] = Wh[v] = R(0);
     /* walls (slip or no-slip) are at rest and adiabatic: neither mass nor
      * energy crosses them (exactly, whatever the rounding of the two sides) */
-    const bool wall = (idx[D] == 0 && P.bcs[D][0] >= 2) || (idx[D] == P.n[D] && P.bcs[D][1] >= 2);
+    auto wall = [&] { return (idx[D] == 0 && P.bcs[D][0] >= 2) || (idx[D] == P.n[D] && P.bcs[D][1] >= 2); };
+    /* FP32 2D: during the second point the first one's sums wait in the slots
+     * that its values left (80 registers spill 16 bytes instead of 180; in 3D,
+     * where they live through the loop, and in FP64 this added spills) */
+    constexpr bool PARK = G == 1 && M == 2 && !SPLIT && !POINTS;
     bool bad = false;
     constexpr int NG = M == 3 ? 4 : 2;
     const int point = SPLIT ? (int)(threadIdx.x % NG) : 0; /* SPLIT: this lane's Gauss point */
@@ -302,6 +306,13 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
 #pragma unroll
                         for (int e = 0; e < M; ++e) dW[g][e][v] = stash[((g * NV + v) * (M + 1) + 1 + e) * SS];
                     }
+                if constexpr (PARK) {
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) {
+                        stash[3 * v * SS] = V(F[v], Ft[v]);
+                        stash[(3 * v + 1) * SS] = V(Wh[v], 0.f);
+                    }
+                }
             }
             auto average = [&](int g, int v) -> V {
                 const int gv = (v >= 1 && v <= M) ? 1 + ax[v - 1] : v;
@@ -315,19 +326,32 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
 #pragma unroll
                     for (int v = 0; v < NV; ++v) {
                         const int gv = (v >= 1 && v <= M) ? 1 + ax[v - 1] : v;
-                        const bool none = !ok || (wall && (v == 0 || v == NV - 1));
+                        const bool none = !ok || (wall() && (v == 0 || v == NV - 1));
                         R *o = ff + ((long)gv * NG + point_at) * P.nftot + (unsigned)P.foff[D] + fl;
                         o[0] = none ? R(0) : f[v];
                         o[(long)NV * NG * P.nftot] = none ? R(0) : ft[v];
                         o[2l * NV * NG * P.nftot] = ok ? wh[v] : R(0);
                     }
                 }
-            } else if (ok) {
+            } else {
+                if constexpr (PARK) {
+                    if (p) {
 #pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    F[v] += f[v];
-                    Ft[v] += ft[v];
-                    Wh[v] += wh[v];
+                        for (int v = 0; v < NV; ++v) {
+                            const V a = stash[3 * v * SS];
+                            F[v] = a.l();
+                            Ft[v] = a.r();
+                            Wh[v] = stash[(3 * v + 1) * SS].l();
+                        }
+                    }
+                }
+                if (ok) {
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) {
+                        F[v] += f[v];
+                        Ft[v] += ft[v];
+                        Wh[v] += wh[v];
+                    }
                 }
             }
             bad = bad || !ok;
@@ -346,8 +370,7 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
             }
         if (!store || point != 0) return;
     }
-    if (wall)
-        F[0] = F[NV - 1] = Ft[0] = Ft[NV - 1] = R(0);
+    if (wall()) F[0] = F[NV - 1] = Ft[0] = Ft[NV - 1] = R(0);
     R *o = ff + group_off<kFaceFields<M>>((unsigned)P.foff[D] + fl);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -367,10 +390,12 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
  * 256^3 launch; 6 and 10 blocks 9.7 and 10.0), Navier-Stokes 8 (0.203 ms per
  * 99 x 64 x 50 launch; 10 blocks 0.25).  The points of a pair are
  * unrolled: as a loop the packed constants stay in registers across it (2D
- * 0.54, 3D 9.0 ms).  FP64 is bound by its pipe: 4 to 6 blocks are equal. */
+ * 0.54, 3D 9.0 ms).  FP64 is bound by its pipe: 4 to 6 blocks are equal, but
+ * for spills (2D Navier-Stokes 4 blocks, 174 registers; 5 and 6 both cap at 168
+ * and spill 190 bytes, as warps come in fours). */
 constexpr int kStepFluxBlock = 64;
 template <typename R, int M, bool NS>
-constexpr int kStepFluxMinBlocks = sizeof(R) == sizeof(float) ? (M == 2 && !NS ? 12 : 8) : (M == 2 ? 6 : 4);
+constexpr int kStepFluxMinBlocks = sizeof(R) == sizeof(float) ? (M == 2 && !NS ? 12 : 8) : (M == 2 && !NS ? 6 : 4);
 
 /* The order of the flux blocks.  2D: runs of kFaceRun blocks of one direction,
  * then the same run of the other, which finds its cells' records in L2 (2048
