@@ -9,6 +9,8 @@
  * no kernel reads or writes memory before everything earlier in the stream is
  * complete (each waits for its predecessor, which waited for its own), and the
  * order is that of ordinary launches.
+ * GB300, a pass, plain / chained: 4 steps of 64^2 mixed 245 / 178 us, 20 steps of
+ * 400 cells 1055 / 964 us, 2 steps of 2048^2 3.97 / 3.92 ms, 256^3 equal.
  */
 #pragma once
 #include <cuda_runtime.h>
@@ -30,8 +32,8 @@ template <typename... T> __device__ __forceinline__ void after_previous(T &...p)
 /* A load of data that the kernel does not write, through a pointer that has
  * passed after_previous (and so lost its __restrict__): the compiler may move it
  * past the kernel's stores.  The update with plain loads instead, each
- * variable's waiting for the last one's stores: 204 us a 2048^2 stage for 172,
- * 1.33 ms at 256^3 for 1.06. */
+ * variable's waiting for the last one's stores: 204 us a 2048^2 stage for 176,
+ * 1.33 ms at 256^3 for 1.14. */
 template <typename T> __device__ __forceinline__ T load_ro(const T *p)
 {
 #ifdef __CUDA_ARCH__
@@ -43,7 +45,7 @@ template <typename T> __device__ __forceinline__ T load_ro(const T *p)
 
 /* Blocks from the last to the first (rev) or in order: the kernels of a step
  * alternate, so each begins with what the one before it wrote last, which L2
- * still holds. */
+ * still holds (99 x 64 x 50 viscous 1246 to 1218 us a pass, 256^3 24.57 to 24.51 ms). */
 __device__ __forceinline__ unsigned block_in_order(bool rev) { return rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x; }
 
 #ifdef __CUDACC__

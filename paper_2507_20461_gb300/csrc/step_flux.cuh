@@ -19,7 +19,8 @@
  * cp.async and the sums exchanged through shared memory, one launch per
  * direction (GB300): 2048^2 mixed 0.77 to 0.48 ms a stage, 256^3 mixed 16.9
  * to 8.0 ms, 99 x 64 x 50 Navier-Stokes 0.39 to 0.20 ms, FP64 512^2 1.87 to
- * 1.50 ms.
+ * 1.50 ms (0.45, 7.9, 0.20 and 1.26 ms with the flux arithmetic, slots and block
+ * order of now).
  *
  * Layouts (step path only): groups of 32 consecutive extended cells, or faces,
  * with the record fields of a group in rows of 32, so that every field of an
