@@ -71,15 +71,14 @@ CELL_UPDATE_2D_LIMITER = {lim: CELL_UPDATE_2D + 2 * 4 * (_flops(f"cubic_cell_var
 # 1D non-compact GENO + HLLC, one classical RK4 step (4 stages)
 NC_CELL_UPDATE = {o: _flops(f"nc_step_cell_update_1d_order{o}") for o in (5, 6)}
 # Executed flops of the face-flux kernel itself (ncu: 2 x FMA + ADD + MUL of
-# the pipe, scalar and packed two-lane forms, per face Gauss point, on a 256^2 case whose index space is whole
-# 128-item groups, so every point is evaluated exactly once; mean of the four
-# launches of a step; the face-flux flop summary under profiles/).  The
-# kernel uses closed forms where the oracle solves moment systems, so it
-# executes fewer flops than the algorithmic count.
-EXECUTED_FLOPS_PER_FACE_GP = {"mixed": None, "fp64": None}
-# DRAM bytes (read + write) per launch of the face-flux kernel at 2048^2, from
-# a 1-pass ncu capture (None: not captured for the current kernel).
-TRAFFIC_PER_FLUX_LAUNCH = {"mixed": None, "fp64": None}
+# the pipe, scalar and packed two-lane forms, per face Gauss point, 256^2; the
+# step kernels' summary under profiles/).  The kernel uses closed forms where
+# the oracle solves moment systems, so it executes fewer flops than the
+# algorithmic count.
+EXECUTED_FLOPS_PER_FACE_GP = {"mixed": 972.0, "fp64": 988.0}
+# DRAM bytes (read + write) per launch of the face-flux kernel at 2048^2: a
+# 1-pass ncu capture at 1024^2 scaled by the faces (None: not captured).
+TRAFFIC_PER_FLUX_LAUNCH = {"mixed": 970e6, "fp64": None}
 # Algorithmic HBM bytes per cell-update of the whole step (FP64 state,
 # stage buffers, accumulator), 2D: 60 doubles.
 BYTES_PER_CELL_UPDATE = 480.0
