@@ -18,28 +18,20 @@
 namespace gks {
 
 /* First statement of a kernel that launch_chained starts, before any access to
- * memory.  The pointers of read-only data pass through it so that the compiler
- * cannot move a (non-coherent) load through one of them above the wait. */
-template <typename... T> __device__ __forceinline__ void after_previous(T &...p)
+ * memory.  The kernel is on the SMs while its predecessors, and theirs, still
+ * write.  The wait orders what the compiler must take as touched by it: the
+ * target of a __restrict__ parameter is not, and a load through a const one may
+ * even become non-coherent.  So the pointers of such a kernel carry no
+ * __restrict__, but for what no kernel of the chain writes (a batch's
+ * descriptors and tile lists, uploaded before its first launch), and nothing is
+ * read by __ldg, whose target may not change while the kernel is resident.
+ * Without either a load does not move past a store before it, so the updates
+ * read everything before they store. */
+__device__ __forceinline__ void after_previous()
 {
 #ifdef __CUDA_ARCH__
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    (..., [&] { asm volatile("" : "+l"(p)); }());
-#endif
-}
-
-/* A load of data that the kernel does not write, through a pointer that has
- * passed after_previous (and so lost its __restrict__): the compiler may move it
- * past the kernel's stores.  The update with plain loads instead, each
- * variable's waiting for the last one's stores: 204 us a 2048^2 stage for 176,
- * 1.33 ms at 256^3 for 1.14. */
-template <typename T> __device__ __forceinline__ T load_ro(const T *p)
-{
-#ifdef __CUDA_ARCH__
-    return __ldg(p);
-#else
-    return *p;
 #endif
 }
 

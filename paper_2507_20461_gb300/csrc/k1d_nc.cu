@@ -190,21 +190,28 @@ __device__ __forceinline__ void nc_update(const KP &P, double dt, const double *
                                           double *__restrict__ Wout, double *__restrict__ Acc, int *__restrict__ status,
                                           long cell, double *out)
 {
+    /* loads before stores (chain.cuh) */
+    double u0[3], acc[3];
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+        u0[v] = W0[v * P.ncell + cell];
+        acc[v] = STAGE == 1 ? 0.0 : Acc[v * P.ncell + cell];
+    }
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
         const double L = -(up[v] - F[v]) * P.ih;
         const long i = (long)v * P.ncell + cell;
         if (STAGE == 1) {
             Acc[i] = L;
-            out[v] = Wout[i] = W0[i] + 0.5 * dt * L;
+            out[v] = Wout[i] = u0[v] + 0.5 * dt * L;
         } else if (STAGE == 2) {
-            Acc[i] += 2.0 * L;
-            out[v] = Wout[i] = W0[i] + 0.5 * dt * L;
+            Acc[i] = acc[v] + 2.0 * L;
+            out[v] = Wout[i] = u0[v] + 0.5 * dt * L;
         } else if (STAGE == 3) {
-            Acc[i] += 2.0 * L;
-            out[v] = Wout[i] = W0[i] + dt * L;
+            Acc[i] = acc[v] + 2.0 * L;
+            out[v] = Wout[i] = u0[v] + dt * L;
         } else {
-            out[v] = W0[i] = W0[i] + dt / 6.0 * (Acc[i] + L);
+            out[v] = W0[i] = u0[v] + dt / 6.0 * (acc[v] + L);
         }
     }
     const double p = P.fp.gm1 * (out[2] - 0.5 * out[1] * out[1] / out[0]);
@@ -223,11 +230,10 @@ __device__ __forceinline__ void nc_update(const KP &P, double dt, const double *
  *   stage 3: Acc += 2 L(U2), U3 = U0 + dt L(U2)
  *   stage 4: U0 += dt/6 (Acc + L(U3)) */
 template <int ORDER, int STAGE>
-__global__ void __launch_bounds__(32) nc_stage_kernel(KP P, const double *__restrict__ Win, double *__restrict__ W0,
-                                                      double *__restrict__ Wout, double *__restrict__ Acc,
-                                                      int *__restrict__ status, StepClock clk)
+__global__ void __launch_bounds__(32) nc_stage_kernel(KP P, const double *Win, double *W0, double *Wout, double *Acc,
+                                                      int *status, StepClock clk)
 {
-    after_previous(Win, clk.dt, clk.in);
+    after_previous();
     const int lane = threadIdx.x, n = P.n[0];
     const int f = min((int)blockIdx.x * kCells1d + lane, n); /* lanes past the last face repeat it */
     const double dt = clock_dt(clk);
@@ -246,11 +252,10 @@ __global__ void __launch_bounds__(32) nc_stage_kernel(KP P, const double *__rest
 /* the same stage for short grids: eight lanes per face, six of them
  * reconstructing one variable of one side each (step_1d.cuh) */
 template <int ORDER, int STAGE>
-__global__ void __launch_bounds__(128) nc_short_kernel(KP P, const double *__restrict__ Win, double *__restrict__ W0,
-                                                       double *__restrict__ Wout, double *__restrict__ Acc,
-                                                       int *__restrict__ status, StepClock clk)
+__global__ void __launch_bounds__(128) nc_short_kernel(KP P, const double *Win, double *W0, double *Wout, double *Acc,
+                                                       int *status, StepClock clk)
 {
-    after_previous(Win, clk.dt, clk.in);
+    after_previous();
     __shared__ double q[kShortFaces][3];
     const int n = P.n[0], sub = threadIdx.x & 7, face = threadIdx.x >> 3;
     const int f = min((int)blockIdx.x * kCellsShort + face, n); /* past the last face: the last face again */

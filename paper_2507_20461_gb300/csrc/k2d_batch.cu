@@ -123,9 +123,9 @@ __global__ void __launch_bounds__(128) bk_poly(const KP common, const GridDesc *
 template <typename R>
 __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, 2, false>))
     bk_flux(const KP common, const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles,
-            const double *__restrict__ dt, int *__restrict__ status, bool rev)
+            const double *dt, int *status, bool rev)
 {
-    after_previous(dt);
+    after_previous();
     __shared__ typename FaceV<R>::V slots[kFaceStash<R, 2> * kStepFluxBlock];
     typename FaceV<R>::V *stash = slots + threadIdx.x;
     const Tile T = tiles[block_in_order(rev)];
@@ -145,10 +145,10 @@ __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, 2, fals
 
 template <typename R, int STAGE>
 __global__ void __launch_bounds__(128) bk_update(const KP common, const GridDesc *__restrict__ gd,
-                                                 const Tile *__restrict__ tiles, const double *__restrict__ dt,
-                                                 const float *__restrict__ updc, int *__restrict__ status)
+                                                 const Tile *__restrict__ tiles, const double *dt,
+                                                 const float *updc, int *status)
 {
-    after_previous(dt, updc);
+    after_previous();
     const Tile T = tiles[block_in_order(STAGE == 2)];
     const unsigned grid = T.grid_kind >> 1;
     const GridDesc &g = gd[grid];

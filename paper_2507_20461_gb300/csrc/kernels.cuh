@@ -751,7 +751,7 @@ __device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R
 }
 
 template <typename R, int M, bool GROUPED = false, bool SPREAD = false>
-__global__ void __launch_bounds__(128) cell_poly_kernel(KP P, Src<R> src, R *__restrict__ B, bool rev = false)
+__global__ void __launch_bounds__(128) cell_poly_kernel(KP P, Src<R> src, R *B, bool rev = false)
 {
     after_previous();
     const long t = (long)block_in_order(rev) * blockDim.x + threadIdx.x;
@@ -1124,17 +1124,25 @@ __device__ __forceinline__ long face_of(const KP &P, int d, int i, int j, int k,
  * and re-splits W into s0, so the shadow never drifts from W.  The sums of
  * the averages are conserved to FP64 rounding.  Gradients (not conserved)
  * come from FP32 differences of the interface states and live in the shadow
- * only (Eq. slope).  mixed_update_var updates variable v (nc cells, fih =
- * 1/h in FP32) and returns its new FP32 value; mixed_update_cell all
- * variables (new FP32 values in wn) and the admissibility flags. */
+ * only (Eq. slope).  mixed_update_read reads and updates variable v of a cell (nc
+ * cells, fih = 1/h in FP32), mixed_update_store stores it; mixed_update_cell all
+ * variables (new FP32 values in wn) and the admissibility flags.  Every load of a
+ * cell comes before its first store, so that they are in flight together (they
+ * may not move past a store: chain.cuh).  GB300, a stage at 2048^2 / 256^3 /
+ * 99 x 64 x 50: 177 us / 1.06 ms / 27 us; with each variable's loads behind the
+ * last one's stores 204 us / 1.33 ms / 39 us. */
+template <int M> struct MixedVar {
+    float g[M]; /* gradients */
+    F2 w, acc;  /* stage 1: the next input and the accumulator */
+    double W;   /* stage 2: the new state */
+};
+
 template <int M, int STAGE, typename FaceSum>
-__device__ __forceinline__ float mixed_update_var(long nc, float fih, const FaceSum &fsum, const UpdC &uc,
-                                                 double *__restrict__ W, float *__restrict__ acc, const Shadow &s0,
-                                                 const Shadow &s1, long cell, int v)
+__device__ __forceinline__ void mixed_update_read(long nc, float fih, const FaceSum &fsum, const UpdC &uc, const double *W,
+                                                  const float *acc, const Shadow &s0, long cell, int v, MixedVar<M> &o)
 {
     constexpr int NV = M + 2, NG = (M == 2) ? 2 : 4;
     const float gw = fih / NG;
-    const Shadow &so = (STAGE == 1) ? s1 : s0;
     float sF = 0.f, eF = 0.f, sT = 0.f, eT = 0.f;
 #pragma unroll
     for (int d = 0; d < M; ++d) {
@@ -1144,29 +1152,39 @@ __device__ __forceinline__ float mixed_update_var(long nc, float fih, const Face
         }
         two_sum_acc(sT, eT, fsum(1, v, d, 1));
         two_sum_acc(sT, eT, -fsum(1, v, d, 0));
-        so.g[(d * NV + v) * nc + cell] = (fsum(2, v, d, 1) - fsum(2, v, d, 0)) * gw;
+        o.g[d] = (fsum(2, v, d, 1) - fsum(2, v, d, 0)) * gw;
     }
     const F2 ST{sT, eT};
     if (STAGE == 1) {
         const F2 SF{sF, eF};
-        const F2 dW = df_add(df_mul(uc.k[0], SF), df_mul(uc.k[1], ST));
-        const F2 A = df_add(df_mul(uc.k[2], SF), df_mul(uc.k[3], ST));
-        acc[v * nc + cell] = A.hi;
-        acc[(NV + v) * nc + cell] = A.lo;
-        const F2 w = df_add(F2{s0.hi[v * nc + cell], s0.lo[v * nc + cell]}, dW);
-        so.hi[v * nc + cell] = w.hi;
-        so.lo[v * nc + cell] = w.lo;
-        return w.hi;
+        o.acc = df_add(df_mul(uc.k[2], SF), df_mul(uc.k[3], ST));
+        o.w = df_add(F2{s0.hi[v * nc + cell], s0.lo[v * nc + cell]}, df_add(df_mul(uc.k[0], SF), df_mul(uc.k[1], ST)));
     } else {
         const F2 dW = df_add(F2{acc[v * nc + cell], acc[(NV + v) * nc + cell]}, df_mul(uc.k[4], ST));
-        const double w = (W[v * nc + cell] + widen(dW.hi)) + widen(dW.lo);
-        W[v * nc + cell] = w;
-        float wh, wl;
-        split(w, wh, wl);
-        so.hi[v * nc + cell] = wh;
-        so.lo[v * nc + cell] = wl;
-        return wh;
+        o.W = (W[v * nc + cell] + widen(dW.hi)) + widen(dW.lo);
     }
+}
+
+/* returns the variable's new FP32 value */
+template <int M, int STAGE>
+__device__ __forceinline__ float mixed_update_store(long nc, const MixedVar<M> &o, double *W, float *acc, const Shadow &s0,
+                                                    const Shadow &s1, long cell, int v)
+{
+    constexpr int NV = M + 2;
+    const Shadow &so = (STAGE == 1) ? s1 : s0;
+#pragma unroll
+    for (int d = 0; d < M; ++d) so.g[(d * NV + v) * nc + cell] = o.g[d];
+    F2 w = o.w;
+    if (STAGE == 1) {
+        acc[v * nc + cell] = o.acc.hi;
+        acc[(NV + v) * nc + cell] = o.acc.lo;
+    } else {
+        W[v * nc + cell] = o.W;
+        split(o.W, w.hi, w.lo);
+    }
+    so.hi[v * nc + cell] = w.hi;
+    so.lo[v * nc + cell] = w.lo;
+    return w.hi;
 }
 
 /* admissibility flags of a new state from the FP32 values of its variables */
@@ -1189,13 +1207,16 @@ __device__ __forceinline__ void mixed_update_cell(const KP &P, const FaceSum &fs
                                                   const Shadow &s1, int *__restrict__ status, long cell, float *wn)
 {
     constexpr int NV = M + 2;
+    MixedVar<M> o[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) wn[v] = mixed_update_var<M, STAGE>(P.ncell, P.fih, fsum, uc, W, acc, s0, s1, cell, v);
+    for (int v = 0; v < NV; ++v) mixed_update_read<M, STAGE>(P.ncell, P.fih, fsum, uc, W, acc, s0, cell, v, o[v]);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) wn[v] = mixed_update_store<M, STAGE>(P.ncell, o[v], W, acc, s0, s1, cell, v);
     mixed_state_flags<M>(P, wn, status);
 }
 
 /* The FP64 stage update of one cell from the face sums over the Gauss points
- * (weight wg each), fsum(q, v, d, plus) as in mixed_update_var; Wn receives
+ * (weight wg each), fsum(q, v, d, plus) as in mixed_update_read; Wn receives
  * the new averages.
  * STAGE 1: Ws = W - dt/2 L(F) - dt^2/8 L(Ft), Gs = Gauss(W(dt/2)), Acc = -dt L(F) - dt^2/6 L(Ft)
  * STAGE 2: W += Acc - dt^2/3 L(Ft*),        G  = Gauss(W*(dt/2))
@@ -1208,6 +1229,7 @@ __device__ __forceinline__ void fp64_update_cell(const KP &P, const FaceSum &fsu
 {
     constexpr int NV = M + 2;
     const double cw = wg * P.ih;
+    double g[M][NV], acc[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         double DF = 0.0, DFt = 0.0;
@@ -1215,19 +1237,25 @@ __device__ __forceinline__ void fp64_update_cell(const KP &P, const FaceSum &fsu
         for (int d = 0; d < M; ++d) {
             if (STAGE == 1) DF += fsum(0, v, d, 1) - fsum(0, v, d, 0);
             DFt += fsum(1, v, d, 1) - fsum(1, v, d, 0);
-            double *Gout = (STAGE == 1) ? Gs : G;
-            Gout[(d * NV + v) * P.ncell + cell] = (fsum(2, v, d, 1) - fsum(2, v, d, 0)) * cw;
+            g[d][v] = (fsum(2, v, d, 1) - fsum(2, v, d, 0)) * cw;
         }
         DF *= cw;
         DFt *= cw;
         if (STAGE == 1) {
             Wn[v] = W[v * P.ncell + cell] - 0.5 * dt * DF - dt * dt * 0.125 * DFt;
-            Ws[v * P.ncell + cell] = Wn[v];
-            Acc[v * P.ncell + cell] = -dt * DF - dt * dt / 6.0 * DFt;
+            acc[v] = -dt * DF - dt * dt / 6.0 * DFt;
         } else {
             Wn[v] = W[v * P.ncell + cell] + Acc[v * P.ncell + cell] - dt * dt / 3.0 * DFt;
-            W[v * P.ncell + cell] = Wn[v];
         }
+    }
+    /* every load of the cell comes before its first store (chain.cuh) */
+    double *Wout = (STAGE == 1) ? Ws : W, *Gout = (STAGE == 1) ? Gs : G;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+#pragma unroll
+        for (int d = 0; d < M; ++d) Gout[(d * NV + v) * P.ncell + cell] = g[d][v];
+        Wout[v * P.ncell + cell] = Wn[v];
+        if (STAGE == 1) Acc[v * P.ncell + cell] = acc[v];
     }
     double ke = 0.0;
 #pragma unroll
@@ -1385,9 +1413,9 @@ template <typename T> __device__ __forceinline__ void block_speed_max(T s, T ir,
 }
 
 template <int M, typename T>
-__global__ void wavespeed_kernel(KP P, const T *__restrict__ W, unsigned long long *__restrict__ smax)
+__global__ void wavespeed_kernel(KP P, const T *W, unsigned long long *smax)
 {
-    after_previous(W);
+    after_previous();
     T s = T(0), ir = T(0); /* max |u_d| + c and max 1 / rho */
     const T gam = pick<T>(P.gamma, (float)(P.fgm1 + 1.0f));
     for (long c = (long)blockIdx.x * blockDim.x + threadIdx.x; c < P.ncell; c += (long)gridDim.x * blockDim.x) {
@@ -1411,11 +1439,11 @@ __device__ __forceinline__ double dt_of_speed(const unsigned long long *smax, do
     return fmin(dt, cfl_h / nu);
 }
 
-static __global__ void dt_from_speed_kernel(const unsigned long long *__restrict__ smax, double cfl_h, double visc,
-                                            double *__restrict__ dtp, float *__restrict__ updc, double cw,
-                                            unsigned long long *__restrict__ clear)
+static __global__ void dt_from_speed_kernel(const unsigned long long *smax, double cfl_h, double visc,
+                                            double *dtp, float *updc, double cw,
+                                            unsigned long long *clear)
 {
-    after_previous(smax);
+    after_previous();
     if (clear) clear[0] = clear[1] = 0ull;
     const double dt = dt_of_speed(smax, cfl_h, visc);
     dtp[0] = dt;

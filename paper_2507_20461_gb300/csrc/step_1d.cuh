@@ -91,12 +91,11 @@ __device__ __forceinline__ void gather3(double x, int from, double *o)
 }
 
 template <bool NS, int STAGE>
-__global__ void __launch_bounds__(128) step1d_short_kernel(KP P, const double *__restrict__ Win, const double *__restrict__ Gin,
-                                                           double *__restrict__ W, double *__restrict__ G,
-                                                           double *__restrict__ Ws, double *__restrict__ Gs,
-                                                           double *__restrict__ Acc, int *__restrict__ status, StepClock clk)
+__global__ void __launch_bounds__(128) step1d_short_kernel(KP P, const double *Win, const double *Gin, double *W,
+                                                           double *G, double *Ws, double *Gs, double *Acc, int *status,
+                                                           StepClock clk)
 {
-    after_previous(Win, Gin, clk.dt, clk.in);
+    after_previous();
     __shared__ double q[kShortFaces][9];
     const int n = P.n[0], sub = threadIdx.x & 7, face = threadIdx.x >> 3;
     const int f = min((int)blockIdx.x * kCellsShort + face, n); /* past the last face: the last face again */
@@ -169,12 +168,10 @@ __global__ void __launch_bounds__(128) step1d_short_kernel(KP P, const double *_
 }
 
 template <typename R, bool NS, int STAGE>
-__global__ void __launch_bounds__(32) step1d_kernel(KP P, const double *__restrict__ Win, const double *__restrict__ Gin,
-                                                    double *__restrict__ W, double *__restrict__ G, double *__restrict__ Ws,
-                                                    double *__restrict__ Gs, double *__restrict__ Acc,
-                                                    int *__restrict__ status, StepClock clk)
+__global__ void __launch_bounds__(32) step1d_kernel(KP P, const double *Win, const double *Gin, double *W, double *G,
+                                                    double *Ws, double *Gs, double *Acc, int *status, StepClock clk)
 {
-    after_previous(Win, Gin, clk.dt, clk.in);
+    after_previous();
     const int lane = threadIdx.x, n = P.n[0];
     const int f = min((int)blockIdx.x * kCells1d + lane, n); /* lanes past the last face repeat it */
     const double dt = clock_dt(clk);

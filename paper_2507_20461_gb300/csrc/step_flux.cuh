@@ -426,13 +426,12 @@ struct FaceOrder {
 /* SPLIT: a lane per Gauss point, 64 / NG faces a block */
 template <typename R, int M, bool NS, bool SPLIT, bool POINTS = false>
 __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, M, NS>))
-    step_flux_kernel(KP P, const R *__restrict__ B, const double *__restrict__ dtp, R *__restrict__ ff,
-                     int *__restrict__ status, FaceOrder order, bool rev)
+    step_flux_kernel(KP P, const R *B, const double *dtp, R *ff, int *status, FaceOrder order, bool rev)
 {
     constexpr int BT = kStepFluxBlock, PER = SPLIT ? (M == 3 ? 4 : 2) : 1, FB = BT / PER;
     __shared__ typename FaceV<R>::V slots[SPLIT ? 1 : kFaceStash<R, M> * BT];
+    after_previous();
     typename FaceV<R>::V *stash = SPLIT ? slots : slots + threadIdx.x;
-    after_previous(B, dtp);
     const R dt = R(dtp[0]), idt = R(dtp[1]);
     unsigned dir, block;
     order.at<M>(block_in_order(rev), dir, block);
@@ -465,7 +464,7 @@ __device__ __forceinline__ void step_update_item(const KP &P, const R *__restric
         fm[d] = ff + group_off<kFaceFields<M>>((unsigned)face_of<M>(P, d, i, j, k, 0));
         fp[d] = ff + group_off<kFaceFields<M>>((unsigned)face_of<M>(P, d, i, j, k, 1));
     }
-    auto fsum = [&](int q, int v, int d, int plus) -> R { return load_ro((plus ? fp[d] : fm[d]) + (q * NV + v) * 32); };
+    auto fsum = [&](int q, int v, int d, int plus) -> R { return (plus ? fp[d] : fm[d])[(q * NV + v) * 32]; };
     if constexpr (sizeof(R) == sizeof(float))
         mixed_update_cell<M, STAGE>(P, fsum, uc, W, (float *)Acc, s0, s1, status, cell, wn);
     else
@@ -475,14 +474,11 @@ __device__ __forceinline__ void step_update_item(const KP &P, const R *__restric
 /* SPEED: the new state's wave speed into smax as well (the last stage of a CFL
  * step that another follows), from the values that wavespeed_kernel would read */
 template <typename R, int M, int STAGE, bool SPEED>
-__global__ void __launch_bounds__(256) step_update_kernel(KP P, const R *__restrict__ ff, const double *__restrict__ dtp,
-                                                          double *__restrict__ W, double *__restrict__ G,
-                                                          double *__restrict__ Ws, double *__restrict__ Gs,
-                                                          double *__restrict__ Acc, Shadow s0, Shadow s1,
-                                                          int *__restrict__ status, const float *__restrict__ updc,
-                                                          unsigned long long *__restrict__ smax, bool rev)
+__global__ void __launch_bounds__(256) step_update_kernel(KP P, const R *ff, const double *dtp, double *W, double *G,
+                                                          double *Ws, double *Gs, double *Acc, Shadow s0, Shadow s1,
+                                                          int *status, const float *updc, unsigned long long *smax, bool rev)
 {
-    after_previous(ff, dtp, updc);
+    after_previous();
     UpdC uc;
     if constexpr (sizeof(R) == sizeof(float)) uc = load_updc(updc);
     const long cell = (long)block_in_order(rev) * blockDim.x + threadIdx.x;
