@@ -78,6 +78,11 @@ GKS_HD double bitsd(uint64_t u)
 /* exponent biases: FP64 1023, FP32 127 */
 constexpr uint32_t kRebias = 1023 - 127;
 
+/* x > 0 and far from the ends of the format (2^-700 to infinity): the sign of a
+ * difference of products that reaches x lost nothing to underflow, and nothing
+ * overflowed.  One integer comparison. */
+GKS_HD bool surely_positive(double x) { return (uint32_t)(dbits(x) >> 32) - 0x14300000u < 0x7ff00000u - 0x14300000u; }
+
 } // namespace fps
 
 /* The hardware conversions, for the values outside the fast ranges: behind a

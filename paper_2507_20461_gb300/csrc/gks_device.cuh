@@ -158,18 +158,31 @@ template <typename R, int M> struct HalfStream {
     R W0[M + 2], Fk[M + 2], WT[M + 2], FT[M + 2], WA[M + 2], FA[M + 2], p;
 };
 
-template <typename R, int M, bool NS>
-__device__ __forceinline__ bool half_stream(const R *W, const R (*dW)[M + 2], R gm1, R Ntot, R s, HalfStream<R, M> &o)
+/* 1 / rho, velocity, rho |U|^2 and pressure of a state (rho |U|^2 from m U: in
+ * range wherever the state is) */
+template <typename R, int M> struct Primitive {
+    R inv, U[M], ke, p;
+};
+template <typename R, int M> __device__ __forceinline__ Primitive<R, M> primitive_of(const R *W, R gm1)
 {
-    const R inv = R(1) / W[0];
-    R U[M], ke = R(0);
+    Primitive<R, M> q;
+    q.inv = R(1) / W[0];
+    q.ke = R(0);
 #pragma unroll
     for (int i = 0; i < M; ++i) {
-        U[i] = W[1 + i] * inv;
-        ke += U[i] * W[1 + i];
+        q.U[i] = W[1 + i] * q.inv;
+        q.ke += q.U[i] * W[1 + i];
     }
-    const R hUU = R(0.5) * ke * inv; /* |U|^2 / 2 */
-    const R p = gm1 * (W[M + 1] - R(0.5) * ke);
+    q.p = gm1 * (W[M + 1] - R(0.5) * q.ke);
+    return q;
+}
+
+template <typename R, int M, bool NS>
+__device__ __forceinline__ bool half_stream(const R *W, const Primitive<R, M> &prim, const R (*dW)[M + 2], R gm1, R Ntot, R s,
+                                            HalfStream<R, M> &o)
+{
+    const R inv = prim.inv, p = prim.p, *U = prim.U;
+    const R hUU = R(0.5) * prim.ke * inv; /* |U|^2 / 2 */
     if (!positive(W[0]) || !positive(p)) return false;
     o.p = p;
     const R th = p * inv;
@@ -357,10 +370,11 @@ template <typename R, int M> struct Streams {
 
 /* FP32: both sides at once on left/right lane pairs (packed two-lane instructions) */
 template <int M, bool NS>
-__device__ __forceinline__ bool streams_of(const FluxParams &fp, const LR *W, const LR (*dW)[M + 2], Streams<float, M> &o)
+__device__ __forceinline__ bool streams_of(const FluxParams &fp, const LR *W, const Primitive<LR, M> &prim,
+                                           const LR (*dW)[M + 2], Streams<float, M> &o)
 {
     HalfStream<LR, M> q;
-    if (!half_stream<LR, M, NS>(W, dW, LR(fp.fgm1), LR(fp.fNtot), LR(1.f, -1.f), q)) return false;
+    if (!half_stream<LR, M, NS>(W, prim, dW, LR(fp.fgm1), LR(fp.fNtot), LR(1.f, -1.f), q)) return false;
     o.pl = q.p.l();
     o.pr = q.p.r();
 #pragma unroll
@@ -379,13 +393,13 @@ __device__ __forceinline__ bool streams_of(const FluxParams &fp, const LR *W, co
     return true;
 }
 
-/* FP64: one side after the other */
-template <int M, bool NS>
-__device__ __forceinline__ bool streams_of(const FluxParams &fp, const double *Wl, const double *Wr,
+/* FP64: one side after the other; prim(g) gives the primitive state of side g */
+template <int M, bool NS, typename Prim>
+__device__ __forceinline__ bool streams_of(const FluxParams &fp, const double *Wl, const double *Wr, const Prim &prim,
                                            const double (*dWl)[M + 2], const double (*dWr)[M + 2], Streams<double, M> &o)
 {
     HalfStream<double, M> q;
-    if (!half_stream<double, M, NS>(Wl, dWl, fp.gm1, fp.Ntot, 1.0, q)) return false;
+    if (!half_stream<double, M, NS>(Wl, prim(0), dWl, fp.gm1, fp.Ntot, 1.0, q)) return false;
     o.pl = q.p;
 #pragma unroll
     for (int b = 0; b < M + 2; ++b) {
@@ -398,7 +412,7 @@ __device__ __forceinline__ bool streams_of(const FluxParams &fp, const double *W
             o.FA[b] = q.FA[b];
         }
     }
-    if (!half_stream<double, M, NS>(Wr, dWr, fp.gm1, fp.Ntot, -1.0, q)) return false;
+    if (!half_stream<double, M, NS>(Wr, prim(1), dWr, fp.gm1, fp.Ntot, -1.0, q)) return false;
     o.pr = q.p;
 #pragma unroll
     for (int b = 0; b < M + 2; ++b) {
@@ -570,9 +584,10 @@ __device__ __forceinline__ bool gks_point_scaled(const FluxParams &fp, R dt, R i
 #pragma unroll
             for (int e = 0; e < M; ++e) dW[e][b] = LR(dWl[e][b], dWr[e][b]);
         }
-        if (!streams_of<M, NS>(fp, W, dW, q)) return false;
+        if (!streams_of<M, NS>(fp, W, primitive_of<LR, M>(W, LR(fp.fgm1)), dW, q)) return false;
     } else {
-        if (!streams_of<M, NS>(fp, Wl, Wr, dWl, dWr, q)) return false;
+        auto prim = [&](int g) { return primitive_of<R, M>(g ? Wr : Wl, fp.gm1); };
+        if (!streams_of<M, NS>(fp, Wl, Wr, prim, dWl, dWr, q)) return false;
     }
     return flux_of_streams<R, M, NS>(fp, dt, idt, ih, q, F, Ft, Wh);
 }

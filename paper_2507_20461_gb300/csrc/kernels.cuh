@@ -311,23 +311,32 @@ __device__ __forceinline__ void ao_weights(const KP &P, const R *d, const R *IS,
     for (int k = 0; k <= K; ++k) w[k] *= is;
 }
 
+/* A face state whose density and pressure are above delta times those of the
+ * cell average.  FP64: without divisions, rho p / (gamma - 1) = q, so p > delta p_c
+ * is q rho_c > delta q_c rho; what that does not surely accept (it leaves the format
+ * at rho^2 E below 2^-1022 or above 2^1024, where the state does not) is tested by
+ * divisions. */
 template <typename R, int M>
 __device__ __forceinline__ bool admissible(const R *w, const R *wc, R, R delta)
 {
+    if constexpr (sizeof(R) == sizeof(double)) {
+        R ke = R(0), kc = R(0);
+#pragma unroll
+        for (int a = 0; a < M; ++a) {
+            ke += w[1 + a] * w[1 + a];
+            kc += wc[1 + a] * wc[1 + a];
+        }
+        const R t = (w[0] * w[M + 1] - R(0.5) * ke) * wc[0] - delta * (wc[0] * wc[M + 1] - R(0.5) * kc) * w[0];
+        const bool dense = (int32_t)(fps::dbits(wc[0]) >> 32) >= 0; /* rho_c >= 0 */
+        if (dense && w[0] > delta * wc[0] && fps::surely_positive(t)) return true;
+    }
     R ke = R(0), kc = R(0);
 #pragma unroll
     for (int a = 0; a < M; ++a) {
-        ke += w[1 + a] * w[1 + a];
-        kc += wc[1 + a] * wc[1 + a];
+        ke += w[1 + a] * (w[1 + a] / w[0]);
+        kc += wc[1 + a] * (wc[1 + a] / wc[0]);
     }
-    if constexpr (sizeof(R) == sizeof(float)) /* products of three factors would leave FP32's range early */
-        return w[0] > delta * wc[0] && w[M + 1] - R(0.5) * ke / w[0] > delta * (wc[M + 1] - R(0.5) * kc / wc[0]);
-    /* p > delta p_c without divisions: rho p / (gamma - 1) = q, so
-     * q rho_c > delta q_c rho (reversed where rho_c < 0; a rho <= 0 fails in the
-     * flux either way) */
-    const R q = w[0] * w[M + 1] - R(0.5) * ke, qc = wc[0] * wc[M + 1] - R(0.5) * kc;
-    const R t = q * wc[0] - delta * qc * w[0];
-    return w[0] > delta * wc[0] && (wc[0] >= R(0) ? t > R(0) : t < R(0));
+    return w[0] > delta * wc[0] && w[M + 1] - R(0.5) * ke > delta * (wc[M + 1] - R(0.5) * kc);
 }
 
 /* ------------------------------------------------------------------ */

@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(128) step1d_short_kernel(KP P, const double *W
         }
     }
     HalfStream<double, 1> hs;
-    bool ok = half_stream<double, 1, NS>(Wq, dW, P.fp.gm1, P.fp.Ntot, side ? -1.0 : 1.0, hs);
+    bool ok = half_stream<double, 1, NS>(Wq, primitive_of<double, 1>(Wq, P.fp.gm1), dW, P.fp.gm1, P.fp.Ntot, side ? -1.0 : 1.0, hs);
     if (!ok) hs = HalfStream<double, 1>{};
     ok = __shfl_xor_sync(0xffffffffu, (int)ok, 1) && ok;
     Streams<double, 1> s;
