@@ -529,10 +529,19 @@ __device__ __forceinline__ bool flux_of_streams(const FluxParams &fp, R dt, R id
     /* relaxation time over dt, kappa = tau_n / dt, and the time integrals */
     R kap, eh = R(0), tau = R(0);
     if constexpr (std::is_same_v<R, double> && !NS) {
-        /* kappa = y / S and 1 / (2 kappa) from one reciprocal of S y */
-        const double S = pl + pr, y = fp.c1 * S + fp.c2 * fabs(pl - pr), q = 1.0 / (S * y);
-        kap = y > 0.0 ? y * y * q : 0.0;
-        if (y > 0.0) eh = exp(-0.5 * S * S * q);
+        /* kappa = y / S and 1 / (2 kappa) from one reciprocal of S y, or by a
+         * division each where S y is 0 or outside 2^-1000 .. 2^1000 */
+        const double S = pl + pr, y = fp.c1 * S + fp.c2 * fabs(pl - pr), Sy = S * y;
+        double z;
+        if ((uint32_t)(fps::dbits(Sy) >> 32) - 0x01700000u < 0x7e700000u - 0x01700000u) {
+            const double q = 1.0 / Sy;
+            kap = y * y * q;
+            z = -0.5 * S * S * q;
+        } else {
+            kap = fp.c1 + fp.c2 * fabs(pl - pr) / S;
+            z = kap > 0.0 ? -0.5 / kap : -1e3; /* exp(-1e3) = 0 */
+        }
+        eh = exp(z);
     } else {
         kap = pick<R>(fp.c1, fp.fc1) + pick<R>(fp.c2, fp.fc2) * RT<R>::abs_(pl - pr) / (pl + pr);
         if constexpr (NS) {

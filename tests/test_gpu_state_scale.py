@@ -47,6 +47,7 @@ def _step(n, W, G, precision, mu, **kw):
 
 CASES = [(1, k, n, {}) for k in (-90, -75, 40) for n in ((40, 24), (300, 260), (12, 9, 10), (40, 41, 42))]
 CASES += [(0, k, n, {}) for k in (-400, -360, 345) for n in ((40, 24), (260, 200), (12, 9, 10), (30, 31, 32), (50,), (9001,))]
+CASES += [(0, -520, n, {}) for n in ((40, 24), (260, 200), (12, 9, 10), (50,), (9001,))]
 CASES += [(0, k, n, {"order": 6}) for k in (-400, 345) for n in ((50,), (9001,))]
 
 

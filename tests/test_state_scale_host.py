@@ -78,6 +78,14 @@ def test_fp64_flux_scales_with_the_state(exe, n, mu, jump, k):
     _check(exe, n, mu, 0, k, jump, 1e-13)
 
 
+@pytest.mark.parametrize("n", GRIDS + [(31,)])
+@pytest.mark.parametrize("mu,jump", [(0.0, False), (0.0, True), (0.01, False)])
+@pytest.mark.parametrize("k", [-900, -520, -515, 515, 520, 900])
+def test_fp64_flux_scales_past_the_root_of_the_range(exe, n, mu, jump, k):
+    """pressures whose products leave the format: the relaxation time is a quotient of them"""
+    _check(exe, n, mu, 0, k, jump, 1e-13)
+
+
 def test_fp64_admissibility_matches_its_definition(tmp_path):
     exe = str(tmp_path / "admissible_check")
     r = subprocess.run(["g++", "-O1", "-std=c++17", "-I", os.path.join(HERE, "hostshim"), "-I", CSRC,
