@@ -2,12 +2,16 @@
 half-space moments of the FP64 gas-kinetic flux.
 
 On each interval |x - k/32| <= 1/64, k = 0 .. 96, the degree-8 Chebyshev
-interpolants of erfc(x) and exp(-x^2), as polynomials in x - k/32 (their
-truncation is below 2^-55 of the value there; checked here).  All arithmetic in
-mpmath at 50 digits; the method is plain Chebyshev interpolation of the
+interpolants of erfc(x) and exp(-x^2), as polynomials in x - x_k (their
+truncation is below 2^-55 of the value there; checked here).  The x_k are
+accurate table points (Gal's method): the first double k/32 + j 2^-40, j = 0, 1,
+.., at which both functions lie within 1/64 of a unit in the last place of a
+double, so that the constant terms carry no rounding and a result little more
+than its last operation's.  All arithmetic in mpmath at 50 digits from the
 functions' definitions.
 
 Run: python gen_erfc.py (writes erfc_table.cuh beside it)."""
+import math
 import os
 
 import mpmath as mp
@@ -15,6 +19,22 @@ import mpmath as mp
 mp.mp.dps = 50
 HERE = os.path.dirname(os.path.abspath(__file__))
 DEG, STEP, ROWS = 8, 32, 97
+FUNCTIONS = (mp.erfc, lambda x: mp.exp(-x * x))
+
+
+def off_grid(v):
+    """distance of v from the nearest double, in units of its last place"""
+    f = float(v)
+    return abs(v - mp.mpf(f)) / (mp.mpf(2) ** (math.frexp(f)[1] - 53))
+
+
+def node(k):
+    j = 0
+    while True:
+        x = mp.mpf(k) / STEP + mp.mpf(j) / 2**40
+        if all(off_grid(f(x)) <= mp.mpf(1) / 64 for f in FUNCTIONS):
+            return x
+        j += 1
 
 
 def interpolant(f, c, r, deg):
@@ -42,15 +62,15 @@ def table():
     rows, worst = [], mp.mpf(0)
     r = mp.mpf(1) / (2 * STEP)
     for k in range(ROWS):
-        c = mp.mpf(k) / STEP
+        c = node(k)
         row = []
-        for f in (mp.erfc, lambda x: mp.exp(-x * x)):
+        for f in FUNCTIONS:
             a = interpolant(f, c, r, DEG)
             for i in range(-16, 17):
                 d = r * i / 16
                 worst = max(worst, abs(horner(a, d) / f(c + d) - 1))
-            row.append([float(v) for v in a])
-        rows.append(row)
+            row.append([float(f(c))] + [float(v) for v in a[1:]])
+        rows.append(row + [[float(c), 0.0]])
     assert worst < mp.mpf(2) ** -55, worst
     return rows, worst
 
@@ -58,10 +78,10 @@ def table():
 def main():
     rows, worst = table()
     L = ["/* Generated by gen_erfc.py (Chebyshev interpolation, 50 digits).  Do not edit. */", "#pragma once", "",
-         f"/* FP64: row k, polynomials in x - k/{STEP} on |x - k/{STEP}| <= 1/{2 * STEP}, x < 3: erfc(x) coefficients 0..{DEG},",
-         f" * then exp(-x^2) coefficients 0..{DEG}; worst relative truncation {mp.nstr(worst, 2)}. */",
+         f"/* FP64: row k, polynomials in x - x_k on |x - k/{STEP}| <= 1/{2 * STEP}, x < 3: erfc(x) coefficients 0..{DEG},",
+         f" * exp(-x^2) coefficients 0..{DEG}, x_k (k/{STEP} but for less than 2^-20) and 0; worst relative truncation {mp.nstr(worst, 2)}. */",
          f"#define ERFC_DEG {DEG}", f"#define ERFC_STEP {STEP}", f"#define ERFC_ROWS {ROWS}",
-         f"static __device__ __align__(16) const double erfc_rows[ERFC_ROWS][2 * (ERFC_DEG + 1)] = {{"]
+         f"static __device__ __align__(16) const double erfc_rows[ERFC_ROWS][2 * (ERFC_DEG + 1) + 2] = {{"]
     for row in rows:
         L.append("    {" + ", ".join(repr(v) for f in row for v in f) + "},")
     L += ["};", ""]

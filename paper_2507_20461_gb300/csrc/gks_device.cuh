@@ -56,11 +56,15 @@ namespace gks {
 
 /* The half-space moments take h = erfc(a) and e = exp(-a^2) of the same
  * argument.
- * FP64, |a| < 3 (Mach 3.5 normal to the face): degree-8 polynomials about the
- * nearest k/32 from a 14 KB table (gen_erfc.py; truncation below 2^-55), 21 FP64
- * instructions for both where the library's erfc and exp take about 71; the
- * table's loads run beside the FP64 pipe, which bounds the kernel (2D 512^2 face
- * flux 1.52 to 1.27 ms a stage).  The interval comes from an exact add of 1.5 2^47, whose unit is 1/32.  Above, the library.
+ * FP64, |a| < 3 (Mach 3.5 normal to the face): degree-8 polynomials about a point
+ * x_k near the nearest k/32 from a 15 KB table (gen_erfc.py; truncation below
+ * 2^-55), 20 FP64 instructions for both where the library's erfc and exp take about
+ * 71; the table's loads run beside the FP64 pipe, which bounds the kernel (2D 512^2
+ * face flux 1.52 to 1.27 ms a stage).  The interval comes from an exact add of 1.5
+ * 2^47, whose unit is 1/32.  Both functions are all but doubles at x_k, so the
+ * constant terms carry no rounding: error 0.76 and 0.61 ulp at most, 0.31 and 0.29
+ * rms, where correct rounding has 0.29 (with x_k = k/32 1.3 and 1.2, 0.39 and 0.40).
+ * Above, the library.
  * FP32: the library's erfc; e is the hardware exponential (__expf, about 2 + 1.2 x
  * ulp, x = a^2; it multiplies terms that vanish as x grows).  A polynomial in
  * 1 / (1 + |a|/2) times e, lanes together, raised the error of W(dt/2) by a third
@@ -79,8 +83,8 @@ template <> struct RT<double> {
         const double x = fps::bitsd(bits & 0x7fffffffffffffffull);
         if (hi < 0x40080000u) { /* |a| < 3 */
             const double m = 211106232532992.0; /* 1.5 2^47 */
-            const double t = x + m, d = x - (t - m);
-            const double *row = erfc_rows[(uint32_t)fps::dbits(t) & 127u];
+            const double *row = erfc_rows[(uint32_t)fps::dbits(x + m) & 127u];
+            const double d = x - row[2 * ERFC_DEG + 2];
             double p = row[ERFC_DEG], q = row[2 * ERFC_DEG + 1];
 #pragma unroll
             for (int j = ERFC_DEG - 1; j >= 0; --j) {
