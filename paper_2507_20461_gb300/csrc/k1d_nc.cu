@@ -71,15 +71,26 @@ __device__ __forceinline__ double nc_value(const KP &P, const double *u)
     return chi * qH + (1.0 - chi) * (ql / ws);
 }
 
+/* a / b, given ib = 1 / b: the product corrected by its remainder, as good as a
+ * division (one rounding but for ib's in the remainder) for two more operations.
+ * With the plain product the 10^6-cell step's error against 64 bits was 15% larger
+ * (4.6e-17 for 4.0e-17, 4.43 ms); with divisions 4.0e-17 and 4.61 ms; so 4.0e-17 and
+ * 4.50 ms. */
+__device__ __forceinline__ double quotient(double a, double b, double ib)
+{
+    const double q = a * ib;
+    return fma(fma(-q, b, a), ib, q);
+}
+
 /* HLLC flux (Toro) with the Davis wave-speed bounds; false if a state is
  * not admissible */
 __device__ __forceinline__ bool hllc(double gamma, const double *L, const double *R, double *F)
 {
     const double il = 1.0 / L[0], ir = 1.0 / R[0];
-    const double rl = L[0], ul = L[1] * il, pl = (gamma - 1.0) * (L[2] - 0.5 * rl * ul * ul);
-    const double rr = R[0], ur = R[1] * ir, pr = (gamma - 1.0) * (R[2] - 0.5 * rr * ur * ur);
+    const double rl = L[0], ul = quotient(L[1], rl, il), pl = (gamma - 1.0) * (L[2] - 0.5 * rl * ul * ul);
+    const double rr = R[0], ur = quotient(R[1], rr, ir), pr = (gamma - 1.0) * (R[2] - 0.5 * rr * ur * ur);
     if (!(rl > 0.0) || !(rr > 0.0) || !(pl > 0.0) || !(pr > 0.0)) return false;
-    const double cl = sqrt(gamma * pl * il), cr = sqrt(gamma * pr * ir);
+    const double cl = sqrt(quotient(gamma * pl, rl, il)), cr = sqrt(quotient(gamma * pr, rr, ir));
     const double SL = fmin(ul - cl, ur - cr), SR = fmax(ul + cl, ur + cr);
     const double Ss = (pr - pl + rl * ul * (SL - ul) - rr * ur * (SR - ur)) / (rl * (SL - ul) - rr * (SR - ur));
     if (0.0 <= SL) {
@@ -88,13 +99,13 @@ __device__ __forceinline__ bool hllc(double gamma, const double *L, const double
         F[2] = ul * (L[2] + pl);
     } else if (0.0 <= Ss) {
         const double k = rl * (SL - ul) / (SL - Ss);
-        const double Us[3] = {k, k * Ss, k * (L[2] * il + (Ss - ul) * (Ss + pl / (rl * (SL - ul))))};
+        const double Us[3] = {k, k * Ss, k * (quotient(L[2], rl, il) + (Ss - ul) * (Ss + pl / (rl * (SL - ul))))};
         const double FL[3] = {rl * ul, rl * ul * ul + pl, ul * (L[2] + pl)};
 #pragma unroll
         for (int v = 0; v < 3; ++v) F[v] = FL[v] + SL * (Us[v] - L[v]);
     } else if (0.0 <= SR) {
         const double k = rr * (SR - ur) / (SR - Ss);
-        const double Us[3] = {k, k * Ss, k * (R[2] * ir + (Ss - ur) * (Ss + pr / (rr * (SR - ur))))};
+        const double Us[3] = {k, k * Ss, k * (quotient(R[2], rr, ir) + (Ss - ur) * (Ss + pr / (rr * (SR - ur))))};
         const double FR[3] = {rr * ur, rr * ur * ur + pr, ur * (R[2] + pr)};
 #pragma unroll
         for (int v = 0; v < 3; ++v) F[v] = FR[v] + SR * (Us[v] - R[v]);
