@@ -142,7 +142,7 @@ __device__ __forceinline__ void nc_states(const KP &P, const double *__restrict_
             for (int i = 0; i < 6; ++i) u[i] = w[side ? 5 - i : i][v] - own[v];
             st[side][v] = own[v] + nc_value<ORDER>(P, u);
         }
-        if (!admissible<double, 1>(st[side], own, P.fp.gm1, P.adm)) {
+        if (!admissible<double, 1>(st[side], own, P.adm)) {
 #pragma unroll
             for (int v = 0; v < 3; ++v) st[side][v] = own[v];
         }
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(128) nc_short_kernel(KP P, const double *Win, 
     for (int side = 0; side < 2; ++side) {
         gather3(val, (threadIdx.x & 24) + 3 * side, st[side]);
         gather3(own, (threadIdx.x & 24) + 3 * side, cw);
-        if (!admissible<double, 1>(st[side], cw, P.fp.gm1, P.adm)) {
+        if (!admissible<double, 1>(st[side], cw, P.adm)) {
 #pragma unroll
             for (int v = 0; v < 3; ++v) st[side][v] = cw[v];
         }

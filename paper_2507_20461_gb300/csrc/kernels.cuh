@@ -317,7 +317,7 @@ __device__ __forceinline__ void ao_weights(const KP &P, const R *d, const R *IS,
  * at rho^2 E below 2^-1022 or above 2^1024, where the state does not) is tested by
  * divisions. */
 template <typename R, int M>
-__device__ __forceinline__ bool admissible(const R *w, const R *wc, R, R delta)
+__device__ __forceinline__ bool admissible(const R *w, const R *wc, R delta)
 {
     if constexpr (sizeof(R) == sizeof(double)) {
         R ke = R(0), kc = R(0);
@@ -480,13 +480,12 @@ __device__ __forceinline__ void states1d_face(const KP &P, const double *__restr
 {
     R st[2][3][2], cw[2][3];
     recon1d_face<R>(P, W, G, f, st, cw);
-    const R gm1 = pick<R>(P.fp.gm1, P.fgm1);
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
         R s[3];
 #pragma unroll
         for (int v = 0; v < 3; ++v) s[v] = st[side][v][0];
-        const bool ok = admissible<R, 1>(s, cw[side], gm1, pick<R>(P.adm, P.fadm));
+        const bool ok = admissible<R, 1>(s, cw[side], pick<R>(P.adm, P.fadm));
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
             const R val = ok ? st[side][v][0] : cw[side][v];
@@ -826,7 +825,6 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
     idx[0] = (int)fdivmod(P.dface[D][0], (unsigned)fl, q0);
     idx[1] = (M >= 2) ? (int)fdivmod(P.dface[D][1], q0, q1) : 0;
     idx[2] = (M >= 3) ? (int)q1 : 0;
-    const R gm1 = pick<R>(P.fp.gm1, P.fgm1);
     /* FP32: the blended coefficients of the two cells of the block's faces
      * are staged in shared memory, stage[side][v * NC + k][face in block].
      * Each face's NG threads copy a share of its 2 NV NC values with cp.async
@@ -889,7 +887,7 @@ __device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, c
         R s[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) s[v] = st[side][v][0];
-        if (!admissible<R, M>(s, cw[side], gm1, pick<R>(P.adm, P.fadm))) {
+        if (!admissible<R, M>(s, cw[side], pick<R>(P.adm, P.fadm))) {
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 st[side][v][0] = cw[side][v];

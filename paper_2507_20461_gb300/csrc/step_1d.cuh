@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(128) step1d_short_kernel(KP P, const double *W
     gather3(val, from, Wq);
     gather3(der, from, dW[0]);
     gather3(own, from, cw);
-    if (!admissible<double, 1>(Wq, cw, P.fp.gm1, P.adm)) {
+    if (!admissible<double, 1>(Wq, cw, P.adm)) {
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
             Wq[v] = cw[v];

@@ -38,7 +38,7 @@ template <int M> static void run(std::mt19937_64 &g, long *count)
         ++count[0];
         const bool want = dr > 0 && dp > 0;
         count[1] += want;
-        count[2] += want != gks::admissible<double, M>(w, c, 0.4, delta);
+        count[2] += want != gks::admissible<double, M>(w, c, delta);
     }
 }
 
