@@ -75,10 +75,12 @@ NC_CELL_UPDATE = {o: _flops(f"nc_step_cell_update_1d_order{o}") for o in (5, 6)}
 # step kernels' summary under profiles/).  The kernel uses closed forms where
 # the oracle solves moment systems, so it executes fewer flops than the
 # algorithmic count.
-EXECUTED_FLOPS_PER_FACE_GP = {"mixed": 972.0, "fp64": 988.0}
-# DRAM bytes (read + write) per launch of the face-flux kernel at 2048^2: a
-# 1-pass ncu capture at 1024^2 scaled by the faces (None: not captured).
-TRAFFIC_PER_FLUX_LAUNCH = {"mixed": 970e6, "fp64": None}
+EXECUTED_FLOPS_PER_FACE_GP = {"mixed": 980.0, "fp64": 978.0}
+# DRAM bytes (read + write) per launch of the face-flux kernel at 2048^2: each
+# extended cell's record of 40 floats read once and each face's 12 written once
+# (L2, 129 MB, holds the end of either; a 1024^2 capture reads its 168 MB of
+# records once).  FP64: not counted.
+TRAFFIC_PER_FLUX_LAUNCH = {"mixed": 4.0 * (40 * (N + 2) ** 2 + 12 * 2 * N * (N + 1)), "fp64": None}
 # Algorithmic HBM bytes per cell-update of the whole step (FP64 state,
 # stage buffers, accumulator), 2D: 60 doubles.
 BYTES_PER_CELL_UPDATE = 480.0

@@ -347,9 +347,10 @@ int gks_batch_get_state(gks_batch_t b, int grid, double *W, double *G, int on_de
 int gks_batch_run(gks_batch_t b, double cfl, int nsteps);
 
 /* JSON text of the launch shapes (per kernel class: block size, items per
- * tile, blocks, and for a tuned class the measured ms; the mixed-precision
- * stage kernels as one entry "stage"; "cached": true and no timings when the
- * choices came from the cache, with the size-class key); "" before the first gks_batch_run.  Owned by the handle. */
+ * tile, blocks, and for the wave speed, the one tuned class, the measured ms; the
+ * three mixed-precision stage kernels as one entry "stage", with the face flux's
+ * shape; "cached": true and no timings when the choices came from the cache, with the
+ * size-class key); "" before the first gks_batch_run.  Owned by the handle. */
 const char *gks_batch_tuning(gks_batch_t b);
 
 /* Synchronise and return the status word (as gks_status): the OR of every

@@ -155,8 +155,8 @@ __device__ __forceinline__ bool positive(LR x) { return x.l() > 0.f && x.r() > 0
  * Against raw transverse moments with tabulated expectations and general
  * slope vectors, and the equilibrium below in the same form (GB300, one step):
  * FP64 2D 512^2 5.5 to 4.4 ms, Navier-Stokes 390 x 195 2.1 to 1.55 ms; mixed
- * 256^3 54.5 to 40.9 ms, 2D 2048^2 2.6 to 2.42 ms.  The 3D FP32 flux spills 190
- * bytes for 500; FP64 registers fell from 254 to 188 (3D) and 172 to 132-151 (2D).
+ * 256^3 54.5 to 40.9 ms, 2D 2048^2 2.6 to 2.42 ms.  (Registers and spills of the
+ * flux kernels: step_flux.cuh.)
  */
 template <typename R, int M> struct HalfStream {
     R W0[M + 2], Fk[M + 2], WT[M + 2], FT[M + 2], WA[M + 2], FA[M + 2], p;

@@ -9,7 +9,7 @@
  * sweep's barriers held it at 16 warps per SM); the FP64 batch of 6 grids 4.67
  * ms against 5.54 ms with its tile loops over the per-point flux.  With chained
  * launches, the alternating block order and states in and out by one kernel
- * 2.42 ms and 3.55 ms.
+ * 2.37 ms and 3.49 ms.
  */
 #include "batch.h"
 #include "step_flux.cuh"
@@ -119,7 +119,9 @@ __global__ void __launch_bounds__(128) bk_poly(const KP common, const GridDesc *
         cell_poly_item<R, 2, true, sizeof(R) == sizeof(double)>(P, stage_src_of<R>(g, stage), (R *)g.B, t, (int)blockIdx.y);
 }
 
-/* block size and register cap of the single-grid face flux */
+/* block size and register cap of the single-grid face flux; FP32 spills 124 / 132
+ * bytes at it (the single grid 16 / 16), most likely for the grid's parameters, which
+ * are registers here and the constant bank there */
 template <typename R>
 __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, 2, false>))
     bk_flux(const KP common, const GridDesc *__restrict__ gd, const Tile *__restrict__ tiles,

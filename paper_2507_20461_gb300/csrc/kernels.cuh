@@ -775,9 +775,7 @@ __device__ __forceinline__ long ext_lin(const KP &P, int i, int j, int k)
     return r;
 }
 
-/* The FP32 flux's staging buffer: one per dimension, shared by the
- * directions (a kernel that runs several directions, such as the batched
- * flux, holds one buffer, not one per direction). */
+/* The staging buffer of the FP32 interface states and of gks_flux_2d_static */
 template <int M> __device__ __forceinline__ float *flux_stage()
 {
     constexpr int NV = M + 2, NG = (M == 2) ? 2 : 4;
@@ -1369,8 +1367,9 @@ template <int M, typename T> __device__ __forceinline__ T speed_of(const T *w, T
 }
 
 /* largest of the warp's speeds s and inverse densities ir into smax[0], smax[1]
- * (non-negative doubles order like their bit patterns; a NaN becomes 1e300,
- * which the host reports) */
+ * (non-negative doubles order like their bit patterns).  A cell whose speed is not a
+ * number does not count, here and below (fmax drops it; every warp has a lane at 0):
+ * the status word reports it. */
 template <typename T> __device__ __forceinline__ void speed_max(T s, T ir, unsigned long long *__restrict__ smax)
 {
 #pragma unroll
@@ -1411,7 +1410,6 @@ template <typename T> __device__ __forceinline__ void block_speed_max(T s, T ir,
             ir = fmax(ir, __shfl_xor_sync(0xffffffffu, ir, o));
         }
         if (threadIdx.x < 2) {
-            /* non-negative doubles order like their bit patterns; NaN is caught on the host */
             const double x = (double)(threadIdx.x ? ir : s);
             const unsigned long long b = (unsigned long long)__double_as_longlong(isnan(x) ? 1e300 : x);
             if (b > *(volatile unsigned long long *)(smax + threadIdx.x)) atomicMax(smax + threadIdx.x, b);

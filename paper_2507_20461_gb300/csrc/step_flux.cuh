@@ -19,8 +19,8 @@
  * cp.async and the sums exchanged through shared memory, one launch per
  * direction (GB300): 2048^2 mixed 0.77 to 0.48 ms a stage, 256^3 mixed 16.9
  * to 8.0 ms, 99 x 64 x 50 Navier-Stokes 0.39 to 0.20 ms, FP64 512^2 1.87 to
- * 1.50 ms (0.45, 7.9, 0.20 and 1.26 ms with the flux arithmetic, slots and block
- * order of now).
+ * 1.50 ms (0.456, 7.97, 0.197 and 1.236 ms with the flux arithmetic, slots and
+ * block order of now).
  *
  * Layouts (step path only): groups of 32 consecutive extended cells, or faces,
  * with the record fields of a group in rows of 32, so that every field of an
@@ -29,6 +29,11 @@
  *   B  : per cell NV (NC + 1) fields, the blended cubic and the (mirrored)
  *        average of each variable, so the flux needs no ghost mapping;
  *   ff : per face 3 NV fields, F, dF/dt and W(dt/2) summed over the Gauss points.
+ * In FP64 the sum over a face's points is rounded at the face value's size, where
+ * the difference of two neighbouring faces' points would be exact: a step's error
+ * against 64 bits is 5% to 8% larger than with every point kept (3.3e-15 for 3.1e-15,
+ * 390 x 195 viscous).  Kept, the points double ff and the update's FP64 work: 512^2
+ * 6.17 to 6.21 ms a pass of two steps, 20^3 609 to 628 us and 12 x 9 x 10 230 to 297 us a step.
  */
 #pragma once
 #include "kernels.cuh"
@@ -395,18 +400,21 @@ __device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict_
     }
 }
 
-/* All faces of a stage in one launch: the first nb0 blocks take the x faces,
- * the next (to nb1) the y faces, the rest the z faces. */
-/* Threads per block and resident blocks asked of the compiler, measured: 64
+/* All faces of a stage in one launch, in the order of FaceOrder.
+ * Threads per block and resident blocks asked of the compiler, measured: 64
  * threads spread a small grid over twice the SMs of 128 (equal on large
  * ones).  FP32 2D Euler 12 blocks (80 registers: 0.481 ms per 2048^2 launch;
- * 10 and 16 blocks 0.49 and 0.55), 3D 8 (128 registers, no spills: 8.0 ms per
- * 256^3 launch; 6 and 10 blocks 9.7 and 10.0), Navier-Stokes 8 (0.203 ms per
- * 99 x 64 x 50 launch; 10 blocks 0.25).  The points of a pair are
+ * 10 and 16 blocks 0.49 and 0.55), 3D 8 (128 registers: 8.0 ms per 256^3 launch;
+ * 6 and 10 blocks 9.7 and 10.0), Navier-Stokes 8 (0.203 ms per 99 x 64 x 50
+ * launch; 10 blocks 0.25).  Spilled at these caps (bytes stored / loaded): 2D Euler
+ * 16 / 16, 3D Euler 4 / 4, 3D Navier-Stokes 28 / 40, with every point written (gks_flux)
+ * 20 / 20, 0 and 44 / 60; the batch's copy of the 2D flux 124 / 132 (k2d_batch.cu).  The points of a pair are
  * unrolled: as a loop the packed constants stay in registers across it (2D
  * 0.54, 3D 9.0 ms).  FP64 is bound by its pipe: 4 to 6 blocks are equal, but
  * for spills (2D Navier-Stokes 4 blocks, 174 registers; 5 and 6 both cap at 168
- * and spill 190 bytes, as warps come in fours). */
+ * and spill 190 bytes, as warps come in fours).  FP64 registers: 2D 158 (a lane per
+ * point 132), Navier-Stokes 174 (148), 3D 224 (210), Navier-Stokes 255 with 4 bytes
+ * spilled (210). */
 constexpr int kStepFluxBlock = 64;
 template <typename R, int M, bool NS>
 constexpr int kStepFluxMinBlocks = sizeof(R) == sizeof(float) ? (M == 2 && !NS ? 12 : 8) : (M == 2 && !NS ? 6 : 4);
