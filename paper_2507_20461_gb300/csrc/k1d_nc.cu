@@ -119,7 +119,7 @@ __device__ __forceinline__ bool hllc(double gamma, const double *L, const double
 
 /* both states of face f, after the admissibility fallback */
 template <int ORDER>
-__device__ __forceinline__ void nc_states(const KP &P, const double *__restrict__ W, int f, double (*st)[3])
+__device__ __forceinline__ void nc_states(const KP &P, const double *W, int f, double (*st)[3])
 {
     double w[6][3]; /* cells f - 3 .. f + 2 */
 #pragma unroll
@@ -150,7 +150,7 @@ __device__ __forceinline__ void nc_states(const KP &P, const double *__restrict_
 }
 
 template <int ORDER>
-__device__ __forceinline__ void nc_flux(const KP &P, const double *__restrict__ W, int f, int *__restrict__ status, double *F)
+__device__ __forceinline__ void nc_flux(const KP &P, const double *W, int f, int *status, double *F)
 {
     double st[2][3];
     nc_states<ORDER>(P, W, f, st);
@@ -197,8 +197,8 @@ __global__ void __launch_bounds__(32) nc_face_kernel(KP P, const double *__restr
 
 /* The RK update of one cell from the fluxes of its faces; returns the new state. */
 template <int STAGE>
-__device__ __forceinline__ void nc_update(const KP &P, double dt, const double *F, const double *up, double *__restrict__ W0,
-                                          double *__restrict__ Wout, double *__restrict__ Acc, int *__restrict__ status,
+__device__ __forceinline__ void nc_update(const KP &P, double dt, const double *F, const double *up, double *W0,
+                                          double *Wout, double *Acc, int *status,
                                           long cell, double *out)
 {
     /* loads before stores (chain.cuh) */

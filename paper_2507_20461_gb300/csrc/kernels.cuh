@@ -415,7 +415,7 @@ __device__ __forceinline__ void sub_quadratics(R wm1, R w1, R w2, R dm1, R (*a)[
 
 /* states[side][v][c]: c = 0 value, 1 physical derivative */
 template <typename R>
-__device__ __forceinline__ void recon1d_face(const KP &P, const double *__restrict__ W, const double *__restrict__ G, int f,
+__device__ __forceinline__ void recon1d_face(const KP &P, const double *W, const double *G, int f,
                                              R (*st)[3][2], R (*cw)[3])
 {
     double w[4][3], d[4][3];
@@ -475,7 +475,7 @@ __device__ __forceinline__ void recon1d_face(const KP &P, const double *__restri
 /* both interface states of face f (physical derivatives), after the
  * admissibility fallback */
 template <typename R>
-__device__ __forceinline__ void states1d_face(const KP &P, const double *__restrict__ W, const double *__restrict__ G, int f,
+__device__ __forceinline__ void states1d_face(const KP &P, const double *W, const double *G, int f,
                                               R *Wl, R *Wr, R (*dWl)[3], R (*dWr)[3])
 {
     R st[2][3][2], cw[2][3];
@@ -498,8 +498,8 @@ __device__ __forceinline__ void states1d_face(const KP &P, const double *__restr
 
 /* F, dF/dt, W(dt/2) of face f */
 template <typename R, bool NS>
-__device__ __forceinline__ void flux1d_face(const KP &P, const double *__restrict__ W, const double *__restrict__ G, int f,
-                                            R dt, int *__restrict__ status, R *F, R *Ft, R *Wh)
+__device__ __forceinline__ void flux1d_face(const KP &P, const double *W, const double *G, int f,
+                                            R dt, int *status, R *F, R *Ft, R *Wh)
 {
     R Wl[3], Wr[3], dWl[1][3], dWr[1][3];
     states1d_face<R>(P, W, G, f, Wl, Wr, dWl, dWr);
@@ -670,7 +670,7 @@ __device__ __forceinline__ void blend_cubic(const KP &P, const R *d, R *b)
  * of 32 consecutive cells in rows of 32, v (NC + 1) + k with k = NC the
  * (mirrored) average itself (step_flux.cuh). */
 template <typename R, int M, bool GROUPED = false, bool ONE = false>
-__device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R *__restrict__ B, long t, int only = -1)
+__device__ __forceinline__ void cell_poly_item(const KP &P, const Src<R> &src, R *B, long t, int only = -1)
 {
     constexpr int NV = M + 2, NC = Cubic<R, M>::NC, ND = Cubic<R, M>::ND;
     int i, j, k;
@@ -787,8 +787,8 @@ template <int M> __device__ __forceinline__ float *flux_stage()
  * face_states[side][v][c][g][face] (double, global axes); FLUX = true the
  * fluxes ff[q][v][g][face] (R, global momentum order). */
 template <typename R, int M, int D, bool FLUX, bool NS = false>
-__device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, const R *__restrict__ B, double dtv,
-                                               double *__restrict__ fs, R *__restrict__ ff, int *__restrict__ status,
+__device__ __forceinline__ void face_flux_item(const KP &P, const Src<R> &src, const R *B, double dtv,
+                                               double *fs, R *ff, int *status,
                                                long t)
 {
     constexpr int NV = M + 2, NC = Cubic<R, M>::NC, NG = (M == 2) ? 2 : 4;
@@ -1088,7 +1088,7 @@ __device__ __forceinline__ void store_updc(float *p, const UpdC &u)
         p[2 * k + 1] = u.k[k].lo;
     }
 }
-__device__ __forceinline__ UpdC load_updc(const float *__restrict__ p)
+__device__ __forceinline__ UpdC load_updc(const float *p)
 {
     UpdC u;
 #pragma unroll
@@ -1193,7 +1193,7 @@ __device__ __forceinline__ float mixed_update_store(long nc, const MixedVar<M> &
 }
 
 /* admissibility flags of a new state from the FP32 values of its variables */
-template <int M> __device__ __forceinline__ void mixed_state_flags(const KP &P, const float *wn, int *__restrict__ status)
+template <int M> __device__ __forceinline__ void mixed_state_flags(const KP &P, const float *wn, int *status)
 {
     float ke = 0.f;
 #pragma unroll
@@ -1208,8 +1208,8 @@ template <int M> __device__ __forceinline__ void mixed_state_flags(const KP &P, 
 
 template <int M, int STAGE, typename FaceSum>
 __device__ __forceinline__ void mixed_update_cell(const KP &P, const FaceSum &fsum, const UpdC &uc,
-                                                  double *__restrict__ W, float *__restrict__ acc, const Shadow &s0,
-                                                  const Shadow &s1, int *__restrict__ status, long cell, float *wn)
+                                                  double *W, float *acc, const Shadow &s0,
+                                                  const Shadow &s1, int *status, long cell, float *wn)
 {
     constexpr int NV = M + 2;
     MixedVar<M> o[NV];
@@ -1228,9 +1228,9 @@ __device__ __forceinline__ void mixed_update_cell(const KP &P, const FaceSum &fs
  * with L(q)_j = (1/h) sum_d sum_g w_g (q(+d face) - q(-d face)). */
 template <int M, int STAGE, typename FaceSum>
 __device__ __forceinline__ void fp64_update_cell(const KP &P, const FaceSum &fsum, double wg, double dt,
-                                                 double *__restrict__ W, double *__restrict__ G, double *__restrict__ Ws,
-                                                 double *__restrict__ Gs, double *__restrict__ Acc,
-                                                 int *__restrict__ status, long cell, double *Wn)
+                                                 double *W, double *G, double *Ws,
+                                                 double *Gs, double *Acc,
+                                                 int *status, long cell, double *Wn)
 {
     constexpr int NV = M + 2;
     const double cw = wg * P.ih;
@@ -1274,10 +1274,10 @@ __device__ __forceinline__ void fp64_update_cell(const KP &P, const FaceSum &fsu
 }
 
 template <typename R, int M, int STAGE>
-__device__ __forceinline__ void update_item(const KP &P, const R *__restrict__ ff, double dt, double *__restrict__ W,
-                                            double *__restrict__ G, double *__restrict__ Ws, double *__restrict__ Gs,
-                                            double *__restrict__ Acc, const Shadow &s0, const Shadow &s1,
-                                            int *__restrict__ status, long cell, const UpdC &uc)
+__device__ __forceinline__ void update_item(const KP &P, const R *ff, double dt, double *W,
+                                            double *G, double *Ws, double *Gs,
+                                            double *Acc, const Shadow &s0, const Shadow &s1,
+                                            int *status, long cell, const UpdC &uc)
 {
     constexpr int NV = M + 2, NG = (M == 1) ? 1 : ((M == 2) ? 2 : 4);
     if constexpr (sizeof(R) == sizeof(float) && M >= 2) {
@@ -1370,7 +1370,7 @@ template <int M, typename T> __device__ __forceinline__ T speed_of(const T *w, T
  * (non-negative doubles order like their bit patterns).  A cell whose speed is not a
  * number does not count, here and below (fmax drops it; every warp has a lane at 0):
  * the status word reports it. */
-template <typename T> __device__ __forceinline__ void speed_max(T s, T ir, unsigned long long *__restrict__ smax)
+template <typename T> __device__ __forceinline__ void speed_max(T s, T ir, unsigned long long *smax)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1387,7 +1387,7 @@ template <typename T> __device__ __forceinline__ void speed_max(T s, T ir, unsig
 /* the same over a block of whole warps, which all call it: one atomic per
  * block and word, and none where the word is already as large (a stale read
  * only adds an atomic) */
-template <typename T> __device__ __forceinline__ void block_speed_max(T s, T ir, unsigned long long *__restrict__ smax)
+template <typename T> __device__ __forceinline__ void block_speed_max(T s, T ir, unsigned long long *smax)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

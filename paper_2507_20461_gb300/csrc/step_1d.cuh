@@ -60,7 +60,7 @@ inline bool short_1d(int n)
 /* one variable of one side of face f (value, physical derivative, and the
  * cell's own average): the left reconstruction of the stencil, mirrored for
  * the right side (derivatives change sign) */
-__device__ __forceinline__ void recon1d_side(const KP &P, const double *__restrict__ W, const double *__restrict__ G, int f,
+__device__ __forceinline__ void recon1d_side(const KP &P, const double *W, const double *G, int f,
                                              int side, int v, double &val, double &der, double &own)
 {
     double w[4], d[4];

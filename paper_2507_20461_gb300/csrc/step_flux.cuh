@@ -240,8 +240,8 @@ __device__ __forceinline__ bool face_point(const FluxParams &fp, R adm, R dt, R 
  * POINTS: the fluxes of every Gauss point into ff[q][v][g][face] (gks_flux)
  * instead of their sums. */
 template <typename R, int M, int D, bool NS, int SS, bool SPLIT = false, bool POINTS = false>
-__device__ __forceinline__ void step_face_item(const KP &P, const R *__restrict__ B, R dt, R idt, R *__restrict__ ff,
-                                               int *__restrict__ status, unsigned fl, typename FaceV<R>::V *stash, bool store = true)
+__device__ __forceinline__ void step_face_item(const KP &P, const R *B, R dt, R idt, R *ff,
+                                               int *status, unsigned fl, typename FaceV<R>::V *stash, bool store = true)
 {
     using FV = FaceV<R>;
     using V = typename FV::V;
@@ -469,10 +469,10 @@ __global__ void __launch_bounds__(kStepFluxBlock, (kStepFluxMinBlocks<R, M, NS>)
 
 /* the stage update from the face sums of step_face_item; wn receives the new averages */
 template <typename R, int M, int STAGE>
-__device__ __forceinline__ void step_update_item(const KP &P, const R *__restrict__ ff, double dt, double *__restrict__ W,
-                                                 double *__restrict__ G, double *__restrict__ Ws, double *__restrict__ Gs,
-                                                 double *__restrict__ Acc, const Shadow &s0, const Shadow &s1,
-                                                 int *__restrict__ status, long cell, const UpdC &uc, R *wn)
+__device__ __forceinline__ void step_update_item(const KP &P, const R *ff, double dt, double *W,
+                                                 double *G, double *Ws, double *Gs,
+                                                 double *Acc, const Shadow &s0, const Shadow &s1,
+                                                 int *status, long cell, const UpdC &uc, R *wn)
 {
     constexpr int NV = M + 2;
     unsigned q0, q1;

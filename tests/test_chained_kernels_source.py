@@ -61,6 +61,13 @@ def test_waits_first_and_orders_every_pointer(name):
     assert set(re.findall(r"__restrict__\s+(\w+)", sig)) <= CONSTANT, f
 
 
+def test_item_functions_do_not_bring_the_promise_back():
+    """the functions inlined into these kernels (csrc/*.cuh, k1d_nc.cu): no __restrict__ pointer parameter"""
+    for f in ("chain.cuh", "kernels.cuh", "step_flux.cuh", "step_1d.cuh", "k1d_nc.cu"):
+        for sig in re.findall(r"__device__ __forceinline__ [^{;]*{", _sources()[f]):
+            assert "__restrict__" not in sig, (f, sig[:80])
+
+
 def test_no_load_that_assumes_constant_memory():
     for f, s in _sources().items():
         assert "__ldg" not in s and "ld.global.nc" not in s, f
